@@ -168,7 +168,8 @@ struct ewv_model {
     int* d_rec = nullptr;
     int* d_nrec = nullptr;      // receivers per shot
     double* d_sigma = nullptr;
-    float* d_btab = nullptr;    // damping profile at half-cell distances (FP32 TMA passes)
+    float* d_btab = nullptr;    // damping profile at half-cell distances (FP32 models)
+    double* d_btab64 = nullptr; // ... (FP64 models)
     int nbtab = 0;
     double* d_kry = nullptr;
     long long* d_clk = nullptr;
@@ -431,6 +432,7 @@ ProblemDev make_problem(ewv_model* m, int shot, int tile_base) {
     P.inv_pml = d.pml_width > 0 ? 1.0 / d.pml_width : 0.0;
     P.fbeta0 = (float)P.beta0;
     P.btab = m->d_btab;
+    P.btab64 = m->d_btab64;
     P.nbtab = m->nbtab;
     P.finv_pml = (float)P.inv_pml;
     P.finv_dx = (float)P.inv_dx;
@@ -1126,10 +1128,9 @@ int run_krylov(Ctx& C, double t, double dt, int m, int nsteps, int* info) {
     ++*C.launches;
     bool expm_ok = true;
     const int window = C.E->models.empty() ? 0 : C.E->models[0]->kry_window;
-    // FP32: the matrix-vector product runs on the TMA stencil pass, which has no dot partner;
-    // a flat pass then forms <q_{j+1}, q_k0> with the same finalisation (FP64 keeps the fused
-    // dot of the plain stencil kernel)
-    const bool split_dot = C.E->precision == EWV_F32;
+    // The matrix-vector product has no dot partner; a flat pass then forms <q_{j+1}, q_k0>
+    // (the plain FP64 3D kernel keeps its fused dot, with the same finalisation)
+    const bool split_dot = C.E->precision == EWV_F32 || C.E->dims == 2;
     // dense output: before the step's own combine (which overwrites q_1 = U^{n-1}), the states
     // x(tau_q dt) = beta V exp(tau_q H_m) e_1 at the 4-point Gauss-Legendre nodes go to the
     // caller's buffer [q][shot]; a key of its own keeps such a call out of the step graphs
@@ -1598,8 +1599,7 @@ int run_leapfrog(Ctx& C, std::vector<ewv_model*>& models, double t, double dt, i
                                     C.s) != 0)
                 C.launch_failed = 1;
         } else {
-            launch_leapfrog(C.E->precision, C.E->R, C.E->ntiles, C.E->d_probs, C.E->d_tile_prob,
-                            cur, prev, variant, dt, C.s);
+            launch_leapfrog(C.E->R, C.E->ntiles, C.E->d_probs, C.E->d_tile_prob, cur, prev, variant, dt, C.s);
         }
         });
         C.record(prev);
@@ -1785,13 +1785,18 @@ int ewv_create_model(const ewv_model_desc* desc, ewv_model_t* out) {
     // beta at distance d = k/2 cells from the first ghost line (Sec. 2 profile), k = 0 .. 2 pml
     m->nbtab = 2 * d.pml_width + 1;
     {
-        std::vector<float> bt((size_t)m->nbtab, 0.f);
+        std::vector<double> bt((size_t)m->nbtab, 0.0);
         for (int k = 0; k < m->nbtab && d.pml_width > 0; ++k) {
             const double r = 1.0 - (0.5 * k) / d.pml_width;
-            bt[k] = (float)(d.beta0 * r * r);
+            bt[k] = d.beta0 * r * r;
         }
-        if (e == cudaSuccess) e = cudaMalloc(&m->d_btab, sizeof(float) * bt.size());
-        if (e == cudaSuccess) e = cudaMemcpy(m->d_btab, bt.data(), sizeof(float) * bt.size(), cudaMemcpyHostToDevice);
+        const std::vector<float> btf(bt.begin(), bt.end());
+        const bool f32 = d.precision == EWV_F32;
+        const size_t bytes = bt.size() * (f32 ? sizeof(float) : sizeof(double));
+        if (e == cudaSuccess) e = f32 ? cudaMalloc(&m->d_btab, bytes) : cudaMalloc(&m->d_btab64, bytes);
+        if (e == cudaSuccess)
+            e = f32 ? cudaMemcpy(m->d_btab, btf.data(), bytes, cudaMemcpyHostToDevice)
+                    : cudaMemcpy(m->d_btab64, bt.data(), bytes, cudaMemcpyHostToDevice);
     }
     if (e == cudaSuccess) e = cudaMalloc(&m->d_kry, sizeof(double) * (size_t)KRY_STRIDE * d.nshots);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_clk, sizeof(long long) * 4 * (size_t)d.nshots);
@@ -1815,6 +1820,7 @@ int ewv_destroy_model(ewv_model_t m) {
     cudaFree(m->d_nrec);
     cudaFree(m->d_sigma);
     cudaFree(m->d_btab);
+    cudaFree(m->d_btab64);
     cudaFree(m->d_kry);
     cudaFree(m->d_clk);
     cudaFree(m->d_tclk);
@@ -2103,12 +2109,25 @@ int ewv_apply_operator(ewv_model_t m, int transpose, const void* x, void* y) {
     if (!m->params || !m->velocity_set) return fail(m->err, EWV_ERR_NOT_BOUND, "velocity not set");
     if (m->d.dims == 3 && transpose)
         return fail(m->err, EWV_ERR_UNSUPPORTED, "the 3D operator has no transpose pass");
-    Engine* E = ensure_model_engine(m);
     ProblemDev P = make_problem(m, 0, 0);
     P.tmaps = nullptr;
     P.has_src = 0;
     P.state = const_cast<void*>(x);
     P.work = y;
+    StageArgs a = stage_defaults();
+    a.x = 0;
+    a.y_out = 1;
+    a.ch = 1.0;
+    a.ck = 1.0;
+    a.transpose = transpose ? 1 : 0;
+    ++m->launches;
+    if (m->d.dims == 2) {
+        // nothing to allocate, copy or wait for: the descriptor travels with the launch
+        if (launch_stage_one(m->d.precision, m->R, P, a, m->stream) != 0)
+            return fail(m->err, EWV_ERR_CUDA, "the operator pass could not be launched");
+        return check_launch(m->err);
+    }
+    Engine* E = ensure_model_engine(m);
     cudaFree(E->d_apply);
     E->d_apply = nullptr;
     CUDA_OR_FAIL(m->err, cudaMalloc(&E->d_apply, sizeof(ProblemDev) + sizeof(int) * P.ntiles));
@@ -2116,18 +2135,7 @@ int ewv_apply_operator(ewv_model_t m, int transpose, const void* x, void* y) {
     int* d_tp = (int*)((char*)E->d_apply + sizeof(ProblemDev));
     CUDA_OR_FAIL(m->err, cudaMemcpyAsync(E->d_apply, &P, sizeof(ProblemDev), cudaMemcpyHostToDevice, m->stream));
     CUDA_OR_FAIL(m->err, cudaMemcpyAsync(d_tp, tp.data(), sizeof(int) * P.ntiles, cudaMemcpyHostToDevice, m->stream));
-    StageArgs a = stage_defaults();
-    a.x = 0;
-    a.y_out = 1;
-    a.ch = 1.0;
-    a.ck = 1.0;
-    a.transpose = transpose ? 1 : 0;
-    if (m->d.dims == 3) {
-        launch_stage3d(m->d.precision, m->R, P.ntiles, E->d_apply, d_tp, a, m->stream);
-    } else {
-        launch_stage(m->d.precision, m->R, P.ntiles, E->d_apply, d_tp, a, m->stream);
-    }
-    ++m->launches;
+    launch_stage3d(m->d.precision, m->R, P.ntiles, E->d_apply, d_tp, a, m->stream);
     // keep the host copies alive until the copies complete
     CUDA_OR_FAIL(m->err, cudaStreamSynchronize(m->stream));
     return check_launch(m->err);
@@ -2427,9 +2435,7 @@ static int adjoint_krylov(ewv_model* m, Engine* E, double t, double dt, int mm, 
         views[2 * ns + sh] = G;
     }
     // FP32: the products of both Arnoldi processes take the persistent TMA passes (the forward
-    // one the autotuned variant, the transposed one 64 x 18 tiles), each followed by a flat
-    // pass forming <q_{j+1}, q_1> with the finalisation of the plain kernel's fused dot; the
-    // tensor maps describe the F and A views and are rebuilt when the buffers change.  The
+    // one the autotuned variant, the transposed one 64 x 18 tiles); the tensor maps describe the F and A views and are rebuilt when the buffers change.  The
     // gradient passes take the TMA gradient pass when the caller built maps of the G view
     // (the cotangent and the workspace from vector 0).
     bool tma = prec == EWV_F32 && E->tma_variant >= 0 && E->d_tbase && E->nprob == ns &&
@@ -2490,77 +2496,35 @@ static int adjoint_krylov(ewv_model* m, Engine* E, double t, double dt, int mm, 
             StageArgs a = stage_defaults();
             a.x = j - 1;
             a.y_out = j;
-            a.d = 0;
             a.src_slot = transpose ? -1 : j;
             a.x_scale_slot = KRY_S + j;
             a.ch = dt;
             a.ck = 1.0;
             a.transpose = transpose ? 1 : 0;
-            a.fin_mode = FIN_MATVEC;
-            a.fin_j = j;
-            a.m = mm;
-            a.tol = tol;
-            a.partials = E->d_partials;
-            a.counters = E->d_counters;
-            bool fused = true;
-            if (col) {
-                // the product without a dot (TMA pass in FP32), then the column kernel
-                StageArgs b = a;
-                b.d = -1;
-                b.fin_mode = FIN_NONE;
-                const int set = transpose ? trset : fset;
-                const int* tbs = tma ? E->d_tbase + (size_t)set * (E->nprob + 1) : nullptr;
-                int rc = 1;
-                if (tma)
-                    rc = transpose ? launch_transpose_tma(R, v, tbs, ns, E->ntiles_by[set], b, E->d_err, s)
-                                   : launch_stage_tma(E->tma_variant, R, v, tbs, ns, E->ntiles_by[set], b, E->d_err, s);
-                if (rc != 0) launch_stage(prec, R, tb, v, d_tp, b, s);
-                ++m->launches;
-                const int kmax = (j == mm) ? j - 1 : j;
-                if (mgs_column(E, prec, v, ns, j, 1, kmax, mm, tol, s)) {
-                    ++m->launches;
-                    continue;
-                }
-                // the column kernel could not be launched: the flat dot, then the flat passes
-                PointArgs pd{};
-                pd.mode = 5;
-                pd.j = j;
-                pd.k = 1;
-                pd.m = mm;
-                pd.tol = tol;
-                pd.partials = E->d_partials;
-                pd.counters = E->d_counters;
-                launch_point_flat(prec, E->nchunks, v, E->d_pbase, ns, pd, s);
-                ++m->launches;
-                fused = false;
-            } else if (tma) {
-                StageArgs b = a;
-                b.d = -1;
-                b.fin_mode = FIN_NONE;
-                const int set = transpose ? trset : fset;
-                const int* tbs = E->d_tbase + (size_t)set * (E->nprob + 1);
-                const int rc = transpose
-                                   ? launch_transpose_tma(R, v, tbs, ns, E->ntiles_by[set], b, E->d_err, s)
-                                   : launch_stage_tma(E->tma_variant, R, v, tbs, ns, E->ntiles_by[set], b, E->d_err, s);
-                if (rc == 0) {
-                    PointArgs pd{};
-                    pd.mode = 5;
-                    pd.j = j;
-                    pd.k = 1;
-                    pd.m = mm;
-                    pd.tol = tol;
-                    pd.partials = E->d_partials;
-                    pd.counters = E->d_counters;
-                    launch_point_flat(prec, E->nchunks, v, E->d_pbase, ns, pd, s);
-                    m->launches += 2;
-                    fused = false;
-                }
-            }
-            if (fused) {
-                launch_stage(prec, R, tb, v, d_tp, a, s);
-                ++m->launches;
-            }
+            // the product (TMA pass in FP32), then its Gram-Schmidt steps
+            const int set = transpose ? trset : fset;
+            const int* tbs = tma ? E->d_tbase + (size_t)set * (E->nprob + 1) : nullptr;
+            int rc = 1;
+            if (tma)
+                rc = transpose ? launch_transpose_tma(R, v, tbs, ns, E->ntiles_by[set], a, E->d_err, s)
+                               : launch_stage_tma(E->tma_variant, R, v, tbs, ns, E->ntiles_by[set], a, E->d_err, s);
+            if (rc != 0) launch_stage(prec, R, tb, v, d_tp, a, s);
+            ++m->launches;
             const int kmax = (j == mm) ? j - 1 : j;
+            if (col && mgs_column(E, prec, v, ns, j, 1, kmax, mm, tol, s)) {
+                ++m->launches;
+                continue;
+            }
+            PointArgs pd{};
+            pd.mode = 5;
+            pd.j = j;
+            pd.k = 1;
+            pd.m = mm;
+            pd.tol = tol;
+            pd.partials = E->d_partials;
+            pd.counters = E->d_counters;
+            launch_point_flat(prec, E->nchunks, v, E->d_pbase, ns, pd, s);
+            ++m->launches;
             for (int k = 1; k <= kmax; ++k) {
                 PointArgs pm{};
                 pm.mode = 1;
@@ -2700,20 +2664,21 @@ static int adjoint_krylov_exact(ewv_model* m, Engine* E, double t, double dt, in
             StageArgs a = stage_defaults();
             a.x = j - 1;
             a.y_out = j;
-            a.d = k0 - 1;
             a.src_slot = j;
             a.x_scale_slot = KRY_S + j;
             a.ch = dt;
             a.ck = 1.0;
-            a.fin_mode = FIN_MATVEC;
-            a.fin_j = j;
-            a.fin_k = k0;
-            a.m = mm;
-            a.tol = tol;
-            a.partials = E->d_partials;
-            a.counters = E->d_counters;
             launch_stage(prec, R, tb, vF, d_tp, a, s);
-            ++m->launches;
+            PointArgs pd{};
+            pd.mode = 5;
+            pd.j = j;
+            pd.k = k0;
+            pd.m = mm;
+            pd.tol = tol;
+            pd.partials = E->d_partials;
+            pd.counters = E->d_counters;
+            launch_point_flat(prec, E->nchunks, vF, E->d_pbase, ns, pd, s);
+            m->launches += 2;
             const int kmax = (j == mm) ? j - 1 : j;
             for (int k = k0; k <= kmax; ++k) {
                 PointArgs pm{};

@@ -70,7 +70,8 @@ struct ProblemDev {
     long long* clk;       // [4]: step within call, recording cursor, (unused), (unused)
     double* tclk;         // [2]: t_start, dt of the current call
     const void* tmaps;    // FP32: this problem's TMA tensor maps (kernels_tma.cu), else null
-    const float* btab;    // beta0 (1 - d/delta)^2 at distances d = k/2 cells, k < nbtab (FP32)
+    const float* btab;    // beta0 (1 - d/delta)^2 at distances d = k/2 cells, k < nbtab (FP32 models)
+    const double* btab64; // the same in FP64 (FP64 models)
     float fbeta0, finv_pml, finv_dx, finv_dx2;   // FP32 copies of the damping / grid constants
     double* kbar;         // exact Krylov adjoint: [KB_STRIDE] reverse-sweep scalars, else null
 };
@@ -128,6 +129,7 @@ struct StageArgs {
     void* grad;                      // gradient mode: grad += gscale q_v G(X), per-shot fields
     int gq;                          // vector index of q (its v field is read)
     double gscale;
+    int terms;                       // plain kernels: which coefficients are not 0 or 1 (set at launch)
     int store_bf16;                  // 1: round every stored Y / ACC value to bfloat16 (RN)
     // FP32 copies of cx .. cax, filled by the FP32 TMA launcher (the kernel reads them from
     // the parameter bank instead of holding converted values in registers)
@@ -162,11 +164,13 @@ struct PointArgs {
 // Host-side launchers (defined in kernels_stencil.cu / kernels_aux.cu).
 int upload_stencil_tables(int order, const double* fs_uyy, const double* fs_uy,
                           const double* fs_dwy);
-void launch_stage(int precision, int R, int nblocks, const ProblemDev* probs,
+void launch_stage(int precision, int R, int ntiles, const ProblemDev* probs,
                   const int* tile_prob, const StageArgs& a, cudaStream_t s);
-void launch_leapfrog(int precision, int R, int nblocks, const ProblemDev* probs,
-                     const int* tile_prob, int cur, int prev, int variant, double dt,
-                     cudaStream_t s);
+// y = H x or H^T x of one problem, whose descriptor travels with the launch (-1: another pass).
+int launch_stage_one(int precision, int R, const ProblemDev& P, const StageArgs& a, cudaStream_t s);
+// One FP64 leap-frog step (2D).
+void launch_leapfrog(int R, int ntiles, const ProblemDev* probs, const int* tile_prob, int cur, int prev,
+                     int variant, double dt, cudaStream_t s);
 // Pointwise parts of the leap-frog adjoint step (mode 0: q from lambda; mode 1: lambda update
 // from y = H^T q); a1_base: the second cotangent vector of every shot (lam of w^{n-1}).
 void launch_leapfrog_adjoint(int precision, int nblocks, const ProblemDev* probs, const int* tile_prob,

@@ -13,25 +13,32 @@
 // surface -- Appendix A's one-sided rows for u_yy (rows 0..3) and u_y (half rows 0..2) and
 // Fornberg rows (Sec. 2.2) for d_y w_y (rows 0..3).  y is the paper's upward axis, the row
 // index j grows downward: d_y u at half row j+1/2 = sum_k s_k (u_{j-k} - u_{j+1+k}) / dx.
-// The damping beta = beta0 (1 - d/delta)^2 (Sec. 2) is evaluated in registers from the
-// node / half-node distance to the first ghost line.
+// The damping beta comes from the model's table at half-cell distances (FP32 and FP64).
 //
-// Layout: per block a BX x BY tile of outputs.  u is staged in shared memory with an
-// R-wide halo on all sides, w_x with an x halo, w_y with a y halo (zero outside the grid =
-// the zero extension); v, c^2 and the integrator's pointwise operands are read straight
-// from global memory (coalesced) and prefetched before the staging barrier.
+// Layout: one thread per grid point, blocks of 32 x 4 points cut out of the BX x BY tiles of
+// the work list; every operand is read straight from global memory (a warp reads 32 adjacent
+// points; the taps of neighbouring points meet in L1).  These kernels serve FP64 (everything
+// but 3D) and the FP32 passes that the TMA pipelines do not take (H x on a caller's vectors,
+// the bfloat16 storage experiment, the allocation-free Faber step, the exact Krylov adjoint).
+// In FP64 they are bound by arithmetic: GB300 issues one FP64 warp instruction per SM in
+// about 16 cycles, so a pass costs its FP64 instruction count and nothing else once every SM
+// has work.  Hence: small blocks (a 101 x 101 grid covers 104 SMs; 64 x 16 tiles with four
+// points a thread covered 14), damping looked up instead of evaluated, terms whose
+// coefficient is zero left out (the w rows of H vanish wherever no damping acts, the
+// epilogue's unused operands), and no shared memory, whose bandwidth is not the limit.
+// Measured on 601 x 301 in FP64: a Faber degree 37 us (102 us before), 65 FP64 instructions a
+// point (about 150), FP64 pipe 63 % busy; HORK 12 on 101 x 101, FP64: 8.5 us a pass (45 us).
+// FP32 on 601 x 301: H x 6.2 us and H^T x 10.2 us a call (29 us).
 //
 // Epilogue (StageArgs), per field f at every output point:
 //   K   = cx X + ch xs (H X + sigma e_src)          (xs: per-problem scale, Krylov)
 //   Y   = cu U + ck K                               -> y_out
 //   ACC = ca A + cau U + cak K + cay Y + cax X      -> acc_out
-// and optionally a partial dot product <Y, D> (Krylov), finalised by the last block.
 #include <cuda_bf16.h>
 
 #include <type_traits>
 
 #include "ewave_internal.cuh"
-#include "krylov_finalize.cuh"
 
 namespace ewv {
 
@@ -101,524 +108,524 @@ __device__ __forceinline__ T* vec_ptr(const ProblemDev* P, int k) {
 }
 
 // --------------------------------------------------------------------------------------
-// Stage kernel
+// Operands of one grid point
 // --------------------------------------------------------------------------------------
-template <typename T, int R, bool TRANS>
-__global__ void __launch_bounds__(NTHREADS)
-stage_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ tile_prob,
-             StageArgs a) {
-    constexpr int SW = BX + 2 * R;    // staged width with x halo
-    constexpr int SH = BY + 2 * R;    // staged height with y halo
-    __shared__ T su[SH][SW];
-    __shared__ T swx[BY][SW];
-    __shared__ T swy[SH][BX];
-    __shared__ double red[NTHREADS / 32];
-    __shared__ int s_last;
+constexpr int DBX = 32, DBY = 4;                              // points (threads) per block
+constexpr int DSUB_X = BX / DBX, DSUB = DSUB_X * (BY / DBY);  // blocks per tile of the work list
+static_assert(BX % DBX == 0 && BY % DBY == 0, "blocks must cut the tiles evenly");
 
-    const int pid = tile_prob[blockIdx.x];
-    const ProblemDev* P = probs + pid;
-    if (a.fin_mode != FIN_NONE && P->kry[KRY_ACTIVE] == 0.0) return;   // Arnoldi stopped
+// beta at k half cells from the first ghost line: the model's table, or (the allocation-free
+// step has none) the profile itself.
+template <typename T>
+__device__ __forceinline__ T beta_at(const ProblemDev& P, int k) {
+    const T* tab;
+    if constexpr (std::is_same<T, float>::value) tab = P.btab;
+    else tab = P.btab64;
+    if (tab) return (unsigned)k < (unsigned)P.nbtab ? __ldg(tab + k) : T(0);
+    if (P.pml <= 0 || k > 2 * P.pml) return T(0);
+    const T r = T(1) - T(0.5) * T(k) * (T)P.inv_pml;
+    return (T)P.beta0 * r * r;
+}
+// Distances (in half cells) of the nodes and half points; the top has no layer under a free
+// surface.
+__device__ __forceinline__ int dist_xn(const ProblemDev& P, int i) { return 2 * min(i + 1, P.nx - i); }
+__device__ __forceinline__ int dist_xh(const ProblemDev& P, int i) { return min(2 * i + 3, 2 * (P.nx - i) - 1); }
+__device__ __forceinline__ int dist_yn(const ProblemDev& P, int j) {
+    return P.fs ? 2 * (P.ny - j) : 2 * min(j + 1, P.ny - j);
+}
+__device__ __forceinline__ int dist_yh(const ProblemDev& P, int j) {
+    return P.fs ? 2 * (P.ny - j) - 1 : min(2 * j + 3, 2 * (P.ny - j) - 1);
+}
+template <typename T>
+struct Damping {
+    T xn, yn, xh, yh;     // at the node, at (i + 1/2, j) and at (i, j + 1/2)
+    bool any;             // false: the w rows of H are zero and the v row has no damping term
+    __device__ __forceinline__ Damping(const ProblemDev& P, int i, int j)
+        : xn(beta_at<T>(P, dist_xn(P, i))), yn(beta_at<T>(P, dist_yn(P, j))),
+          xh(beta_at<T>(P, dist_xh(P, i))), yh(beta_at<T>(P, dist_yh(P, j))),
+          // (by distance: a comparison of FP64 values would occupy the FP64 pipe)
+          any(min(min(dist_xn(P, i), dist_xh(P, i)), min(dist_yn(P, j), dist_yh(P, j))) < 2 * P.pml) {}
+};
 
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int nx = P->nx, ny = P->ny, pitch = P->pitch, pml = P->pml;
-    const bool fs = P->fs != 0;
-    const int lt = blockIdx.x - P->tile_base;
-    const int x0 = (lt % P->tiles_x) * BX;
-    const int y0 = (lt / P->tiles_x) * BY;
-    const long long fstr = P->field_stride;
-    const T beta0 = (T)P->beta0, inv_pml = (T)P->inv_pml;
-    const T idx1 = (T)P->inv_dx, idx2 = (T)P->inv_dx2;
+// The grid point of this thread in sub-block `sub` of tile `lt` of its problem.
+struct PointAt {
+    int i, j;
+    __device__ __forceinline__ PointAt(const ProblemDev& P, int lt, int sub)
+        : i((lt % P.tiles_x) * BX + (sub % DSUB_X) * DBX + (int)threadIdx.x),
+          j((lt / P.tiles_x) * BY + (sub / DSUB_X) * DBY + (int)threadIdx.y) {}
+};
 
-    const T* X = vec_ptr<T>(P, a.x);
-    const T* C2 = (const T*)P->c2;
-
-    // ---- prefetch pointwise operands (registers) ---------------------------------------
-    T pv[VY][VX], pc2[VY][VX];
-    T pU[4][VY][VX], pA[4][VY][VX];
-    const T* U = a.u >= 0 ? vec_ptr<T>(P, a.u) : nullptr;
-    const T* A = a.a >= 0 ? vec_ptr<T>(P, a.a) : nullptr;
+// Taps at (i, j) along the row and down the column, zero off the grid: row[R + d] = x(i + d);
+// col[q] = x(base + q), base = j - R, or 0 for the free-surface rows 0..3 (BAND: the rows take
+// their own code, so that the others do not issue its predicated-off FP64 instructions).  N taps
+// each way; nx, ny: extent of the field along its row and column.  u and w are loaded and summed one
+// after the other (both at once would not fit the registers that six blocks an SM leave).
+template <typename T, int R, int N, bool BAND>
+struct Taps {
+    T row[N], col[N];
+    __device__ __forceinline__ Taps(const T* rowf, const T* colf, int i, int j, long long pitch, int nx, int ny) {
+        const int base = BAND ? 0 : j - R;
+        const T* r = rowf + j * pitch + i - R;
+        const T* c = colf + base * pitch + i;
+        if (i >= R && i - R + N <= nx && base >= 0 && base + N <= ny) {
 #pragma unroll
-    for (int b = 0; b < VY; ++b) {
+            for (int q = 0; q < N; ++q) {
+                row[q] = r[q];
+                col[q] = c[q * pitch];
+            }
+        } else {
 #pragma unroll
-        for (int c = 0; c < VX; ++c) {
-            const int i = x0 + tx + c * TPX, j = y0 + ty + b * TPY;
-            const bool in = (i < nx) && (j < ny);
-            const long long o = (long long)j * pitch + i;
-            pv[b][c] = in ? X[fstr + o] : T(0);
-            pc2[b][c] = in ? C2[o] : T(0);
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                pU[f][b][c] = (in && U) ? U[f * fstr + o] : T(0);
-                pA[f][b][c] = (in && A) ? A[f * fstr + o] : T(0);
+            for (int q = 0; q < N; ++q) {
+                row[q] = (i + q >= R && i + q < nx + R) ? r[q] : T(0);
+                col[q] = (base + q >= 0 && base + q < ny) ? c[q * pitch] : T(0);
             }
         }
     }
+};
 
-    // ---- stage halo tiles ----------------------------------------------------------------
-    // Row-wise: thread (tx, ty) fills columns tx, tx + TPX, ... of rows ty, ty + TPY, ...; the
-    // row's bounds test and (in the transpose) its damping factor are taken once per row.
-    if constexpr (!TRANS) {
-        const T* Xu = X;
-        const T* Xwx = X + 2 * fstr;
-        const T* Xwy = X + 3 * fstr;
-        for (int r = ty; r < SH; r += TPY) {
-            const int gy = y0 - R + r;
-            const bool rok = gy >= 0 && gy < ny;
-            const T* row = Xu + (long long)(rok ? gy : 0) * pitch;
-            for (int c = tx; c < SW; c += TPX) {
-                const int gx = x0 - R + c;
-                su[r][c] = (rok && gx >= 0 && gx < nx) ? row[gx] : T(0);
-            }
+// Sums of u at (i, j): the Laplacian (times dx^2) and the half-point differences d_x u at
+// (i + 1/2, j), d_y u at (i, j + 1/2) (times dx).
+template <typename T, int R, bool BAND>
+struct USums {
+    Taps<T, R, 2 * R + 1, BAND> t;
+    int j;
+    __device__ __forceinline__ USums(const ProblemDev& P, const T* X, int i, int jj)
+        : t(X, X, i, jj, P.pitch, P.nx, P.ny), j(jj) {}
+    __device__ __forceinline__ T u() const { return t.row[R]; }
+    __device__ __forceinline__ T laplacian() const {
+        T uxx = CENT<T, R>(0) * t.row[R], uyy;
+#pragma unroll
+        for (int k = 1; k <= R; ++k) uxx += CENT<T, R>(k) * (t.row[R + k] + t.row[R - k]);
+        if constexpr (BAND) {
+            uyy = T(0);
+#pragma unroll
+            for (int q = 0; q <= 2 * R; ++q) uyy += fs_coef<T>(FS_UYY_OFF + j * 9 + q) * t.col[q];
+        } else {
+            uyy = CENT<T, R>(0) * t.row[R];
+#pragma unroll
+            for (int k = 1; k <= R; ++k) uyy += CENT<T, R>(k) * (t.col[R + k] + t.col[R - k]);
         }
-        for (int r = ty; r < BY; r += TPY) {
-            const int gy = y0 + r;
-            const bool rok = gy < ny;
-            const T* row = Xwx + (long long)(rok ? gy : 0) * pitch;
-            for (int c = tx; c < SW; c += TPX) {
-                const int gx = x0 - R + c;
-                swx[r][c] = (rok && gx >= 0 && gx < nx - 1) ? row[gx] : T(0);
-            }
+        return uxx + uyy;
+    }
+    __device__ __forceinline__ T du_x() const {
+        T d = T(0);
+#pragma unroll
+        for (int k = 0; k < R; ++k) d += STAG<T, R>(k) * (t.row[R + 1 + k] - t.row[R - k]);
+        return d;
+    }
+    __device__ __forceinline__ T du_y() const {
+        T d = T(0);
+        if constexpr (!BAND) {
+#pragma unroll
+            for (int k = 0; k < R; ++k) d += STAG<T, R>(k) * (t.col[R - k] - t.col[R + 1 + k]);
+        } else if (j < 3) {
+#pragma unroll
+            for (int q = 0; q < 2 * R; ++q) d += fs_coef<T>(FS_UY_OFF + j * 8 + q) * t.col[q];
+        } else {     // row 3: the interior stencil, counted from row 0
+#pragma unroll
+            for (int k = 0; k < R; ++k) d += STAG<T, R>(k) * (t.col[R - 1 - k] - t.col[R + k]);
         }
-        for (int r = ty; r < SH; r += TPY) {
-            const int gy = y0 - R + r;
-            const bool rok = gy >= 0 && gy < ny - 1;
-            const T* row = Xwy + (long long)(rok ? gy : 0) * pitch;
-            for (int c = tx; c < BX; c += TPX) {
-                const int gx = x0 + c;
-                swy[r][c] = (rok && gx < nx) ? row[gx] : T(0);
-            }
-        }
+        return d;
+    }
+};
+
+// (d_x w_x + d_y w_y) dx at the node: w_x[i+k] - w_x[i-1-k] and (upward y) w_y[j-1-k] - w_y[j+k];
+// w_x has nx - 1 columns, w_y ny - 1 rows.
+template <typename T, int R, bool BAND>
+__device__ __forceinline__ T divergence(const ProblemDev& P, const T* X, int i, int j) {
+    const Taps<T, R, 2 * R, BAND> t(X + 2 * P.field_stride, X + 3 * P.field_stride, i, j, P.pitch, P.nx - 1, P.ny - 1);
+    T dwx = T(0), dwy = T(0);
+#pragma unroll
+    for (int k = 0; k < R; ++k) dwx += STAG<T, R>(k) * (t.row[R + k] - t.row[R - 1 - k]);
+    if constexpr (BAND) {
+#pragma unroll
+        for (int q = 0; q < 2 * R; ++q) dwy += fs_coef<T>(FS_DWY_OFF + j * 8 + q) * t.col[q];
     } else {
-        // Transpose: stage z_v = c^2 y_v (2D halo), z_x = g_x y_wx (x halo) and
-        // z_y = g_y y_wy (y halo), g_x = by(j) - bx(i+1/2), g_y = bx(i) - by(j+1/2).
-        const T* Xv = X + fstr;
-        const T* Xwx = X + 2 * fstr;
-        const T* Xwy = X + 3 * fstr;
-        for (int r = ty; r < SH; r += TPY) {
-            const int gy = y0 - R + r;
-            const bool rok = gy >= 0 && gy < ny;
-            const long long ro = (long long)(rok ? gy : 0) * pitch;
-            for (int c = tx; c < SW; c += TPX) {
-                const int gx = x0 - R + c;
-                su[r][c] = (rok && gx >= 0 && gx < nx) ? C2[ro + gx] * Xv[ro + gx] : T(0);
-            }
-        }
-        for (int r = ty; r < BY; r += TPY) {
-            const int gy = y0 + r;
-            const bool rok = gy < ny;
-            const T* row = Xwx + (long long)(rok ? gy : 0) * pitch;
-            const T byn = rok ? damp<T>(beta0, inv_pml, fs ? T(ny - gy) : T(min(gy + 1, ny - gy)), pml) : T(0);
-            for (int c = tx; c < SW; c += TPX) {
-                const int gx = x0 - R + c;
-                T val = T(0);
-                if (rok && gx >= 0 && gx < nx - 1) {
-                    const T dxh = min(T(gx) + T(1.5), T(nx - gx) - T(0.5));
-                    val = (byn - damp<T>(beta0, inv_pml, dxh, pml)) * row[gx];
-                }
-                swx[r][c] = val;
-            }
-        }
-        for (int r = ty; r < SH; r += TPY) {
-            const int gy = y0 - R + r;
-            const bool rok = gy >= 0 && gy < ny - 1;
-            const T* row = Xwy + (long long)(rok ? gy : 0) * pitch;
-            const T byh = rok ? damp<T>(beta0, inv_pml,
-                                        fs ? (T(ny - gy) - T(0.5)) : min(T(gy) + T(1.5), T(ny - gy) - T(0.5)), pml)
-                              : T(0);
-            for (int c = tx; c < BX; c += TPX) {
-                const int gx = x0 + c;
-                T val = T(0);
-                if (rok && gx < nx) val = (damp<T>(beta0, inv_pml, T(min(gx + 1, nx - gx)), pml) - byh) * row[gx];
-                swy[r][c] = val;
-            }
-        }
+#pragma unroll
+        for (int k = 0; k < R; ++k) dwy += STAG<T, R>(k) * (t.col[R - 1 - k] - t.col[R + k]);
     }
-    __syncthreads();
+    return dwx + dwy;
+}
 
-    const T cx = (T)a.cx, ch = (T)a.ch, cu = (T)a.cu, ck = (T)a.ck, ca = (T)a.ca;
-    const T cau = (T)a.cau, cak = (T)a.cak, cay = (T)a.cay, cax = (T)a.cax;
-    const T xs = a.x_scale_slot >= 0 ? (T)P->kry[a.x_scale_slot] : T(1);
-    const T sig = (a.src_slot >= 0 && P->has_src) ? (T)P->sigma[a.src_slot] : T(0);
-    T* Y = a.y_out >= 0 ? vec_ptr<T>(P, a.y_out) : nullptr;
-    T* ACC = a.acc_out >= 0 ? vec_ptr<T>(P, a.acc_out) : nullptr;
-    const T* D = a.d >= 0 ? vec_ptr<T>(P, a.d) : nullptr;
-    float dotf = 0.f;
-    double dotd = 0.0;
+// --------------------------------------------------------------------------------------
+// Epilogue of one point (StageArgs): terms whose coefficient is zero or one, or whose operand
+// is absent, cost nothing.  The host sets the bits (stage_terms); the bits of the FP64 integrators
+// are compile-time constants (TERMS >= 0), because a term that is skipped by predication still
+// occupies the FP64 pipe.  hw: the w components of H X are not zero.
+// --------------------------------------------------------------------------------------
+enum { TERM_CX = 1, TERM_CK = 2, TERM_CU = 4, TERM_CA = 8, TERM_CAU = 16, TERM_CAK = 32, TERM_CAY = 64,
+       TERM_CAX = 128, TERM_XS = 256, TERM_A = 512 };
 
+static int stage_terms(const StageArgs& a) {
+    int t = 0;
+    if (a.cx != 0.0) t |= TERM_CX;
+    if (a.ck != 1.0) t |= TERM_CK;                         // a factor other than one
+    if (a.u >= 0 && a.cu != 0.0) t |= TERM_CU;
+    if (a.a >= 0) t |= TERM_A;
+    if (a.a >= 0 && a.ca != 1.0) t |= TERM_CA;             // ... also zero: A is read, as before
+    if (a.u >= 0 && a.cau != 0.0) t |= TERM_CAU;
+    if (a.cak != 0.0) t |= TERM_CAK;
+    if (a.cay != 0.0) t |= TERM_CAY;
+    if (a.cax != 0.0) t |= TERM_CAX;
+    if (a.x_scale_slot >= 0) t |= TERM_XS;
+    return t;
+}
+
+template <typename T, int TERMS>
+__device__ __forceinline__ void epilogue(const ProblemDev& P, const StageArgs& a, long long o, const T (&xf)[4],
+                                         const T (&hf)[4], bool hw, bool padx, bool pady) {
+    const int t = TERMS >= 0 ? TERMS : a.terms;
+    const T* U = (t & (TERM_CU | TERM_CAU)) ? vec_ptr<T>(&P, a.u) + o : nullptr;
+    const T* A = (t & TERM_A) ? vec_ptr<T>(&P, a.a) + o : nullptr;
+    T* Y = a.y_out >= 0 ? vec_ptr<T>(&P, a.y_out) + o : nullptr;
+    T* ACC = a.acc_out >= 0 ? vec_ptr<T>(&P, a.acc_out) + o : nullptr;
+    T uv[4], av[4];
 #pragma unroll
-    for (int b = 0; b < VY; ++b) {
-#pragma unroll
-        for (int c = 0; c < VX; ++c) {
-            const int lx = tx + c * TPX, ly = ty + b * TPY;
-            const int i = x0 + lx, j = y0 + ly;
-            if (i >= nx || j >= ny) continue;
-            const long long o = (long long)j * pitch + i;
-            // damping at this node and its two half points
-            const T bxn = damp<T>(beta0, inv_pml, T(min(i + 1, nx - i)), pml);
-            const T byn = damp<T>(beta0, inv_pml, fs ? T(ny - j) : T(min(j + 1, ny - j)), pml);
-            const T bxh = damp<T>(beta0, inv_pml, min(T(i) + T(1.5), T(nx - i) - T(0.5)), pml);
-            const T byh = damp<T>(beta0, inv_pml,
-                                  fs ? (T(ny - j) - T(0.5)) : min(T(j) + T(1.5), T(ny - j) - T(0.5)),
-                                  pml);
-            const T c2 = pc2[b][c];
-            T xu, xv, xwx, xwy, hu, hv, hwx, hwy;
-            if constexpr (!TRANS) {
-                xu = su[ly + R][lx + R];
-                xv = pv[b][c];
-                xwx = swx[ly][lx + R];
-                xwy = swy[ly + R][lx];
-                // u_xx
-                T uxx = CENT<T, R>(0) * xu;
-#pragma unroll
-                for (int k = 1; k <= R; ++k)
-                    uxx += CENT<T, R>(k) * (su[ly + R][lx + R + k] + su[ly + R][lx + R - k]);
-                // u_yy
-                T uyy;
-                if (fs && j < 4) {
-                    uyy = T(0);
-#pragma unroll
-                    for (int q = 0; q < 9; ++q)
-                        uyy += fs_coef<T>(FS_UYY_OFF + j * 9 + q) * su[q - y0 + R][lx + R];
-                } else {
-                    uyy = CENT<T, R>(0) * xu;
-#pragma unroll
-                    for (int k = 1; k <= R; ++k)
-                        uyy += CENT<T, R>(k) * (su[ly + R + k][lx + R] + su[ly + R - k][lx + R]);
-                }
-                // d_x w_x at the node: w_x[i+k] - w_x[i-1-k]
-                T dwx = T(0);
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    dwx += STAG<T, R>(k) * (swx[ly][lx + R + k] - swx[ly][lx + R - 1 - k]);
-                // d_y w_y at the node (upward y): w_y[j-1-k] - w_y[j+k]
-                T dwy = T(0);
-                if (fs && j < 4) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        dwy += fs_coef<T>(FS_DWY_OFF + j * 8 + q) * swy[q - y0 + R][lx];
-                } else {
-#pragma unroll
-                    for (int k = 0; k < R; ++k)
-                        dwy += STAG<T, R>(k) * (swy[ly + R - 1 - k][lx] - swy[ly + R + k][lx]);
-                }
-                // d_x u at (i+1/2, j)
-                T dux = T(0);
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    dux += STAG<T, R>(k) * (su[ly + R][lx + R + 1 + k] - su[ly + R][lx + R - k]);
-                // d_y u at (i, j+1/2)
-                T duy = T(0);
-                if (fs && j < 3) {
-#pragma unroll
-                    for (int q = 0; q < 8; ++q)
-                        duy += fs_coef<T>(FS_UY_OFF + j * 8 + q) * su[q - y0 + R][lx + R];
-                } else {
-#pragma unroll
-                    for (int k = 0; k < R; ++k)
-                        duy += STAG<T, R>(k) * (su[ly + R - k][lx + R] - su[ly + R + 1 + k][lx + R]);
-                }
-                if (a.grad) {
-                    // FWI gradient w.r.t. m = c^2: d(H X)_v / dm = L X_u + D X_w
-                    T* G = (T*)a.grad + (long long)P->shot * fstr;
-                    const T* Q = vec_ptr<T>(P, a.gq);
-                    const T gval = (uxx + uyy) * idx2 + (dwx + dwy) * idx1;
-                    G[o] += (T)a.gscale * xs * Q[fstr + o] * gval;   // xs: per-problem scale
-                    continue;
-                }
-                hu = xv;
-                hv = -bxn * byn * xu + c2 * ((uxx + uyy) * idx2 + (dwx + dwy) * idx1)
-                     - (bxn + byn) * xv;
-                hwx = (i < nx - 1) ? (byn - bxh) * dux * idx1 - bxh * xwx : T(0);
-                hwy = (j < ny - 1) ? (bxn - byh) * duy * idx1 - byh * xwy : T(0);
-                if (i == P->src_i && j == P->src_j) hv += sig;
-            } else {
-                // H^T y.  Pointwise inputs: y_u (not staged), y_v = pv, y_wx, y_wy from the
-                // unscaled vector; staged: zv = c^2 y_v, zx = g_x y_wx, zy = g_y y_wy.
-                const T* Xg = X;
-                xu = Xg[o];
-                xv = pv[b][c];
-                xwx = (i < nx - 1) ? Xg[2 * fstr + o] : T(0);
-                xwy = (j < ny - 1) ? Xg[3 * fstr + o] : T(0);
-                // (Lxx^T zv)(i) = Lxx zv (symmetric)
-                T lxx = CENT<T, R>(0) * su[ly + R][lx + R];
-#pragma unroll
-                for (int k = 1; k <= R; ++k)
-                    lxx += CENT<T, R>(k) * (su[ly + R][lx + R + k] + su[ly + R][lx + R - k]);
-                // (Lyy^T zv)(j): interior rows r >= rfs contribute CENT(|r-j|), free-surface
-                // rows r < 4 contribute FS_UYY[r][j] for j <= 8.
-                T lyy = T(0);
-                const int rfs = fs ? 4 : 0;
-#pragma unroll
-                for (int k = -R; k <= R; ++k) {
-                    const int r = j + k;
-                    if (r >= rfs && r < ny) lyy += CENT<T, R>(k < 0 ? -k : k) * su[ly + R + k][lx + R];
-                }
-                if (fs && j <= 8) {
-#pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        if (r < ny) lyy += fs_coef<T>(FS_UYY_OFF + r * 9 + j) * su[r - y0 + R][lx + R];
-                }
-                // (Dxh^T zx)(i) = sum_k s_k (zx[i-1-k] - zx[i+k])
-                T gxt = T(0);
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    gxt += STAG<T, R>(k) * (swx[ly][lx + R - 1 - k] - swx[ly][lx + R + k]);
-                // (Dyh^T zy)(j): interior half rows h >= hfs: d_y u at h uses
-                // s_k (u[h-k] - u[h+1+k]); free-surface half rows h < 3 use FS_UY[h][j].
-                T gyt = T(0);
-                const int hfs = fs ? 3 : 0;
-#pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    const int h1 = j + k;        // u[j] = u[h1 - k] with + sign
-                    const int h2 = j - 1 - k;    // u[j] = u[h2 + 1 + k] with - sign
-                    if (h1 >= hfs && h1 < ny - 1) gyt += STAG<T, R>(k) * swy[ly + R + k][lx];
-                    if (h2 >= hfs && h2 >= 0) gyt -= STAG<T, R>(k) * swy[ly + R - 1 - k][lx];
-                }
-                if (fs && j <= 7) {
-#pragma unroll
-                    for (int h = 0; h < 3; ++h)
-                        if (h < ny - 1) gyt += fs_coef<T>(FS_UY_OFF + h * 8 + j) * swy[h - y0 + R][lx];
-                }
-                // (Dxn^T zv)(i+1/2) = sum_k s_k (zv[i-k] - zv[i+1+k])
-                T dxt = T(0);
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    dxt += STAG<T, R>(k) * (su[ly + R][lx + R - k] - su[ly + R][lx + R + 1 + k]);
-                // (Dyn^T zv)(j+1/2): interior rows r >= rfs: d_y w_y at r uses
-                // s_k (w[r-1-k] - w[r+k]); free-surface rows r < 4 use FS_DWY[r][j].
-                T dyt = T(0);
-#pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    const int r1 = j + 1 + k;    // w[j] = w[r1 - 1 - k], + sign
-                    const int r2 = j - k;        // w[j] = w[r2 + k], - sign
-                    if (r1 >= rfs && r1 < ny) dyt += STAG<T, R>(k) * su[ly + R + 1 + k][lx + R];
-                    if (r2 >= rfs && r2 >= 0) dyt -= STAG<T, R>(k) * su[ly + R - k][lx + R];
-                }
-                if (fs && j <= 7) {
-#pragma unroll
-                    for (int r = 0; r < 4; ++r)
-                        if (r < ny) dyt += fs_coef<T>(FS_DWY_OFF + r * 8 + j) * su[r - y0 + R][lx + R];
-                }
-                hu = -bxn * byn * xv + (lxx + lyy) * idx2 + (gxt + gyt) * idx1;
-                hv = xu - (bxn + byn) * xv;
-                hwx = (i < nx - 1) ? dxt * idx1 - bxh * xwx : T(0);
-                hwy = (j < ny - 1) ? dyt * idx1 - byh * xwy : T(0);
-            }
-            // ---- epilogue ------------------------------------------------------------
-            const T xf[4] = {xu, xv, xwx, xwy};
-            const T hf[4] = {hu, hv, hwx, hwy};
-#pragma unroll
-            for (int f = 0; f < 4; ++f) {
-                const bool pad = (f == 2 && i >= nx - 1) || (f == 3 && j >= ny - 1);
-                const T kf = cx * xs * xf[f] + ch * xs * hf[f];
-                T yf = pad ? T(0) : (cu * pU[f][b][c] + ck * kf);
-                if (a.store_bf16) yf = bf16_round(yf);     // storage-precision experiment
-                if (Y) Y[f * fstr + o] = yf;
-                if (ACC) {
-                    T af = ca * pA[f][b][c] + cau * pU[f][b][c] + cak * kf + cay * yf
-                           + cax * xs * xf[f];
-                    if (a.store_bf16) af = bf16_round(af);
-                    ACC[f * fstr + o] = pad ? T(0) : af;
-                }
-                if (D && !pad) {
-                    const T dv = D[f * fstr + o];
-                    if constexpr (std::is_same<T, float>::value) dotf = fmaf(yf, dv, dotf);
-                    else dotd = fma(yf, dv, dotd);
-                }
-            }
-        }
+    for (int f = 0; f < 4; ++f) {
+        uv[f] = U ? U[f * P.field_stride] : T(0);
+        av[f] = A ? A[f * P.field_stride] : T(0);
     }
-    if (a.fin_mode != FIN_NONE) {
-        const double mine = (double)dotf + dotd;
-        const double bsum = block_sum_fixed(mine, red);
-        partial_and_finalize(P, pid, a, bsum, red, &s_last);
+    T cx = (T)a.cx, ch = (T)a.ch, cax = (T)a.cax;
+    if (t & TERM_XS) {
+        const T xs = (T)P.kry[a.x_scale_slot];
+        cx *= xs;
+        ch *= xs;
+        cax *= xs;
+    }
+#pragma unroll
+    for (int f = 0; f < 4; ++f) {
+        const bool pad = (f == 2 && padx) || (f == 3 && pady);
+        T kf;
+        if (f < 2 || hw) {
+            kf = ch * hf[f];
+            if (t & TERM_CX) kf += cx * xf[f];
+        } else {
+            kf = (t & TERM_CX) ? cx * xf[f] : T(0);
+        }
+        T yf = (t & TERM_CK) ? (T)a.ck * kf : kf;
+        if (t & TERM_CU) yf += (T)a.cu * uv[f];
+        if (pad) yf = T(0);
+        if (a.store_bf16) yf = bf16_round(yf);     // storage-precision experiment
+        if (Y) Y[f * P.field_stride] = yf;
+        if (ACC) {
+            T af = (t & TERM_CA) ? (T)a.ca * av[f] : av[f];
+            if (t & TERM_CAY) af += (T)a.cay * yf;
+            if (t & TERM_CAU) af += (T)a.cau * uv[f];
+            if (t & TERM_CAK) af += (T)a.cak * kf;
+            if (t & TERM_CAX) af += cax * xf[f];
+            if (a.store_bf16) af = bf16_round(af);
+            ACC[f * P.field_stride] = pad ? T(0) : af;
+        }
     }
 }
 
 // --------------------------------------------------------------------------------------
-// Leap-frog kernel (Sec. 3.1).  Vectors `cur` (u^n, w^n) and `prev` (u^{n-1}, w^{n-1}) use
+// Stage kernels: one point of the forward pass, the gradient pass, the transposed pass
+// --------------------------------------------------------------------------------------
+enum { PASS_FORWARD = 0, PASS_GRADIENT = 1, PASS_TRANSPOSE = 2 };
+
+template <typename T, int R, bool BAND, int TERMS>
+__device__ __forceinline__ void forward_point(const ProblemDev& P, const StageArgs& a, int i, int j) {
+    const int nx = P.nx, ny = P.ny;
+    const long long o = (long long)j * P.pitch + i;
+    const T* X = vec_ptr<T>(&P, a.x);
+    const T idx1 = (T)P.inv_dx, idx2 = (T)P.inv_dx2;
+    const Damping<T> b(P, i, j);
+    const bool padx = i >= nx - 1, pady = j >= ny - 1;
+    const T xv = X[P.field_stride + o], c2 = static_cast<const T*>(P.c2)[o];
+    const T xwx = padx ? T(0) : X[2 * P.field_stride + o], xwy = pady ? T(0) : X[3 * P.field_stride + o];
+    T xu, lap, damping = T(0), hwx = T(0), hwy = T(0);
+    {
+        const USums<T, R, BAND> s(P, X, i, j);
+        xu = s.u();
+        lap = s.laplacian();
+        if (b.any) {
+            damping = -b.xn * b.yn * xu - (b.xn + b.yn) * xv;
+            hwx = (b.yn - b.xh) * s.du_x() * idx1 - b.xh * xwx;
+            hwy = (b.xn - b.yh) * s.du_y() * idx1 - b.yh * xwy;
+        }
+    }
+    T hv = c2 * (lap * idx2 + divergence<T, R, BAND>(P, X, i, j) * idx1);
+    if (b.any) hv += damping;
+    if (i == P.src_i && j == P.src_j && a.src_slot >= 0 && P.has_src) hv += (T)P.sigma[a.src_slot];
+    const T xf[4] = {xu, xv, xwx, xwy}, hf[4] = {xv, hv, hwx, hwy};
+    epilogue<T, TERMS>(P, a, o, xf, hf, b.any, padx, pady);
+}
+
+// FWI gradient with respect to m = c^2: grad += gscale q_v xs (L X_u + D X_w) = gscale q_v d(H X)_v/dm
+template <typename T, int R, bool BAND>
+__device__ __forceinline__ void gradient_point(const ProblemDev& P, const StageArgs& a, int i, int j) {
+    const long long o = (long long)j * P.pitch + i;
+    const T* X = vec_ptr<T>(&P, a.x);
+    T* G = static_cast<T*>(a.grad) + (long long)P.shot * P.field_stride;
+    const T xs = a.x_scale_slot >= 0 ? (T)P.kry[a.x_scale_slot] : T(1);
+    const T g = USums<T, R, BAND>(P, X, i, j).laplacian() * (T)P.inv_dx2 + divergence<T, R, BAND>(P, X, i, j) * (T)P.inv_dx;
+    G[o] += (T)a.gscale * xs * vec_ptr<T>(&P, a.gq)[P.field_stride + o] * g;
+}
+
+// H^T y from y (unscaled): z_v = c^2 y_v, z_x = (by - bx^h) y_wx, z_y = (bx - by^h) y_wy.
+template <typename T, int R, int TERMS>
+__device__ __forceinline__ void transpose_point(const ProblemDev& P, const StageArgs& a, int i, int j) {
+    const int nx = P.nx, ny = P.ny;
+    const bool fs = P.fs != 0;
+    const long long pitch = P.pitch, o = j * pitch + i;
+    const T* X = vec_ptr<T>(&P, a.x);
+    const T* Xv = X + P.field_stride;
+    const T* Xwx = X + 2 * P.field_stride;
+    const T* Xwy = X + 3 * P.field_stride;
+    const T* C2 = static_cast<const T*>(P.c2);
+    const T idx1 = (T)P.inv_dx, idx2 = (T)P.inv_dx2;
+    const bool padx = i >= nx - 1, pady = j >= ny - 1;
+    const T xu = X[o], xv = Xv[o], xwx = padx ? T(0) : Xwx[o], xwy = pady ? T(0) : Xwy[o];
+    const Damping<T> b(P, i, j);
+    T zx[2 * R + 1], zy[2 * R + 1];           // z_v along the row and down the column
+#pragma unroll
+    for (int q = 0; q <= 2 * R; ++q) {
+        const int c = i + q - R, r = j + q - R;
+        zx[q] = (c >= 0 && c < nx) ? C2[o + q - R] * Xv[o + q - R] : T(0);
+        const long long p = o + (q - R) * pitch;
+        zy[q] = (r >= 0 && r < ny) ? C2[p] * Xv[p] : T(0);
+    }
+    // (Lxx^T z_v)(i) = Lxx z_v; (Lyy^T z_v)(j): rows r >= rfs contribute CENT(|r - j|), the
+    // free-surface rows r < 4 FS_UYY[r][j] for j <= 8
+    T lxx = CENT<T, R>(0) * zx[R], lyy = T(0);
+#pragma unroll
+    for (int k = 1; k <= R; ++k) lxx += CENT<T, R>(k) * (zx[R + k] + zx[R - k]);
+    const int rfs = fs ? 4 : 0;
+#pragma unroll
+    for (int k = -R; k <= R; ++k)
+        if (j + k >= rfs) lyy += CENT<T, R>(k < 0 ? -k : k) * zy[R + k];
+    // (Dxn^T z_v)(i+1/2) = sum_k s_k (z_v[i-k] - z_v[i+1+k]); (Dyn^T z_v)(j+1/2) with the rows'
+    // s_k (w[r-1-k] - w[r+k]), the free-surface rows r < 4 FS_DWY[r][j] for j <= 7
+    T dxt = T(0), dyt = T(0);
+#pragma unroll
+    for (int k = 0; k < R; ++k) dxt += STAG<T, R>(k) * (zx[R - k] - zx[R + 1 + k]);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        if (j + 1 + k >= rfs) dyt += STAG<T, R>(k) * zy[R + 1 + k];
+        if (j - k >= rfs) dyt -= STAG<T, R>(k) * zy[R - k];
+    }
+    if (fs && j <= 8) {
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+            if (r >= ny) break;
+            const T z = C2[r * pitch + i] * Xv[r * pitch + i];
+            lyy += fs_coef<T>(FS_UYY_OFF + r * 9 + j) * z;
+            if (j <= 7) dyt += fs_coef<T>(FS_DWY_OFF + r * 8 + j) * z;
+        }
+    }
+    // (Dxh^T z_x)(i) = sum_k s_k (z_x[i-1-k] - z_x[i+k]), the half columns i-R .. i+R-1 (beta
+    // falls towards the middle: none damps unless one of the two ends does)
+    T gxt = T(0), gyt = T(0);
+    if (min(dist_yn(P, j), min(dist_xh(P, max(i - R, 0)), dist_xh(P, min(i + R - 1, nx - 2)))) < 2 * P.pml) {
+#pragma unroll
+        for (int q = 0; q < 2 * R; ++q) {
+            const int p = i - R + q;
+            if (p < 0 || p >= nx - 1) continue;
+            const T z = (b.yn - beta_at<T>(P, dist_xh(P, p))) * Xwx[o + q - R];
+            gxt += (q < R ? STAG<T, R>(R - 1 - q) : -STAG<T, R>(q - R)) * z;
+        }
+    }
+    // (Dyh^T z_y)(j): half rows h >= hfs of d_y u use s_k (u[h-k] - u[h+1+k]), the
+    // free-surface half rows h < 3 FS_UY[h][j] for j <= 7
+    if ((fs && j <= 7) ||
+        min(dist_xn(P, i), min(dist_yh(P, max(j - R, 0)), dist_yh(P, min(j + R - 1, ny - 2)))) < 2 * P.pml) {
+        const int hfs = fs ? 3 : 0;
+#pragma unroll
+        for (int q = 0; q < 2 * R; ++q) {
+            const int h = j - R + q;
+            if (h < hfs || h >= ny - 1) continue;
+            const T z = (b.xn - beta_at<T>(P, dist_yh(P, h))) * Xwy[o + (q - R) * pitch];
+            gyt += (q < R ? -STAG<T, R>(R - 1 - q) : STAG<T, R>(q - R)) * z;
+        }
+        if (fs && j <= 7) {
+#pragma unroll
+            for (int h = 0; h < 3; ++h)
+                if (h < ny - 1)
+                    gyt += fs_coef<T>(FS_UY_OFF + h * 8 + j) *
+                           ((b.xn - beta_at<T>(P, dist_yh(P, h))) * Xwy[h * pitch + i]);
+        }
+    }
+    const T xf[4] = {xu, xv, xwx, xwy};
+    const T hf[4] = {-b.xn * b.yn * xv + (lxx + lyy) * idx2 + (gxt + gyt) * idx1, xu - (b.xn + b.yn) * xv,
+                     padx ? T(0) : dxt * idx1 - b.xh * xwx, pady ? T(0) : dyt * idx1 - b.yh * xwy};
+    epilogue<T, TERMS>(P, a, o, xf, hf, true, padx, pady);
+}
+
+template <typename T, int R, int PASS, int TERMS>
+__device__ __forceinline__ void stage_point(const ProblemDev& P, const StageArgs& a, int lt, int sub) {
+    const PointAt q(P, lt, sub);
+    if (q.i >= P.nx || q.j >= P.ny) return;
+    const bool band = R == 4 && P.fs != 0 && q.j < 4;       // (a warp is one row)
+    if constexpr (PASS == PASS_FORWARD) {
+        if (band) forward_point<T, R, R == 4, TERMS>(P, a, q.i, q.j);
+        else forward_point<T, R, false, TERMS>(P, a, q.i, q.j);
+    } else if constexpr (PASS == PASS_GRADIENT) {
+        if (band) gradient_point<T, R, R == 4>(P, a, q.i, q.j);
+        else gradient_point<T, R, false>(P, a, q.i, q.j);
+    } else {
+        transpose_point<T, R, TERMS>(P, a, q.i, q.j);
+    }
+}
+
+// Every problem of an engine through its tile work list.
+template <typename T, int R, int PASS, int TERMS>
+__global__ void __launch_bounds__(DBX * DBY, 6)
+stage_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ tile_prob, StageArgs a) {
+    const int tile = blockIdx.x / DSUB;
+    const ProblemDev& P = probs[tile_prob[tile]];
+    stage_point<T, R, PASS, TERMS>(P, a, tile - P.tile_base, blockIdx.x % DSUB);
+}
+
+// One problem whose descriptor travels with the launch (H x on a caller's vectors: no device
+// copy of the descriptor to allocate, fill and wait for).
+template <typename T, int R, int PASS, int TERMS>
+__global__ void __launch_bounds__(DBX * DBY, 6)
+stage_one_kernel(const __grid_constant__ ProblemDev P, StageArgs a) {
+    stage_point<T, R, PASS, TERMS>(P, a, blockIdx.x / DSUB, blockIdx.x % DSUB);
+}
+
+// --------------------------------------------------------------------------------------
+// Leap-frog step in FP64 (Sec. 3.1).  Vectors `cur` (u^n, w^n) and `prev` (u^{n-1}, w^{n-1}) use
 // fields 0 (u), 2 (w_x), 3 (w_y); level n+1 overwrites `prev`.  Variant 2 (difference form)
 // reads d^n = u^n - u^{n-1} from field 1 of `prev` instead of u^{n-1} and writes d^{n+1} to
 // field 1 of `cur` (read by no other thread of the step), u^{n+1} = u^n + d^{n+1}.
+// Where nothing damps, the w fields keep their level n-1 values and u^{n+1} needs no division
+// (an FP64 division costs as much as half the stencil).
 // --------------------------------------------------------------------------------------
+template <typename T, int R, bool BAND>
+__device__ __forceinline__ void leapfrog_point(const ProblemDev& P, int i, int j, int cur, int prev, int variant,
+                                               double dt_d) {
+    const int nx = P.nx, ny = P.ny;
+    const long long fstr = P.field_stride, o = (long long)j * P.pitch + i;
+    T* Cn = vec_ptr<T>(&P, cur);
+    T* Pn = vec_ptr<T>(&P, prev);
+    const T dt = (T)dt_d, idx1 = (T)P.inv_dx, idx2 = (T)P.inv_dx2;
+    const bool inx = i < nx - 1, iny = j < ny - 1;
+    const T um = Pn[(variant == 2 ? fstr : 0) + o];
+    const T wxm = inx ? Pn[2 * fstr + o] : T(0), wym = iny ? Pn[3 * fstr + o] : T(0);
+    const T c2 = static_cast<const T*>(P.c2)[o];
+    const Damping<T> b(P, i, j);
+    const T wx = inx ? Cn[2 * fstr + o] : T(0), wy = iny ? Cn[3 * fstr + o] : T(0);
+    T u, lap, gx = T(0), gy = T(0);
+    {
+        const USums<T, R, BAND> s(P, Cn, i, j);
+        u = s.u();
+        lap = s.laplacian();
+        if (b.any) {
+            gx = (b.yn - b.xh) * s.du_x() * idx1;
+            gy = (b.xn - b.yh) * s.du_y() * idx1;
+        }
+    }
+    T rhs = c2 * (lap * idx2 + divergence<T, R, BAND>(P, Cn, i, j) * idx1);
+    if (i == P.src_i && j == P.src_j && P.has_src) rhs += (T)P.sigma[0];
+    T up, wxp = wxm, wyp = wym;
+    if (!b.any) {
+        if (variant == 2) {
+            const T dn = um + dt * dt * rhs;
+            Cn[fstr + o] = dn;
+            up = u + dn;
+        } else {
+            up = (T(2) * u - um) + dt * dt * rhs;
+        }
+    } else {
+        const T bsum = b.xn + b.yn;
+        rhs -= b.xn * b.yn * u;
+        if (variant == 2) {
+            // (u^{n+1} - u^n)(1 + b dt/2) = d^n (1 - b dt/2) + dt^2 rhs, with d^n = um
+            const T hb = T(0.5) * bsum * dt;
+            const T dn = (um * (T(1) - hb) + dt * dt * rhs) / (T(1) + hb);
+            Cn[fstr + o] = dn;
+            up = u + dn;
+        } else {
+            const T inv_dt2 = T(1) / (dt * dt), inv_2dt = T(1) / (T(2) * dt);
+            up = ((T(2) * u - um) * inv_dt2 + bsum * um * inv_2dt + rhs) / (inv_dt2 + bsum * inv_2dt);
+        }
+        if (inx)
+            wxp = variant != 1 ? ((T(1) - b.xh * dt) * wxm + T(2) * dt * gx) / (T(1) + b.xh * dt)
+                               : wxm + T(2) * dt * (-b.xh * wx + gx);
+        if (iny)
+            wyp = variant != 1 ? ((T(1) - b.yh * dt) * wym + T(2) * dt * gy) / (T(1) + b.yh * dt)
+                               : wym + T(2) * dt * (-b.yh * wy + gy);
+    }
+    Pn[o] = up;
+    Pn[2 * fstr + o] = wxp;
+    Pn[3 * fstr + o] = wyp;
+}
+
 template <typename T, int R>
-__global__ void __launch_bounds__(NTHREADS)
+__global__ void __launch_bounds__(DBX * DBY, 6)
 leapfrog_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ tile_prob,
-                int cur, int prev, int variant, double dt_d) {
-    constexpr int SW = BX + 2 * R;
-    constexpr int SH = BY + 2 * R;
-    __shared__ T su[SH][SW];
-    __shared__ T swx[BY][SW];
-    __shared__ T swy[SH][BX];
-    const int pid = tile_prob[blockIdx.x];
-    const ProblemDev* P = probs + pid;
-    const int tx = threadIdx.x, ty = threadIdx.y;
-    const int nx = P->nx, ny = P->ny, pitch = P->pitch, pml = P->pml;
-    const bool fs = P->fs != 0;
-    const int lt = blockIdx.x - P->tile_base;
-    const int x0 = (lt % P->tiles_x) * BX, y0 = (lt / P->tiles_x) * BY;
-    const long long fstr = P->field_stride;
-    const T beta0 = (T)P->beta0, inv_pml = (T)P->inv_pml;
-    const T idx1 = (T)P->inv_dx, idx2 = (T)P->inv_dx2;
-    const T dt = (T)dt_d;
-    T* Cn = vec_ptr<T>(P, cur);
-    T* Pn = vec_ptr<T>(P, prev);
-    const T* C2 = (const T*)P->c2;
-    T pum[VY][VX], pwxm[VY][VX], pwym[VY][VX], pc2[VY][VX];
-#pragma unroll
-    for (int b = 0; b < VY; ++b)
-#pragma unroll
-        for (int c = 0; c < VX; ++c) {
-            const int i = x0 + tx + c * TPX, j = y0 + ty + b * TPY;
-            const bool in = (i < nx) && (j < ny);
-            const long long o = (long long)j * pitch + i;
-            pum[b][c] = in ? Pn[(variant == 2 ? fstr : 0) + o] : T(0);
-            pwxm[b][c] = in ? Pn[2 * fstr + o] : T(0);
-            pwym[b][c] = in ? Pn[3 * fstr + o] : T(0);
-            pc2[b][c] = in ? C2[o] : T(0);
-        }
-    for (int r = ty; r < SH; r += TPY) {
-        const int gy = y0 - R + r;
-        const bool rok = gy >= 0 && gy < ny;
-        const T* row = Cn + (long long)(rok ? gy : 0) * pitch;
-        for (int c = tx; c < SW; c += TPX) {
-            const int gx = x0 - R + c;
-            su[r][c] = (rok && gx >= 0 && gx < nx) ? row[gx] : T(0);
-        }
-    }
-    for (int r = ty; r < BY; r += TPY) {
-        const int gy = y0 + r;
-        const bool rok = gy < ny;
-        const T* row = Cn + 2 * fstr + (long long)(rok ? gy : 0) * pitch;
-        for (int c = tx; c < SW; c += TPX) {
-            const int gx = x0 - R + c;
-            swx[r][c] = (rok && gx >= 0 && gx < nx - 1) ? row[gx] : T(0);
-        }
-    }
-    for (int r = ty; r < SH; r += TPY) {
-        const int gy = y0 - R + r;
-        const bool rok = gy >= 0 && gy < ny - 1;
-        const T* row = Cn + 3 * fstr + (long long)(rok ? gy : 0) * pitch;
-        for (int c = tx; c < BX; c += TPX) {
-            const int gx = x0 + c;
-            swy[r][c] = (rok && gx < nx) ? row[gx] : T(0);
-        }
-    }
-    __syncthreads();
-    const T sig = P->has_src ? (T)P->sigma[0] : T(0);
-#pragma unroll
-    for (int b = 0; b < VY; ++b)
-#pragma unroll
-        for (int c = 0; c < VX; ++c) {
-            const int lx = tx + c * TPX, ly = ty + b * TPY;
-            const int i = x0 + lx, j = y0 + ly;
-            if (i >= nx || j >= ny) continue;
-            const long long o = (long long)j * pitch + i;
-            const T bxn = damp<T>(beta0, inv_pml, T(min(i + 1, nx - i)), pml);
-            const T byn = damp<T>(beta0, inv_pml, fs ? T(ny - j) : T(min(j + 1, ny - j)), pml);
-            const T bxh = damp<T>(beta0, inv_pml, min(T(i) + T(1.5), T(nx - i) - T(0.5)), pml);
-            const T byh = damp<T>(beta0, inv_pml,
-                                  fs ? (T(ny - j) - T(0.5)) : min(T(j) + T(1.5), T(ny - j) - T(0.5)),
-                                  pml);
-            const T u = su[ly + R][lx + R];
-            T uxx = CENT<T, R>(0) * u;
-#pragma unroll
-            for (int k = 1; k <= R; ++k)
-                uxx += CENT<T, R>(k) * (su[ly + R][lx + R + k] + su[ly + R][lx + R - k]);
-            T uyy;
-            if (fs && j < 4) {
-                uyy = T(0);
-#pragma unroll
-                for (int q = 0; q < 9; ++q)
-                    uyy += fs_coef<T>(FS_UYY_OFF + j * 9 + q) * su[q - y0 + R][lx + R];
-            } else {
-                uyy = CENT<T, R>(0) * u;
-#pragma unroll
-                for (int k = 1; k <= R; ++k)
-                    uyy += CENT<T, R>(k) * (su[ly + R + k][lx + R] + su[ly + R - k][lx + R]);
-            }
-            T dwx = T(0);
-#pragma unroll
-            for (int k = 0; k < R; ++k)
-                dwx += STAG<T, R>(k) * (swx[ly][lx + R + k] - swx[ly][lx + R - 1 - k]);
-            T dwy = T(0);
-            if (fs && j < 4) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    dwy += fs_coef<T>(FS_DWY_OFF + j * 8 + q) * swy[q - y0 + R][lx];
-            } else {
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    dwy += STAG<T, R>(k) * (swy[ly + R - 1 - k][lx] - swy[ly + R + k][lx]);
-            }
-            T dux = T(0);
-#pragma unroll
-            for (int k = 0; k < R; ++k)
-                dux += STAG<T, R>(k) * (su[ly + R][lx + R + 1 + k] - su[ly + R][lx + R - k]);
-            T duy = T(0);
-            if (fs && j < 3) {
-#pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    duy += fs_coef<T>(FS_UY_OFF + j * 8 + q) * su[q - y0 + R][lx + R];
-            } else {
-#pragma unroll
-                for (int k = 0; k < R; ++k)
-                    duy += STAG<T, R>(k) * (su[ly + R - k][lx + R] - su[ly + R + 1 + k][lx + R]);
-            }
-            const T bsum = bxn + byn;
-            T rhs = -bxn * byn * u + pc2[b][c] * ((uxx + uyy) * idx2 + (dwx + dwy) * idx1);
-            if (i == P->src_i && j == P->src_j) rhs += sig;
-            const T um = pum[b][c];
-            T up;
-            if (variant == 2) {
-                // (u^{n+1} - u^n)(1 + b dt/2) = d^n (1 - b dt/2) + dt^2 rhs, with d^n = um
-                const T hb = T(0.5) * bsum * dt;
-                const T dn = (um * (T(1) - hb) + dt * dt * rhs) / (T(1) + hb);
-                Cn[fstr + o] = dn;
-                up = u + dn;
-            } else {
-                const T inv_dt2 = T(1) / (dt * dt), inv_2dt = T(1) / (T(2) * dt);
-                up = ((T(2) * u - um) * inv_dt2 + bsum * um * inv_2dt + rhs) / (inv_dt2 + bsum * inv_2dt);
-            }
-            T wxp = T(0), wyp = T(0);
-            if (i < nx - 1) {
-                const T gx = (byn - bxh) * dux * idx1;
-                wxp = variant != 1 ? ((T(1) - bxh * dt) * pwxm[b][c] + T(2) * dt * gx) / (T(1) + bxh * dt)
-                                   : pwxm[b][c] + T(2) * dt * (-bxh * swx[ly][lx + R] + gx);
-            }
-            if (j < ny - 1) {
-                const T gy = (bxn - byh) * duy * idx1;
-                wyp = variant != 1 ? ((T(1) - byh * dt) * pwym[b][c] + T(2) * dt * gy) / (T(1) + byh * dt)
-                                   : pwym[b][c] + T(2) * dt * (-byh * swy[ly + R][lx] + gy);
-            }
-            Pn[o] = up;
-            Pn[2 * fstr + o] = wxp;
-            Pn[3 * fstr + o] = wyp;
-        }
+                int cur, int prev, int variant, double dt) {
+    const int tile = blockIdx.x / DSUB;
+    const ProblemDev& P = probs[tile_prob[tile]];
+    const PointAt q(P, tile - P.tile_base, blockIdx.x % DSUB);
+    if (q.i >= P.nx || q.j >= P.ny) return;
+    if (R == 4 && P.fs != 0 && q.j < 4) leapfrog_point<T, R, R == 4>(P, q.i, q.j, cur, prev, variant, dt);
+    else leapfrog_point<T, R, false>(P, q.i, q.j, cur, prev, variant, dt);
 }
 
 // --------------------------------------------------------------------------------------
-void launch_stage(int precision, int R, int nblocks, const ProblemDev* probs,
-                  const int* tile_prob, const StageArgs& a, cudaStream_t s) {
-    const dim3 block(TPX, TPY);
-    if (nblocks <= 0) return;
-    if (precision == 0) {
-        if (R == 4) {
-            if (a.transpose) stage_kernel<float, 4, true><<<nblocks, block, 0, s>>>(probs, tile_prob, a);
-            else stage_kernel<float, 4, false><<<nblocks, block, 0, s>>>(probs, tile_prob, a);
-        } else {
-            if (a.transpose) stage_kernel<float, 2, true><<<nblocks, block, 0, s>>>(probs, tile_prob, a);
-            else stage_kernel<float, 2, false><<<nblocks, block, 0, s>>>(probs, tile_prob, a);
+template <int V>
+using Int = std::integral_constant<int, V>;
+
+// Calls launch(T(), Int<R>, Int<PASS>) for the pass that `a` asks for.
+template <int PASS, class F>
+static void with_type(int precision, int R, F&& launch) {
+    if (precision == 0 && R == 4) launch(float(), Int<4>(), Int<PASS>());
+    else if (precision == 0) launch(float(), Int<2>(), Int<PASS>());
+    else if (R == 4) launch(double(), Int<4>(), Int<PASS>());
+    else launch(double(), Int<2>(), Int<PASS>());
+}
+template <class F>
+static void with_pass(int precision, int R, const StageArgs& a, F&& launch) {
+    if (a.transpose) with_type<PASS_TRANSPOSE>(precision, R, launch);
+    else if (a.grad) with_type<PASS_GRADIENT>(precision, R, launch);
+    else with_type<PASS_FORWARD>(precision, R, launch);
+}
+
+void launch_stage(int precision, int R, int ntiles, const ProblemDev* probs, const int* tile_prob,
+                  const StageArgs& a_in, cudaStream_t s) {
+    if (ntiles <= 0) return;
+    StageArgs a = a_in;
+    a.terms = stage_terms(a);
+    with_pass(precision, R, a, [&](auto zero, auto r, auto pass) {
+        using T = decltype(zero);
+        constexpr int RR = decltype(r)::value, PASS = decltype(pass)::value;
+        const int blocks = ntiles * DSUB;
+        const dim3 block(DBX, DBY);
+        if constexpr (sizeof(T) == 8 && PASS == PASS_FORWARD) {
+            constexpr int FABER = TERM_CX | TERM_CU | TERM_A | TERM_CAY, HORK = TERM_CX | TERM_A | TERM_CAY;
+            switch (a.terms) {
+                case FABER: stage_kernel<T, RR, PASS, FABER><<<blocks, block, 0, s>>>(probs, tile_prob, a); return;
+                case HORK: stage_kernel<T, RR, PASS, HORK><<<blocks, block, 0, s>>>(probs, tile_prob, a); return;
+                case TERM_CU: stage_kernel<T, RR, PASS, TERM_CU><<<blocks, block, 0, s>>>(probs, tile_prob, a); return;
+                case TERM_XS: stage_kernel<T, RR, PASS, TERM_XS><<<blocks, block, 0, s>>>(probs, tile_prob, a); return;
+                default: break;
+            }
         }
-    } else {
-        if (R == 4) {
-            if (a.transpose) stage_kernel<double, 4, true><<<nblocks, block, 0, s>>>(probs, tile_prob, a);
-            else stage_kernel<double, 4, false><<<nblocks, block, 0, s>>>(probs, tile_prob, a);
-        } else {
-            if (a.transpose) stage_kernel<double, 2, true><<<nblocks, block, 0, s>>>(probs, tile_prob, a);
-            else stage_kernel<double, 2, false><<<nblocks, block, 0, s>>>(probs, tile_prob, a);
-        }
-    }
+        stage_kernel<T, RR, PASS, -1><<<blocks, block, 0, s>>>(probs, tile_prob, a);
+    });
+}
+
+// (only y = H x and y = H^T x come here: no term but the product)
+int launch_stage_one(int precision, int R, const ProblemDev& P, const StageArgs& a, cudaStream_t s) {
+    if (stage_terms(a) != 0 || a.grad || a.store_bf16) return -1;
+    with_pass(precision, R, a, [&](auto zero, auto r, auto pass) {
+        constexpr int PASS = decltype(pass)::value;
+        if constexpr (PASS != PASS_GRADIENT)
+            stage_one_kernel<decltype(zero), decltype(r)::value, PASS, 0>
+                <<<P.ntiles * DSUB, dim3(DBX, DBY), 0, s>>>(P, a);
+    });
+    return 0;
+}
+
+void launch_leapfrog(int R, int ntiles, const ProblemDev* probs, const int* tile_prob, int cur, int prev,
+                     int variant, double dt, cudaStream_t s) {
+    if (ntiles <= 0) return;
+    const dim3 block(DBX, DBY);
+    if (R == 4) leapfrog_kernel<double, 4><<<ntiles * DSUB, block, 0, s>>>(probs, tile_prob, cur, prev, variant, dt);
+    else leapfrog_kernel<double, 2><<<ntiles * DSUB, block, 0, s>>>(probs, tile_prob, cur, prev, variant, dt);
 }
 
 // --------------------------------------------------------------------------------------
@@ -707,20 +714,6 @@ void launch_leapfrog_adjoint(int precision, int nblocks, const ProblemDev* probs
         leapfrog_adjoint_kernel<float><<<nblocks, block, 0, s>>>(probs, tile_prob, mode, qv, yv, a1_base, dt);
     else
         leapfrog_adjoint_kernel<double><<<nblocks, block, 0, s>>>(probs, tile_prob, mode, qv, yv, a1_base, dt);
-}
-
-void launch_leapfrog(int precision, int R, int nblocks, const ProblemDev* probs,
-                     const int* tile_prob, int cur, int prev, int variant, double dt,
-                     cudaStream_t s) {
-    const dim3 block(TPX, TPY);
-    if (nblocks <= 0) return;
-    if (precision == 0) {
-        if (R == 4) leapfrog_kernel<float, 4><<<nblocks, block, 0, s>>>(probs, tile_prob, cur, prev, variant, dt);
-        else leapfrog_kernel<float, 2><<<nblocks, block, 0, s>>>(probs, tile_prob, cur, prev, variant, dt);
-    } else {
-        if (R == 4) leapfrog_kernel<double, 4><<<nblocks, block, 0, s>>>(probs, tile_prob, cur, prev, variant, dt);
-        else leapfrog_kernel<double, 2><<<nblocks, block, 0, s>>>(probs, tile_prob, cur, prev, variant, dt);
-    }
 }
 
 }  // namespace ewv

@@ -359,8 +359,10 @@ class Model:
 
     # ---------------------------------------------------------------- compute
     def apply_device(self, x, y, transpose=False):
-        self._check(self.lib.ewv_apply_operator(self.h, int(transpose), ctypes.c_void_p(x.data_ptr()),
-                                                ctypes.c_void_p(y.data_ptr())), "apply_operator")
+        self._check(self.lib.ewv_apply_operator(self.h, int(transpose), x.data_ptr(), y.data_ptr()),
+                    "apply_operator")
+        if self.stream.cuda_stream != self.torch._C._cuda_getCurrentRawStream(self.stream.device_index):
+            self.stream.synchronize()    # x and y belong to the caller's stream
 
     def apply(self, compact, transpose=False):
         x, y = self.new_vector(), self.new_vector()
