@@ -506,9 +506,9 @@ int ewv_debug_set_wait_limit(unsigned long long ns);
  * column's modified Gram-Schmidt steps on the column kernel -- one cooperative launch per
  * column with q_{j+1} in shared memory and a bounded grid barrier per step, taken when every
  * flat chunk of the engine fits one co-resident grid -- (1, the default) or on one flat
- * pass per step (0).  In FP32 both give the same values bit for bit; in FP64 the flat form
- * fuses the first dot of a column into the stencil pass, so they agree to rounding.
- * Process-wide; waits for the device to be idle first. */
+ * pass per step (0).  Both give the same values bit for bit.  FP32 problem sets too large for
+ * the column kernel take two passes per column (dots and a triangular solve, then the update)
+ * whatever this is set to.  Process-wide; waits for the device to be idle first. */
 int ewv_debug_set_column_kernel(int enable);
 
 #ifdef __cplusplus

@@ -223,6 +223,8 @@ struct Engine {
     // only), double-buffered partials and the grid-barrier words
     int mgs_cpb = 0;
     double* d_mgs_partials = nullptr;
+    double* d_gs_partials = nullptr;   // FP32 Gram-Schmidt passes (allocated at their first use)
+    double* d_gram = nullptr;
     unsigned int* d_mgs_bar = nullptr;
     double* d_ecoef = nullptr;    // [nprob][MAX_TAU][MAX_M]: exp(tau H) e_1 of a multi-output combine
     // adaptive Krylov step: tolerance, dimension range and statistics of the current call
@@ -295,6 +297,8 @@ struct Engine {
         cudaFree(d_kadj);
         cudaFree(d_kexp_maps);
         cudaFree(d_mgs_partials);
+        cudaFree(d_gs_partials);
+        cudaFree(d_gram);
         cudaFree(d_mgs_bar);
         cudaFree(d_ecoef);
         cudaFree(d_kbar);
@@ -311,15 +315,9 @@ struct ewv_batch {
 
 namespace {
 
-// Krylov steps run each Arnoldi column's Gram-Schmidt steps on the column kernel when the
-// engine's chunks fit one co-resident grid (ewv_debug_set_column_kernel(0) keeps the flat
-// passes, for comparisons)
+// Modified Gram-Schmidt steps run on the column kernel when the engine's chunks fit one
+// co-resident grid (ewv_debug_set_column_kernel(0) keeps the flat passes, for comparisons)
 bool g_mgs_enabled = true;
-
-// One column's Gram-Schmidt steps (first dot, then k = k0 .. kmax) on the column kernel over
-// nprob problems laid out like the engine's (its chunk table); false if it cannot run.
-bool mgs_column(Engine* E, int precision, const ProblemDev* probs, int nprob, int j, int k0, int kmax, int m,
-                double tol, cudaStream_t s);
 
 int fail(std::string& err, int code, const char* fmt, ...) {
     char buf[512];
@@ -509,6 +507,10 @@ int build_engine(Engine* E, std::string& err) {
         E->d_mgs_partials = nullptr;
         E->d_mgs_bar = nullptr;
         E->mgs_cpb = mgs_column_chunks_per_block(E->precision, E->nchunks);
+        cudaFree(E->d_gs_partials);
+        cudaFree(E->d_gram);
+        E->d_gs_partials = nullptr;
+        E->d_gram = nullptr;
         cudaFree(E->d_ecoef);
         E->d_ecoef = nullptr;
         CUDA_OR_FAIL(err, cudaMalloc(&E->d_ecoef, sizeof(double) * (size_t)E->nprob * MAX_TAU * MAX_M));
@@ -1105,19 +1107,75 @@ int run_rk(Ctx& C, double t, double dt, int scheme, int nsteps) {
     return check_launch(*C.err);
 }
 
-bool mgs_column(Engine* E, int precision, const ProblemDev* probs, int nprob, int j, int k0, int kmax, int m,
-                double tol, cudaStream_t s) {
-    if (E->mgs_cpb <= 0 || nprob != E->nprob || !E->d_mgs_partials || !E->d_mgs_bar) return false;
-    MgsArgs ma{};
-    ma.j = j;
-    ma.k0 = k0;
-    ma.kmax = kmax;
-    ma.m = m;
-    ma.tol = tol;
-    ma.partials = E->d_mgs_partials;
-    ma.bar = E->d_mgs_bar;
-    ma.err = E->d_err;
-    return launch_mgs_column(precision, E->nchunks, E->mgs_cpb, probs, E->d_pbase, nprob, ma, s) == 0;
+// Whether the engine's Arnoldi columns take the two Gram-Schmidt passes (see gram_schmidt).
+bool gs_two_pass(const Engine* E) { return E->precision == EWV_F32 && E->mgs_cpb == 0; }
+
+// Buffers of the two Gram-Schmidt passes (not inside a capture).
+int gs_ready(Engine* E, std::string& err) {
+    if (!gs_two_pass(E)) return EWV_OK;
+    if (!E->d_gs_partials)
+        CUDA_OR_FAIL(err, cudaMalloc(&E->d_gs_partials, sizeof(double) * 2 * MAX_M * (size_t)E->nchunks));
+    if (!E->d_gram) CUDA_OR_FAIL(err, cudaMalloc(&E->d_gram, sizeof(double) * MAX_M * MAX_M * (size_t)E->nprob));
+    return EWV_OK;
+}
+
+// Gram-Schmidt of Arnoldi column j (q_{j+1} = the product, against q_k0 .. q_j) over the problems
+// `probs`, laid out like the engine's; m: the last column, whose h_{m+1,m} is not needed.
+//   FP32 problem sets too large for one co-resident grid (E->mgs_cpb 0, above ~30 MB a vector):
+//     the two passes of kernels_gs.cu, 2 j + 3 vectors moved and two launches a column where a pass
+//     per step moves 4 j (Krylov 20, 1001 x 501, 16 shots: 24.0 -> 12.0 ms a step).
+//   FP32 sets that fit: modified Gram-Schmidt step by step in one cooperative launch.  The two
+//     passes are faster there too (5.2 -> 3.6 ms of a step on 401 x 201, 16 shots), but another
+//     order of the sums moves the gradient of the large Krylov steps used for inversion (dt |H|
+//     near m) by 1.3e-5 to 2.1e-5: it amplifies FP32 rounding about a hundredfold.
+//   FP64: the cooperative launch, or a pass per step: its dots are bound by the FP64 pipe, which
+//     the two passes would load with twice the dots.
+void gram_schmidt(Engine* E, const ProblemDev* probs, int j, int k0, int m, double tol, cudaStream_t s,
+                  long long* launches) {
+    const int np = E->nprob;
+    if (gs_two_pass(E)) {
+        GsArgs ga{};
+        ga.j = j;
+        ga.k0 = k0;
+        ga.m = m;
+        ga.tol = tol;
+        ga.partials = E->d_gs_partials;
+        ga.counters = E->d_counters;
+        ga.gram = E->d_gram;
+        launch_gs_column(E->nchunks, probs, E->d_pbase, np, ga, s);
+        *launches += j < m ? 2 : 1;
+        return;
+    }
+    // at j = m the pass k = m only feeds h_{m+1,m}
+    const int kmax = j == m ? j - 1 : j;
+    if (g_mgs_enabled && E->mgs_cpb > 0 && E->d_mgs_partials && E->d_mgs_bar) {
+        MgsArgs ma{};
+        ma.j = j;
+        ma.k0 = k0;
+        ma.kmax = kmax;
+        ma.m = m;
+        ma.tol = tol;
+        ma.partials = E->d_mgs_partials;
+        ma.bar = E->d_mgs_bar;
+        ma.err = E->d_err;
+        if (launch_mgs_column(E->precision, E->nchunks, E->mgs_cpb, probs, E->d_pbase, np, ma, s) == 0) {
+            ++*launches;
+            return;
+        }
+    }
+    PointArgs pa{};
+    pa.j = j;
+    pa.m = m;
+    pa.tol = tol;
+    pa.partials = E->d_partials;
+    pa.counters = E->d_counters;
+    pa.mode = 5;               // <q_{j+1}, q_k0>
+    pa.k = k0;
+    launch_point_flat(E->precision, E->nchunks, probs, E->d_pbase, np, pa, s);
+    pa.mode = 1;
+    for (pa.k = k0; pa.k <= kmax; ++pa.k)
+        launch_point_flat(E->precision, E->nchunks, probs, E->d_pbase, np, pa, s);
+    *launches += 1 + std::max(0, kmax - k0 + 1);
 }
 
 int run_krylov(Ctx& C, double t, double dt, int m, int nsteps, int* info) {
@@ -1128,9 +1186,11 @@ int run_krylov(Ctx& C, double t, double dt, int m, int nsteps, int* info) {
     ++*C.launches;
     bool expm_ok = true;
     const int window = C.E->models.empty() ? 0 : C.E->models[0]->kry_window;
-    // The matrix-vector product has no dot partner; a flat pass then forms <q_{j+1}, q_k0>
-    // (the plain FP64 3D kernel keeps its fused dot, with the same finalisation)
-    const bool split_dot = C.E->precision == EWV_F32 || C.E->dims == 2;
+    int rc_gs = gs_ready(C.E, err);
+    if (rc_gs != EWV_OK) return rc_gs;
+    // The 3D FP64 product carries its first dot with it (the plain kernel of kernels_3d.cu); every
+    // other product is followed by the Gram-Schmidt of its column.
+    const bool fused_dot = C.E->precision == EWV_F64 && C.E->dims == 3 && !(g_mgs_enabled && C.E->mgs_cpb > 0);
     // dense output: before the step's own combine (which overwrites q_1 = U^{n-1}), the states
     // x(tau_q dt) = beta V exp(tau_q H_m) e_1 at the 4-point Gauss-Legendre nodes go to the
     // caller's buffer [q][shot]; a key of its own keeps such a call out of the step graphs
@@ -1148,45 +1208,30 @@ int run_krylov(Ctx& C, double t, double dt, int m, int nsteps, int* info) {
         pn.partials = C.E->d_partials;
         pn.counters = C.E->d_counters;
         C.point(pn);
-        const bool col = g_mgs_enabled && C.E->mgs_cpb > 0;
         for (int j = 1; j <= m; ++j) {
             // orthogonalise q_{j+1} against q_{k0} .. q_j (all of them without a window)
             const int k0 = window > 0 ? std::max(1, j - window + 1) : 1;
             StageArgs a = stage_defaults();
             a.x = j - 1;
             a.y_out = j;
-            a.d = k0 - 1;
             a.src_slot = j;
             a.x_scale_slot = KRY_S + j;
             a.ch = dt;
             a.ck = 1.0;
-            a.fin_mode = FIN_MATVEC;
-            a.fin_j = j;
-            a.fin_k = k0;
-            a.m = m;
-            a.tol = tol;
-            a.partials = C.E->d_partials;
-            a.counters = C.E->d_counters;
-            if (split_dot || col) {
-                a.d = -1;
-                a.fin_mode = FIN_NONE;
+            if (fused_dot) {
+                a.d = k0 - 1;
+                a.fin_mode = FIN_MATVEC;
+                a.fin_j = j;
+                a.fin_k = k0;
+                a.m = m;
+                a.tol = tol;
+                a.partials = C.E->d_partials;
+                a.counters = C.E->d_counters;
             }
             C.stage(a);
-            if (col && mgs_column(C.E, C.E->precision, C.E->d_probs, C.E->nprob, j, k0, (j == m) ? j - 1 : j, m,
-                                  tol, C.s)) {
-                ++*C.launches;
+            if (!fused_dot) {
+                gram_schmidt(C.E, C.E->d_probs, j, k0, m, tol, C.s, C.launches);
                 continue;
-            }
-            if (split_dot || col) {        // (col: the column kernel could not be launched)
-                PointArgs pd{};
-                pd.mode = 5;
-                pd.j = j;
-                pd.k = k0;
-                pd.m = m;
-                pd.tol = tol;
-                pd.partials = C.E->d_partials;
-                pd.counters = C.E->d_counters;
-                C.point(pd);
             }
             // at j = m the pass k = m only feeds h_{m+1,m}, which the result does not use
             const int kmax = (j == m) ? j - 1 : j;
@@ -1364,6 +1409,8 @@ int run_krylov_adaptive(Ctx& C, double t, double dt, double tol, int mmin, int m
     if (mmin < 1 || mmax < mmin || mmax + 1 > MAX_M || !(tol > 0.0))
         return fail(err, EWV_ERR_INVALID_ARG, "adaptive Krylov: need 1 <= m_min <= m_max <= %d, tol > 0", MAX_M - 1);
     const int np = E->nprob;
+    int rc_gs = gs_ready(E, err);
+    if (rc_gs != EWV_OK) return rc_gs;
     const double btol = E->precision == EWV_F64 ? 1e-14 : 1e-6;
     const int window = E->models.empty() ? 0 : E->models[0]->kry_window;
     std::vector<std::vector<double>> kb((size_t)np, std::vector<double>(KRY_STRIDE));
@@ -1442,8 +1489,12 @@ int run_krylov_adaptive(Ctx& C, double t, double dt, double tol, int mmin, int m
                     matvec(j);
                     ++tot_mv;
                 }
-                flat(5, j, k0, 0);                 // <q_{j+1}, q_k0> -> tail_{j+1}, h_{k0,j}
-                for (int k = k0; k <= j; ++k) flat(1, j, k, 0);
+                if (gs_two_pass(E)) {
+                    gram_schmidt(E, E->d_probs, j, k0, mmax + 1, btol, C.s, C.launches);
+                } else {
+                    flat(5, j, k0, 0);             // <q_{j+1}, q_k0> -> tail_{j+1}, h_{k0,j}
+                    for (int k = k0; k <= j; ++k) flat(1, j, k, 0);
+                }
                 have_next = false;
                 if (j >= mmin && j < mmax + 1) {
                     matvec(j + 1);                 // A v_{j+1}: the estimate, reused by column j+1
@@ -2481,7 +2532,8 @@ static int adjoint_krylov(ewv_model* m, Engine* E, double t, double dt, int mm, 
                                  0.32607257743127307, 0.17392742256872693};
     const int fset = tma ? tma_map_set(tma_variant_tile_height_for(E->tma_variant, false)) : 0;
     const int trset = tma_map_set(18), gset = tma_map_set(30);
-    const bool col = g_mgs_enabled && E->mgs_cpb > 0 && E->nprob == ns;
+    const int rc_gs = gs_ready(E, m->err);
+    if (rc_gs != EWV_OK) return rc_gs;
     auto arnoldi = [&](const ProblemDev* v, bool transpose) {
         PointArgs pn{};
         pn.mode = 0;
@@ -2510,33 +2562,7 @@ static int adjoint_krylov(ewv_model* m, Engine* E, double t, double dt, int mm, 
                                : launch_stage_tma(E->tma_variant, R, v, tbs, ns, E->ntiles_by[set], a, E->d_err, s);
             if (rc != 0) launch_stage(prec, R, tb, v, d_tp, a, s);
             ++m->launches;
-            const int kmax = (j == mm) ? j - 1 : j;
-            if (col && mgs_column(E, prec, v, ns, j, 1, kmax, mm, tol, s)) {
-                ++m->launches;
-                continue;
-            }
-            PointArgs pd{};
-            pd.mode = 5;
-            pd.j = j;
-            pd.k = 1;
-            pd.m = mm;
-            pd.tol = tol;
-            pd.partials = E->d_partials;
-            pd.counters = E->d_counters;
-            launch_point_flat(prec, E->nchunks, v, E->d_pbase, ns, pd, s);
-            ++m->launches;
-            for (int k = 1; k <= kmax; ++k) {
-                PointArgs pm{};
-                pm.mode = 1;
-                pm.j = j;
-                pm.k = k;
-                pm.m = mm;
-                pm.tol = tol;
-                pm.partials = E->d_partials;
-                pm.counters = E->d_counters;
-                launch_point_flat(prec, E->nchunks, v, E->d_pbase, ns, pm, s);
-                ++m->launches;
-            }
+            gram_schmidt(E, v, j, 1, mm, tol, s, &m->launches);
         }
     };
     // dense output of a basis at ntau values of tau from one read of it: vectors dst .. dst + 3

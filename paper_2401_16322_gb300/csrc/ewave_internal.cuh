@@ -258,6 +258,18 @@ struct ExpmTaus {
 int launch_expm_multi(const ProblemDev* probs, int nprob, int mmax, cudaStream_t s, const double* taus, int ntau,
                       double* out);
 
+// kernels_gs.cu (FP32): Gram-Schmidt of one Arnoldi column over the flat chunks in two passes
+// (the second only while j < m): column j of H, q_{j+1}, its tail, h_{j+1,j} and s_{j+1}.
+struct GsArgs {
+    int j, k0, m;
+    double tol;
+    double* partials;         // 2 MAX_M nchunks
+    unsigned int* counters;   // one per problem
+    double* gram;             // MAX_M x MAX_M per problem: <v_k, v_i>, i < k
+};
+void launch_gs_column(int nchunks, const ProblemDev* probs, const int* pbase, int nprob, const GsArgs& ga,
+                      cudaStream_t s);
+
 // kernels_mgs.cu: the modified Gram-Schmidt steps of one Arnoldi column (first dot, then
 // k = k0 .. kmax) in one cooperative launch over the flat chunks, q_{j+1} in shared memory.
 constexpr int MGS_MAX_CPB = 4;   // chunks per block at most

@@ -1,5 +1,6 @@
 // Modified Gram-Schmidt of one Arnoldi column in one cooperative launch (Sec. 3.2, the inner
-// loop of the Krylov listing).
+// loop of the Krylov listing), for problem sets whose chunks fit one co-resident grid (larger
+// FP32 sets take the two passes of kernels_gs.cu).
 //
 // After the product q_{j+1} = dt H~ v_j (its own pass, without a dot), the column's steps
 //   h_{k0,j} = <q_{j+1}, v_{k0}>,
@@ -14,8 +15,7 @@
 // Layout: block b owns the flat passes' chunks b cpb .. b cpb + cpb - 1 (PCHUNK elements of one
 // problem's padded vector each, found through the chunk table), with the same thread-to-element
 // mapping, the same per-chunk partial sums and the same fixed-order totals as the flat passes,
-// so both forms give the same values bit for bit (FP32; in FP64 the flat form fuses the first
-// dot into the stencil pass, another summation order).  Each step's partials go to a buffer of
+// so both forms give the same values bit for bit.  Each step's partials go to a buffer of
 // their own (two, alternating), a grid barrier makes them visible, and every block sums its
 // problems' partials and replays the scalar recurrence on a private copy of tail_{j+1} and of
 // column j of H; the block that owns a problem's chunk 0 writes the results back.
