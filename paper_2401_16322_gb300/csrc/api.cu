@@ -808,7 +808,13 @@ struct Ctx {
         launch_record(E->precision, E->d_probs, E->nprob, vec, s);
         ++*launches;
     }
-    // Run nsteps steps.  Steps are parameter-free (time comes from the device clock), so
+    // record, and the source scalars of the next step (prologue() gives those of a call's first)
+    void record_next(int vec, int kind, int m, double g = 0, double c0 = 0, double c1 = 0) {
+        launch_record_next(E->precision, E->d_probs, E->nprob, vec, kind, m, g, c0, c1, s);
+        ++*launches;
+    }
+    // Run nsteps steps.  Steps are parameter-free (time comes from the device clock, and a step
+    // ends by preparing the source scalars of the next: record_next), so
     // after the first step(s) the launch sequence of one step is captured once into a CUDA
     // graph and replayed; `nparity` distinct sequences alternate (leap-frog buffer swap).
     // With kernel timing on, the captured step records its own event pairs (external event
@@ -892,8 +898,8 @@ int run_faber(Ctx& C, double t, double dt, int m, int nsteps, double g, double c
     const std::vector<double>& a = it->second;
     launch_set_clock(C.E->d_probs, C.E->nprob, t, dt, C.s);
     ++*C.launches;
+    C.prologue(PRO_FABER, m, g, c0, c1);
     int rc = C.step_loop(nsteps, EWV_METHOD_FABER, m, dt, g, c0, c1, 1, [&](int) {
-        C.prologue(PRO_FABER, m, g, c0, c1);
         StageArgs s1 = stage_defaults();
         s1.x = 0;
         s1.y_out = 1;
@@ -941,7 +947,7 @@ int run_faber(Ctx& C, double t, double dt, int m, int nsteps, double g, double c
                 C.stage(sj);
             }
         }
-        C.record();
+        C.record_next(0, PRO_FABER, m, g, c0, c1);
     });
     if (rc != EWV_OK) return rc;
     return check_launch(err);
@@ -975,8 +981,8 @@ std::vector<double> hork_lambdas(int m) {
 int run_hork_horner(Ctx& C, double t, double dt, int m, int nsteps) {
     launch_set_clock(C.E->d_probs, C.E->nprob, t, dt, C.s);
     ++*C.launches;
+    C.prologue(PRO_HORK_HORNER, m);
     int rc = C.step_loop(nsteps, EWV_METHOD_HORK, m, dt, 0, 0, 0, 1, [&](int) {
-        C.prologue(PRO_HORK_HORNER, m);
         int prev = 0;
         for (int k = 0; k < m; ++k) {
             const int j = m - k;
@@ -997,7 +1003,7 @@ int run_hork_horner(Ctx& C, double t, double dt, int m, int nsteps) {
             prev = s.y_out;
         }
         if (prev != 0) C.copy(prev, 0, ALL_FIELDS, false);   // m = 1: V_1 is in a work vector
-        C.record();
+        C.record_next(0, PRO_HORK_HORNER, m);
     });
     if (rc != EWV_OK) return rc;
     return check_launch(*C.err);
@@ -1012,8 +1018,8 @@ int run_hork(Ctx& C, double t, double dt, int m, int nsteps) {
     auto wgt = [&](int i) { return i <= m - 2 ? lam[i] : (i == m - 1 ? 0.0 : lam[m - 1]); };
     launch_set_clock(C.E->d_probs, C.E->nprob, t, dt, C.s);
     ++*C.launches;
+    C.prologue(PRO_HORK, m);
     int rc = C.step_loop(nsteps, EWV_METHOD_HORK, m, dt, 0, 0, 0, 1, [&](int) {
-        C.prologue(PRO_HORK, m);
         if (m == 1) {
             StageArgs s1 = stage_defaults();
             s1.x = 0;
@@ -1025,7 +1031,7 @@ int run_hork(Ctx& C, double t, double dt, int m, int nsteps) {
             s1.cay = lam[0];
             C.stage(s1);
             C.copy(1, 0, ALL_FIELDS, false);
-            C.record();
+            C.record_next(0, PRO_HORK, m);
             return;
         }
         for (int i = 1; i <= m; ++i) {
@@ -1057,7 +1063,7 @@ int run_hork(Ctx& C, double t, double dt, int m, int nsteps) {
             }
             C.stage(si);
         }
-        C.record();
+        C.record_next(0, PRO_HORK, m);
     });
     if (rc != EWV_OK) return rc;
     return check_launch(err);
@@ -1066,9 +1072,10 @@ int run_hork(Ctx& C, double t, double dt, int m, int nsteps) {
 int run_rk(Ctx& C, double t, double dt, int scheme, int nsteps) {
     launch_set_clock(C.E->d_probs, C.E->nprob, t, dt, C.s);
     ++*C.launches;
+    const int pro = scheme == EWV_METHOD_RK32 ? PRO_RK32 : PRO_RK44, stages = scheme == EWV_METHOD_RK32 ? 3 : 4;
+    C.prologue(pro, stages);
     int rc = C.step_loop(nsteps, scheme, 0, dt, 0, 0, 0, 1, [&](int) {
         if (scheme == EWV_METHOD_RK32) {
-            C.prologue(PRO_RK32, 3);
             const int xs[3] = {0, 1, 2}, ys[3] = {1, 2, 0};
             const double al[3] = {0.5 * dt, 0.5 * dt, dt};
             for (int q = 0; q < 3; ++q) {
@@ -1083,7 +1090,6 @@ int run_rk(Ctx& C, double t, double dt, int scheme, int nsteps) {
                 C.stage(a);
             }
         } else {
-            C.prologue(PRO_RK44, 4);
             StageArgs a = stage_defaults();
             a.x = 0; a.u = 0; a.y_out = 1; a.acc_out = 3; a.src_slot = 0;
             a.ch = 1.0; a.cu = 1.0; a.ck = 0.5 * dt; a.cau = 1.0; a.cak = dt / 6.0;
@@ -1101,7 +1107,7 @@ int run_rk(Ctx& C, double t, double dt, int scheme, int nsteps) {
             a.ch = 1.0; a.ca = 1.0; a.cak = dt / 6.0;
             C.stage(a);
         }
-        C.record();
+        C.record_next(0, pro, stages);
     });
     if (rc != EWV_OK) return rc;
     return check_launch(*C.err);
@@ -1199,8 +1205,8 @@ int run_krylov(Ctx& C, double t, double dt, int m, int nsteps, int* info) {
                                      0.66999052179242813, 0.93056815579702629};
     const long long vel = C.E->nprob > 0 ? (long long)C.E->models[0]->vec_elems : 0;
     const int key_method = dense ? -EWV_METHOD_KRYLOV : EWV_METHOD_KRYLOV;
+    C.prologue(PRO_KRYLOV, m);
     int rc0 = C.step_loop(nsteps, key_method, m, dt, tol, (double)window, 0, 1, [&](int) {
-        C.prologue(PRO_KRYLOV, m);
         PointArgs pn{};
         pn.mode = 0;
         pn.m = m;
@@ -1270,7 +1276,7 @@ int run_krylov(Ctx& C, double t, double dt, int m, int nsteps, int* info) {
             pc.m = m;
             C.point(pc);
         }
-        C.record();
+        C.record_next(0, PRO_KRYLOV, m);
     });
     if (rc0 != EWV_OK) return rc0;
     if (!expm_ok) return fail(err, EWV_ERR_CUDA, "expm shared-memory configuration failed");
@@ -1632,9 +1638,9 @@ int run_leapfrog(Ctx& C, std::vector<ewv_model*>& models, double t, double dt, i
     launch_set_clock(C.E->d_probs, C.E->nprob, t, dt, C.s);
     ++*C.launches;
     // step n reads level n from vector (n even ? 0 : 1) and writes level n+1 over the other
+    C.prologue(PRO_LEAPFROG, 1);
     int rc = C.step_loop(nsteps, EWV_METHOD_LEAPFROG, variant, dt, 0, 0, 0, 2, [&](int n) {
         const int cur = (n & 1) ? 1 : 0, prev = 1 - cur;
-        C.prologue(PRO_LEAPFROG, 1);
         C.timed([&] {
         if (C.E->dims == 3 && C.E->precision == EWV_F32 && C.E->tma_variant != 1) {
             if (launch_leapfrog_tma3d(C.E->R, tma3d_warps(C.E), C.E->d_probs, C.E->d_tbase, C.E->nprob,
@@ -1653,7 +1659,7 @@ int run_leapfrog(Ctx& C, std::vector<ewv_model*>& models, double t, double dt, i
             launch_leapfrog(C.E->R, C.E->ntiles, C.E->d_probs, C.E->d_tile_prob, cur, prev, variant, dt, C.s);
         }
         });
-        C.record(prev);
+        C.record_next(prev, PRO_LEAPFROG, 1);
     });
     if (rc != EWV_OK) return rc;
     // level n back into the state, n-1 into history (and d^n with it in the difference form)

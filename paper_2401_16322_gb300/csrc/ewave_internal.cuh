@@ -229,6 +229,9 @@ void launch_reset_cursor(const ProblemDev* probs, int nprob, cudaStream_t s);
 void launch_prologue(const ProblemDev* probs, int nprob, int kind, int m, double gamma,
                      double c0, double c1, cudaStream_t s);
 void launch_record(int precision, const ProblemDev* probs, int nprob, int vec, cudaStream_t s);
+// launch_record, then the prologue of the step that follows, in one launch.
+void launch_record_next(int precision, const ProblemDev* probs, int nprob, int vec, int kind, int m, double gamma,
+                        double c0, double c1, cudaStream_t s);
 void launch_point(int precision, int nblocks, const ProblemDev* probs, const int* tile_prob,
                   const PointArgs& pa, cudaStream_t s);
 // Flat pointwise passes (modes 0, 1, 2 of PointArgs) over whole padded vectors, PCHUNK

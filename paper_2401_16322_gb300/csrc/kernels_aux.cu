@@ -43,8 +43,8 @@ __device__ __forceinline__ double ricker(double t, double f, double t0) {
 enum { PRO_FABER = 1, PRO_KRYLOV = 2, PRO_HORK = 3, PRO_RK32 = 4, PRO_RK44 = 5, PRO_LEAPFROG = 6,
        PRO_HORK_HORNER = 7 };
 
-// One warp per problem.  Fills sigma[] (the value added at the source node's v entry in
-// each pass of this step) from t_n = t_start + step * dt:
+// Source scalars of one step: fills sigma[] (the value added at the source node's v entry in
+// each pass) from t_n:
 //   Faber: sigma_j = W . y_j, y_0 = e_p, y_1 = F1 y_0, y_2 = F1 y_1 - 2 c1 y_0,
 //          y_j = F1 y_{j-1} - c1 y_{j-2}, F1 = (J/dt)/gamma - c0 (tail of Eq. matrix_ampli)
 //   HORK:  sigma_i = W . (I + J)^i e_p
@@ -52,134 +52,157 @@ enum { PRO_FABER = 1, PRO_KRYLOV = 2, PRO_HORK = 3, PRO_RK32 = 4, PRO_RK44 = 5, 
 //          y_{m+1} = e_p, y_j = e_p + (1/j) J y_{j+1}
 //   RK3-2 / RK4-4 / leap-frog: f at the stage times
 //   Krylov: W stored for the Arnoldi passes
-// W[p-1-k] = dt^k r^(k)(t_n) amp / dx^2 (tail scaled by dt).  Lane q holds tail entry q;
-// the shift J (J y)_q = y_{q+1} is a warp shuffle, each W . y a warp reduction.
-__device__ __forceinline__ double warp_sum(double v) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
+// W[p-1-k] = dt^k r^(k)(t_n) amp / dx^2 (tail scaled by dt).  Warp 0 of the problem's block runs
+// the recurrences (lane q holds tail entry q; the shift J is a warp shuffle) and leaves every y
+// in shared memory; then one thread per pass forms its W . y.  The chain of one recurrence step
+// is a shuffle and one FP64 fma: divisions and the products W . y, each a chain of its own, are
+// kept out of it (a launch took 34 us for Horner HORK 20 and 83 us for Faber 60; with the record
+// of the step before it in the same launch, Horner 20 on one 601 x 301 shot went from 159 to 131
+// us a step).
+constexpr int PRO_THREADS = 256;
+constexpr int PRO_LD = MAX_P + 1;       // row length of the shared tails (odd: no bank conflicts)
 
-__global__ void prologue_kernel(const ProblemDev* probs, int nprob, int kind, int m,
-                                double gamma, double c0, double c1) {
-    const int pid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int q = threadIdx.x & 31;
-    if (pid >= nprob) return;           // whole warps exit together
-    const ProblemDev* P = probs + pid;
-    const double dt = P->tclk[1];
-    const double tn = P->tclk[0] + (double)P->clk[0] * dt;
+__device__ __forceinline__ void source_scalars(const ProblemDev* P, double tn, double dt, int kind, int m,
+                                               double gamma, double c0, double c1, double* sy, double* sw,
+                                               double* sr) {
+    const int tid = threadIdx.x, q = tid & 31;
     double* sg = P->sigma;
     if (!P->has_src) {
-        for (int s = q; s < MAX_SIGMA; s += 32) sg[s] = 0.0;
-        if (kind == PRO_KRYLOV && q < MAX_P) P->kry[KRY_W + q] = 0.0;
+        for (int s = tid; s < MAX_SIGMA; s += PRO_THREADS) sg[s] = 0.0;
+        if (kind == PRO_KRYLOV && tid < MAX_P) P->kry[KRY_W + tid] = 0.0;
         return;
     }
     const double scale = P->amp * P->inv_dx2;
     if (kind == PRO_RK32 || kind == PRO_RK44 || kind == PRO_LEAPFROG) {
-        if (q == 0) {
-            if (kind == PRO_LEAPFROG) {
-                sg[0] = scale * ricker(tn, P->f_peak, P->t0);
-            } else {
-                sg[0] = scale * ricker(tn, P->f_peak, P->t0);
-                sg[1] = sg[2] = scale * ricker(tn + 0.5 * dt, P->f_peak, P->t0);
-                if (kind == PRO_RK44) sg[3] = scale * ricker(tn + dt, P->f_peak, P->t0);
-            }
-        }
+        // thread 0: f(t_n); 1 and 2: f(t_n + dt/2); 3: f(t_n + dt)
+        const int n = kind == PRO_LEAPFROG ? 1 : kind == PRO_RK32 ? 3 : 4;
+        if (tid < n) sg[tid] = scale * ricker(tn + (tid == 0 ? 0.0 : tid == 3 ? 1.0 : 0.5) * dt, P->f_peak, P->t0);
         return;
     }
     const int p = P->p;
-    // W_q = dt^k r^(k)(t_n) scale with k = p-1-q: every lane runs the Hermite recurrence
-    // g^(k) = -2 a tau g^(k-1) - 2 a (k-1) g^(k-2) and keeps its own term.
-    const int kq = p - 1 - q;
-    const double a = (M_PI * P->f_peak) * (M_PI * P->f_peak);
-    const double tau = tn - P->t0;
-    double gm2 = exp(-a * tau * tau), gm1 = -2.0 * a * tau * gm2, rk = 0.0, dk = 1.0;
-    for (int k = 2; k < p + 2; ++k) {
-        const double g = -2.0 * a * tau * gm1 - 2.0 * a * (double)(k - 1) * gm2;
-        if (k - 2 == kq) rk = -g / (2.0 * a);
-        gm2 = gm1;
-        gm1 = g;
-    }
-    for (int k = 0; k < kq && kq >= 0; ++k) dk *= dt;
-    const double W = (q < p) ? dk * rk * scale : 0.0;
-    if (kind == PRO_KRYLOV) {
-        if (q < MAX_P) P->kry[KRY_W + q] = W;
-        return;
-    }
-    double y0 = (q == p - 1) ? 1.0 : 0.0;
-    if (kind == PRO_HORK_HORNER) {
-        double y = y0;
-        for (int k = 0; k < m && k < MAX_SIGMA; ++k) {
-            const double s = warp_sum(W * y);
-            if (q == 0) sg[k] = s;
-            double up = __shfl_down_sync(0xffffffffu, y, 1);
-            if (q + 1 >= p) up = 0.0;
-            y = ((q == p - 1) ? 1.0 : 0.0) + up / (double)(m - k);
+    const int rows = m < MAX_SIGMA ? m : MAX_SIGMA;
+    if (kind == PRO_HORK_HORNER)
+        for (int k = tid; k < rows; k += PRO_THREADS) sr[k] = 1.0 / (double)(m - k);
+    __syncthreads();
+    if (tid < 32) {
+        // W_q = dt^k r^(k)(t_n) scale with k = p-1-q: every lane runs the Hermite recurrence
+        // g^(k) = -2 a tau g^(k-1) - 2 a (k-1) g^(k-2) and keeps its own term
+        const int kq = p - 1 - q;
+        const double a = (M_PI * P->f_peak) * (M_PI * P->f_peak);
+        const double tau = tn - P->t0;
+        double gm2 = exp(-a * tau * tau), gm1 = -2.0 * a * tau * gm2, gk = 0.0, dk = 1.0, pw = 1.0;
+        for (int k = 2; k < p + 2; ++k) {
+            const double g = -2.0 * a * tau * gm1 - 2.0 * a * (double)(k - 1) * gm2;
+            if (k - 2 == kq) {
+                gk = g;
+                dk = pw;
+            }
+            pw *= dt;
+            gm2 = gm1;
+            gm1 = g;
         }
-        return;
-    }
-    if (kind == PRO_HORK) {
-        // y_i = (I + J) y_{i-1}
-        for (int i = 0; i < m && i < MAX_SIGMA; ++i) {
-            const double s = warp_sum(W * y0);
-            if (q == 0) sg[i] = s;
-            double up = __shfl_down_sync(0xffffffffu, y0, 1);
-            if (q + 1 >= p) up = 0.0;
-            y0 = y0 + up;
+        const double W = (q < p) ? dk * (-gk / (2.0 * a)) * scale : 0.0;
+        if (kind == PRO_KRYLOV) {
+            if (q < MAX_P) P->kry[KRY_W + q] = W;
+        } else {
+            if (q < MAX_P) sw[q] = W;
+            const bool up_in = q + 1 < p;
+            const double e = (q == p - 1) ? 1.0 : 0.0;
+            auto shift = [&](double y) {           // J y
+                const double u = __shfl_down_sync(0xffffffffu, y, 1);
+                return up_in ? u : 0.0;
+            };
+            double y = e;
+            if (kind == PRO_FABER) {
+                const double ig = 1.0 / gamma / dt;
+                double ym = 0.0;
+                for (int j = 0; j < rows; ++j) {
+                    if (q < p) sy[j * PRO_LD + q] = y;
+                    const double cj = (j == 1) ? 2.0 * c1 : c1;       // (y_{-1} = 0)
+                    const double t = -c0 * y - cj * ym;
+                    ym = y;
+                    y = fma(ig, shift(y), t);
+                }
+            } else if (kind == PRO_HORK_HORNER) {
+                for (int k = 0; k < rows; ++k) {
+                    if (q < p) sy[k * PRO_LD + q] = y;
+                    y = fma(shift(y), sr[k], e);
+                }
+            } else {
+                for (int i = 0; i < rows; ++i) {                       // y_i = (I + J) y_{i-1}
+                    if (q < p) sy[i * PRO_LD + q] = y;
+                    y = y + shift(y);
+                }
+            }
         }
-        return;
     }
-    // Faber
-    const double ig = 1.0 / gamma;
-    auto F1 = [&](double y) {
-        double up = __shfl_down_sync(0xffffffffu, y, 1);
-        if (q + 1 >= p) up = 0.0;
-        return ig * up / dt - c0 * y;
-    };
-    double s0 = warp_sum(W * y0);
-    if (q == 0) sg[0] = s0;
-    double y1 = F1(y0);
-    if (m >= 2) {
-        const double s1 = warp_sum(W * y1);
-        if (q == 0) sg[1] = s1;
-    }
-    for (int j = 2; j < m && j < MAX_SIGMA; ++j) {
-        const double cj = (j == 2) ? 2.0 * c1 : c1;
-        const double y2 = F1(y1) - cj * y0;
-        const double sj = warp_sum(W * y2);
-        if (q == 0) sg[j] = sj;
-        y0 = y1;
-        y1 = y2;
+    __syncthreads();
+    if (kind == PRO_KRYLOV) return;
+    for (int k = tid; k < rows; k += PRO_THREADS) {
+        double s0 = 0.0, s1 = 0.0;
+        for (int e = 0; e < p; e += 2) {
+            s0 = fma(sw[e], sy[k * PRO_LD + e], s0);
+            if (e + 1 < p) s1 = fma(sw[e + 1], sy[k * PRO_LD + e + 1], s1);
+        }
+        sg[k] = s0 + s1;
     }
 }
 
-// ---------------------------------------------------------------- recording
+// ---------------------------------------------------------------- between two steps
+// One block per problem: records sample clk[1] from vector `vec` (record), advances the clock
+// and prepares the source scalars of the step that follows (kind >= 0); or, before the first
+// step of a call, only the latter.  One launch between two steps instead of two: at the sizes
+// where a pass takes a few microseconds every launch counts.
 template <typename T>
-__global__ void record_kernel(const ProblemDev* probs, int nprob, int vec) {
+__global__ void __launch_bounds__(PRO_THREADS)
+between_kernel(const ProblemDev* probs, int nprob, int record, int vec, int kind, int m, double gamma, double c0,
+               double c1) {
+    __shared__ double sy[MAX_SIGMA * PRO_LD];
+    __shared__ double sw[MAX_P];
+    __shared__ double sr[MAX_SIGMA];
     const ProblemDev* P = probs + blockIdx.x;
-    const long long cur = P->clk[1];
-    if (P->seismo && cur < P->capacity) {
-        const T* u = vptr<T>(P, vec);
-        T* out = (T*)P->seismo + cur * P->rec_stride;
-        for (int r = threadIdx.x; r < P->nrec; r += blockDim.x) out[r] = u[P->rec_off[r]];
+    const long long step = P->clk[0] + (record ? 1 : 0);
+    const double dt = P->tclk[1];
+    const double tn = P->tclk[0] + (double)step * dt;
+    if (record) {
+        const long long cur = P->clk[1];
+        if (P->seismo && cur < P->capacity) {
+            const T* u = vptr<T>(P, vec);
+            T* out = (T*)P->seismo + cur * P->rec_stride;
+            // (from the last warp down: the first one has the recurrences to run)
+            for (int r = PRO_THREADS - 1 - (int)threadIdx.x; r < P->nrec; r += PRO_THREADS) out[r] = u[P->rec_off[r]];
+        }
+        __syncthreads();          // every thread has read the clock
+        if (threadIdx.x == 0) {
+            P->clk[1] = cur + 1;
+            P->clk[0] = step;
+        }
     }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        P->clk[1] = cur + 1;
-        P->clk[0] += 1;
-    }
+    if (kind >= 0) source_scalars(P, tn, dt, kind, m, gamma, c0, c1, sy, sw, sr);
 }
 
 // ---------------------------------------------------------------- adjoint source
-// lambda_u[rec] += values[shot][rec] (the transpose of recording, R^T r); one thread per
-// shot adds its receivers in order, so coincident receivers are summed deterministically.
+// lambda_u[rec] += values[shot][rec] (the transpose of recording, R^T r); one block per shot, one
+// thread per receiver.  Of coincident receivers the first adds all their values in order, so the
+// sums are deterministic (62 us with one thread per shot adding 200 receivers one after another).
 template <typename T>
 __global__ void inject_kernel(T* adj, long long vec_elems, const T* values, const int* rec_off,
-                              const int* nrec, int nshots, int max_rec) {
-    const int sh = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sh >= nshots) return;
+                              const int* nrec, int max_rec) {
+    const int sh = blockIdx.x;
     T* lam = adj + (long long)sh * vec_elems;
+    const int* off = rec_off + (long long)sh * max_rec;
+    const T* val = values + (long long)sh * max_rec;
     const int n = nrec[sh];
-    for (int r = 0; r < n; ++r) lam[rec_off[sh * max_rec + r]] += values[(long long)sh * max_rec + r];
+    for (int r = threadIdx.x; r < n; r += blockDim.x) {
+        const int o = off[r];
+        bool first = true;
+        for (int e = 0; e < r && first; ++e) first = off[e] != o;
+        if (!first) continue;
+        T v = lam[o] + val[r];
+        for (int e = r + 1; e < n; ++e)
+            if (off[e] == o) v += val[e];
+        lam[o] = v;
+    }
 }
 
 // out[o] = sum_s in[s][o], shots summed in index order (deterministic).
@@ -361,10 +384,21 @@ point_flat_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
         __syncthreads();
         V* St = pa.out ? reinterpret_cast<V*>(static_cast<T*>(pa.out) + (long long)pid * pa.out_stride)
                        : reinterpret_cast<V*>(vptr<T>(P, pa.dst));
-        for (long long q = q0 + tid; q < q1; q += NTHREADS) {
-            V acc = {};
-            for (int k = 1; k <= meff; ++k) fma16(acc, s_coef[k - 1], reinterpret_cast<const V*>(vptr<T>(P, k - 1))[q]);
-            St[q] = acc;
+        // eight vectors a thread at a time: eight loads in flight for every basis vector
+        constexpr int G = 8;
+        for (long long q = q0 + tid; q < q1; q += G * NTHREADS) {
+            V acc[G];
+#pragma unroll
+            for (int g = 0; g < G; ++g) acc[g] = V{};
+            for (int k = 1; k <= meff; ++k) {
+                const V* B = reinterpret_cast<const V*>(vptr<T>(P, k - 1));
+#pragma unroll
+                for (int g = 0; g < G; ++g)
+                    if (q + g * NTHREADS < q1) fma16(acc[g], s_coef[k - 1], B[q + g * NTHREADS]);
+            }
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                if (q + g * NTHREADS < q1) St[q + g * NTHREADS] = acc[g];
         }
         return;
     }
@@ -422,7 +456,7 @@ point_flat_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
 // output equals the single combine with the same coefficients bit for bit).  A kernel of its
 // own keeps the accumulators out of the flat passes' register budget.
 template <typename T>
-__global__ void __launch_bounds__(NTHREADS)
+__global__ void __launch_bounds__(NTHREADS, 2)
 combine_multi_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ pbase, int nprob, PointArgs pa) {
     using V = typename Vec16<T>::type;
     constexpr int NV = Vec16<T>::N;
@@ -457,42 +491,80 @@ combine_multi_kernel(const ProblemDev* __restrict__ probs, const int* __restrict
         else if (q == pa.nout && pa.final_out)
             outs[q] = reinterpret_cast<V*>(vptr<T>(P, 0));
     }
-    for (long long i = q0 + tid; i < q1; i += NTHREADS) {
-        V acc[MAX_TAU];
+    // four vectors a thread at a time (230 us one at a time, 16 shots of 401 x 201, 20 vectors)
+    constexpr int G = 4;
+    for (long long i = q0 + tid; i < q1; i += G * NTHREADS) {
+        V acc[G][MAX_TAU];
 #pragma unroll
-        for (int q = 0; q < MAX_TAU; ++q) acc[q] = V{};
+        for (int g = 0; g < G; ++g)
+#pragma unroll
+            for (int q = 0; q < MAX_TAU; ++q) acc[g][q] = V{};
         for (int k = 1; k <= meff; ++k) {
-            const V v = reinterpret_cast<const V*>(vptr<T>(P, k - 1))[i];
+            const V* B = reinterpret_cast<const V*>(vptr<T>(P, k - 1)) + i;
+            V v[G];
 #pragma unroll
-            for (int q = 0; q < MAX_TAU; ++q)
-                if (q < nt) fma16(acc[q], s_mc[q][k - 1], v);
+            for (int g = 0; g < G; ++g) v[g] = i + g * NTHREADS < q1 ? B[g * NTHREADS] : V{};
+#pragma unroll
+            for (int q = 0; q < MAX_TAU; ++q) {
+                if (q >= nt) break;
+                const T c = s_mc[q][k - 1];
+#pragma unroll
+                for (int g = 0; g < G; ++g) fma16(acc[g][q], c, v[g]);
+            }
         }
 #pragma unroll
-        for (int q = 0; q < MAX_TAU; ++q)
-            if (q < nt) outs[q][i] = acc[q];
+        for (int q = 0; q < MAX_TAU; ++q) {
+            if (q >= nt) break;
+#pragma unroll
+            for (int g = 0; g < G; ++g)
+                if (i + g * NTHREADS < q1) outs[q][i + g * NTHREADS] = acc[g][q];
+        }
     }
 }
 
 // ---------------------------------------------------------------- Hessenberg exponential
 // [13/13] Pade approximant with scaling and squaring (Higham 2005), FP64, one block per
-// problem; writes exp(H_meff) e_1 to kry[KRY_E..].  Shared memory: 7 matrices of meff^2.
+// problem; writes exp(H_meff) e_1 to kry[KRY_E..].  Shared memory: 8 matrices of meff^2.
+// One SM works alone here, at 16 cycles an FP64 warp instruction: scalar work (norm, scaling, pivot
+// search, the pivot's reciprocal) is done by one warp and not by all of them, the coefficients are
+// constants, products run in four interleaved sums, and Gauss-Jordan elimination takes the
+// place of the serial back substitution.
+struct PadeCoefs {
+    double b[14];      // b_k = (26-k)! 13! / (26! k! (13-k)!)
+    constexpr PadeCoefs() : b{} {
+        double f[27] = {1.0};
+        for (int i = 1; i <= 26; ++i) f[i] = f[i - 1] * (double)i;
+        for (int k = 0; k <= 13; ++k) b[k] = f[26 - k] * f[13] / (f[26] * f[k] * f[13 - k]);
+    }
+};
+constexpr int EXPM_THREADS = 512;
+
+// sum_k a[k as] b[k bs], k < n
+__device__ __forceinline__ double dot_strided(const double* a, int as, const double* b, int bs, int n) {
+    double s[4] = {0.0, 0.0, 0.0, 0.0};
+    int k = 0;
+    for (; k + 3 < n; k += 4)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) s[q] = fma(a[(k + q) * as], b[(k + q) * bs], s[q]);
+    for (; k < n; ++k) s[0] = fma(a[k * as], b[k * bs], s[0]);
+    return (s[0] + s[1]) + (s[2] + s[3]);
+}
 __device__ void mat_mul(const double* A, const double* B, double* C, int n) {
     for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
         const int r = e / n, c = e - r * n;
-        double s = 0.0;
-        for (int k = 0; k < n; ++k) s = fma(A[r * n + k], B[k * n + c], s);
-        C[e] = s;
+        C[e] = dot_strided(A + r * n, 1, B + c, n, n);
     }
     __syncthreads();
 }
 
 // Block (p, q) writes exp(tau_q H_meff) e_1 of problem p to kry[KRY_E..] (et.out null, one
 // tau) or to et.out[(p ntau + q) MAX_M ..] (several taus in one launch).
-__global__ void expm_kernel(const ProblemDev* probs, int nprob, ExpmTaus et) {
+__global__ void __launch_bounds__(EXPM_THREADS) expm_kernel(const ProblemDev* probs, int nprob, ExpmTaus et) {
     extern __shared__ double sm[];
-    __shared__ double b[14];
-    __shared__ double colmax[MAX_M];
-    __shared__ int s_scale, s_piv;
+    __shared__ double colsum[MAX_M];
+    __shared__ int s_piv, s_scale;
+    __shared__ double s_fac, s_inv;
+    constexpr PadeCoefs pade;
     const ProblemDev* P = probs + blockIdx.x;
     double* kry = P->kry;
     const double hscale = et.tau[blockIdx.y];
@@ -507,128 +579,133 @@ __global__ void expm_kernel(const ProblemDev* probs, int nprob, ExpmTaus et) {
     double* Um = A6 + nn;
     double* Vm = Um + nn;
     double* Tm = Vm + nn;
+    double* Wm = Tm + nn;
     const int tid = threadIdx.x;
-    if (tid == 0) {
-        // b_k = (26-k)! 13! / (26! k! (13-k)!)
-        double f[27];
-        f[0] = 1.0;
-        for (int i = 1; i <= 26; ++i) f[i] = f[i - 1] * (double)i;
-        for (int k = 0; k <= 13; ++k) b[k] = f[26 - k] * f[13] / (f[26] * f[k] * f[13 - k]);
-    }
     for (int e = tid; e < nn; e += blockDim.x) {
         const int r = e / n, c = e - r * n;
         A[e] = hscale * kry[KRY_H + r * MAX_M + c];   // exp(tau H_m): dense output at tau
     }
     __syncthreads();
-    for (int c = tid; c < n; c += blockDim.x) {
-        double s = 0.0;
-        for (int r = 0; r < n; ++r) s += fabs(A[r * n + c]);
-        colmax[c] = s;
+    if (tid < n) {
+        double s0 = 0.0, s1 = 0.0;
+        int r = 0;
+        for (; r + 1 < n; r += 2) {
+            s0 += fabs(A[r * n + tid]);
+            s1 += fabs(A[(r + 1) * n + tid]);
+        }
+        if (r < n) s0 += fabs(A[r * n + tid]);
+        colsum[tid] = s0 + s1;
     }
     __syncthreads();
-    if (tid == 0) {
-        double nrm = 0.0;
-        for (int c = 0; c < n; ++c) nrm = fmax(nrm, colmax[c]);
-        const double theta13 = 5.371920351148152;
-        int s = 0;
-        if (nrm > theta13) s = (int)ceil(log2(nrm / theta13));
-        s_scale = s;
+    if (tid < 32) {
+        double nrm = fmax(tid < n ? colsum[tid] : 0.0, tid + 32 < n ? colsum[tid + 32] : 0.0);
+        for (int o = 16; o > 0; o >>= 1) nrm = fmax(nrm, __shfl_xor_sync(0xffffffffu, nrm, o));
+        // s = max(0, ceil(log2(norm / theta_13)))
+        int sq = 0;
+        for (double v = nrm; v > 5.371920351148152 && sq < 1000; v *= 0.5) ++sq;
+        if (tid == 0) {
+            s_scale = sq;
+            s_fac = ldexp(1.0, -sq);
+        }
     }
     __syncthreads();
     const int s = s_scale;
-    const double sc = ldexp(1.0, -s);
-    for (int e = tid; e < nn; e += blockDim.x) A[e] *= sc;
+    for (int e = tid; e < nn; e += blockDim.x) A[e] *= s_fac;
     __syncthreads();
     mat_mul(A, A, A2, n);
     mat_mul(A2, A2, A4, n);
     mat_mul(A4, A2, A6, n);
-    for (int e = tid; e < nn; e += blockDim.x) Tm[e] = b[13] * A6[e] + b[11] * A4[e] + b[9] * A2[e];
-    __syncthreads();
-    mat_mul(A6, Tm, Um, n);   // Um = A6 (b13 A6 + b11 A4 + b9 A2)
     for (int e = tid; e < nn; e += blockDim.x) {
-        const int r = e / n, c = e - r * n;
-        Tm[e] = Um[e] + b[7] * A6[e] + b[5] * A4[e] + b[3] * A2[e] + (r == c ? b[1] : 0.0);
+        Tm[e] = pade.b[13] * A6[e] + pade.b[11] * A4[e] + pade.b[9] * A2[e];
+        Vm[e] = pade.b[12] * A6[e] + pade.b[10] * A4[e] + pade.b[8] * A2[e];
     }
     __syncthreads();
-    mat_mul(A, Tm, Um, n);    // U = A (...)
-    for (int e = tid; e < nn; e += blockDim.x) Tm[e] = b[12] * A6[e] + b[10] * A4[e] + b[8] * A2[e];
-    __syncthreads();
-    mat_mul(A6, Tm, Vm, n);
-    for (int e = tid; e < nn; e += blockDim.x) {
-        const int r = e / n, c = e - r * n;
-        Vm[e] += b[6] * A6[e] + b[4] * A4[e] + b[2] * A2[e] + (r == c ? b[0] : 0.0);
+    // odd part U = A (A6 (b13 A6 + b11 A4 + b9 A2) + b7 A6 + b5 A4 + b3 A2 + b1 I), even part V alike
+    for (int e = tid; e < 2 * nn; e += blockDim.x) {
+        const bool odd = e < nn;
+        const int f = odd ? e : e - nn;
+        const int r = f / n, c = f - r * n;
+        const double v = dot_strided(A6 + r * n, 1, (odd ? Tm : Vm) + c, n, n);
+        const double a2 = A2[f], a4 = A4[f], a6 = A6[f];
+        if (odd) Um[f] = v + pade.b[7] * a6 + pade.b[5] * a4 + pade.b[3] * a2 + (r == c ? pade.b[1] : 0.0);
+        else Wm[f] = v + pade.b[6] * a6 + pade.b[4] * a4 + pade.b[2] * a2 + (r == c ? pade.b[0] : 0.0);
     }
     __syncthreads();
-    // Solve (V - U) Rm = (V + U): LU with partial pivoting; P_ in A, RHS in A2.
-    double* Pm = A;
-    double* Q = A2;
+    mat_mul(A, Um, Tm, n);
+    // Solve (V - U) X = (V + U): Gauss-Jordan elimination with partial pivoting; P in A2, X in A4.
+    double* Pm = A2;
+    double* Q = A4;
+    double* mult = A6;        // multipliers of the current column
     for (int e = tid; e < nn; e += blockDim.x) {
-        Pm[e] = Vm[e] - Um[e];
-        Q[e] = Vm[e] + Um[e];
+        Pm[e] = Wm[e] - Tm[e];
+        Q[e] = Wm[e] + Tm[e];
     }
     __syncthreads();
     for (int c = 0; c < n; ++c) {
-        if (tid == 0) {
+        if (tid < 32) {
+            double best = -1.0;
             int piv = c;
-            double best = fabs(Pm[c * n + c]);
-            for (int r = c + 1; r < n; ++r)
-                if (fabs(Pm[r * n + c]) > best) {
-                    best = fabs(Pm[r * n + c]);
+            for (int r = c + tid; r < n; r += 32) {
+                const double v = fabs(Pm[r * n + c]);
+                if (v > best) {
+                    best = v;
                     piv = r;
                 }
-            s_piv = piv;
+            }
+            for (int o = 16; o > 0; o >>= 1) {
+                const double ob = __shfl_xor_sync(0xffffffffu, best, o);
+                const int op = __shfl_xor_sync(0xffffffffu, piv, o);
+                if (ob > best || (ob == best && op < piv)) {
+                    best = ob;
+                    piv = op;
+                }
+            }
+            if (tid == 0) {
+                s_piv = piv;
+                s_inv = 1.0 / Pm[piv * n + c];
+            }
         }
         __syncthreads();
         const int piv = s_piv;
-        if (piv != c) {
-            for (int e = tid; e < n; e += blockDim.x) {
-                double t = Pm[c * n + e];
-                Pm[c * n + e] = Pm[piv * n + e];
-                Pm[piv * n + e] = t;
-                t = Q[c * n + e];
-                Q[c * n + e] = Q[piv * n + e];
-                Q[piv * n + e] = t;
-            }
+        const double inv = s_inv;
+        // multipliers (row piv will hold what row c holds now), then the pivot row scaled into row c
+        for (int r = tid; r < n; r += blockDim.x) mult[r] = r == c ? 0.0 : Pm[(r == piv ? c : r) * n + c];
+        double keep_c = 0.0, keep_p = 0.0;
+        const bool in_p = tid > c && tid < n, in_q = tid >= n && tid < 2 * n;
+        double* M = in_p ? Pm + tid : Q + (tid - n);
+        if (in_p || in_q) {
+            keep_c = M[c * n];
+            keep_p = M[piv * n];
         }
         __syncthreads();
-        const double d = Pm[c * n + c];
-        // eliminate rows below
-        for (int e = tid; e < (n - c - 1) * n; e += blockDim.x) {
-            const int r = c + 1 + e / n, col = e % n;
-            const double l = Pm[r * n + c] / d;
-            if (col > c) Pm[r * n + col] -= l * Pm[c * n + col];
-            Q[r * n + col] -= l * Q[c * n + col];
+        if (in_p || in_q) {
+            if (piv != c) M[piv * n] = keep_c;
+            M[c * n] = keep_p * inv;
         }
         __syncthreads();
-        for (int r = c + 1 + tid; r < n; r += blockDim.x) Pm[r * n + c] = 0.0;
+        const int wp = n - c - 1, w = wp + n;      // columns c + 1 .. n - 1 of P, then all of X
+        for (int e = tid; e < n * w; e += blockDim.x) {
+            const int r = e / w, k = e - r * w;
+            if (r == c) continue;
+            double* T = k < wp ? Pm + c + 1 + k : Q + (k - wp);
+            T[r * n] = fma(-mult[r], T[c * n], T[r * n]);
+        }
         __syncthreads();
     }
-    // back substitution, column-parallel over the RHS
-    for (int col = tid; col < n; col += blockDim.x) {
-        for (int r = n - 1; r >= 0; --r) {
-            double v = Q[r * n + col];
-            for (int k = r + 1; k < n; ++k) v -= Pm[r * n + k] * Q[k * n + col];
-            Q[r * n + col] = v / Pm[r * n + r];
-        }
-    }
-    __syncthreads();
-    // Rm = Q.  Undo the scaling: Rm^(2^s) e_1 by squarings or repeated products.
+    // X^(2^s) e_1 by products with e_1 or by squarings, whichever is less work
     double* Rm = Q;
-    const long long nmv = 1LL << s;
-    if ((double)nmv <= (double)s * n) {
-        double* x = A4;
-        double* y = A6;
+    const long long nmv = s < 40 ? 1LL << s : 1LL << 40;
+    if ((double)nmv <= (double)s * n || s == 0) {
+        double* x = Um;
+        double* y = Wm;
         for (int r = tid; r < n; r += blockDim.x) x[r] = (r == 0) ? 1.0 : 0.0;
         __syncthreads();
         for (long long it = 0; it < nmv; ++it) {
-            for (int r = tid; r < n; r += blockDim.x) {
-                double v = 0.0;
-                for (int k = 0; k < n; ++k) v = fma(Rm[r * n + k], x[k], v);
-                y[r] = v;
-            }
+            for (int r = tid; r < n; r += blockDim.x) y[r] = dot_strided(Rm + r * n, 1, x, 1, n);
             __syncthreads();
-            for (int r = tid; r < n; r += blockDim.x) x[r] = y[r];
-            __syncthreads();
+            double* t = x;
+            x = y;
+            y = t;
         }
         for (int r = tid; r < n; r += blockDim.x) eo[r] = x[r];
     } else {
@@ -678,23 +755,31 @@ void launch_set_clock(const ProblemDev* probs, int nprob, double t, double dt, c
 void launch_reset_cursor(const ProblemDev* probs, int nprob, cudaStream_t s) {
     reset_cursor_kernel<<<(nprob + 127) / 128, 128, 0, s>>>(probs, nprob);
 }
+static void launch_between(int precision, const ProblemDev* probs, int nprob, int record, int vec, int kind, int m,
+                           double gamma, double c0, double c1, cudaStream_t s) {
+    if (precision == 0)
+        between_kernel<float><<<nprob, PRO_THREADS, 0, s>>>(probs, nprob, record, vec, kind, m, gamma, c0, c1);
+    else
+        between_kernel<double><<<nprob, PRO_THREADS, 0, s>>>(probs, nprob, record, vec, kind, m, gamma, c0, c1);
+}
 void launch_prologue(const ProblemDev* probs, int nprob, int kind, int m, double gamma,
                      double c0, double c1, cudaStream_t s) {
-    prologue_kernel<<<(nprob + 3) / 4, 128, 0, s>>>(probs, nprob, kind, m, gamma, c0, c1);
+    launch_between(0, probs, nprob, 0, 0, kind, m, gamma, c0, c1, s);
 }
 void launch_record(int precision, const ProblemDev* probs, int nprob, int vec, cudaStream_t s) {
-    if (precision == 0) record_kernel<float><<<nprob, 128, 0, s>>>(probs, nprob, vec);
-    else record_kernel<double><<<nprob, 128, 0, s>>>(probs, nprob, vec);
+    launch_between(precision, probs, nprob, 1, vec, -1, 0, 0.0, 0.0, 0.0, s);
+}
+void launch_record_next(int precision, const ProblemDev* probs, int nprob, int vec, int kind, int m, double gamma,
+                        double c0, double c1, cudaStream_t s) {
+    launch_between(precision, probs, nprob, 1, vec, kind, m, gamma, c0, c1, s);
 }
 void launch_inject(int precision, void* adj, long long vec_elems, const void* values,
                    const int* rec_off, const int* nrec, int nshots, int max_rec, cudaStream_t s) {
-    const int blocks = (nshots + 63) / 64;
     if (precision == 0)
-        inject_kernel<float><<<blocks, 64, 0, s>>>((float*)adj, vec_elems, (const float*)values, rec_off,
-                                                   nrec, nshots, max_rec);
+        inject_kernel<float><<<nshots, 256, 0, s>>>((float*)adj, vec_elems, (const float*)values, rec_off, nrec, max_rec);
     else
-        inject_kernel<double><<<blocks, 64, 0, s>>>((double*)adj, vec_elems, (const double*)values,
-                                                    rec_off, nrec, nshots, max_rec);
+        inject_kernel<double><<<nshots, 256, 0, s>>>((double*)adj, vec_elems, (const double*)values, rec_off, nrec,
+                                                     max_rec);
 }
 
 void launch_sum_shots(int precision, const void* in, void* out, long long n, int nshots,
@@ -761,13 +846,13 @@ void launch_point_flat(int precision, int nchunks, const ProblemDev* probs, cons
     else point_flat_kernel<double><<<nchunks, block, 0, s>>>(probs, pbase, nprob, pa);
 }
 static int launch_expm_taus(const ProblemDev* probs, int nprob, int mmax, cudaStream_t s, const ExpmTaus& et) {
-    const size_t smem = (size_t)7 * mmax * mmax * sizeof(double);
+    const size_t smem = (size_t)8 * mmax * mmax * sizeof(double);
     if (smem > 48 * 1024) {
         if (cudaFuncSetAttribute(expm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)smem) != cudaSuccess)
             return -1;
     }
-    expm_kernel<<<dim3(nprob, et.n), 256, smem, s>>>(probs, nprob, et);
+    expm_kernel<<<dim3(nprob, et.n), EXPM_THREADS, smem, s>>>(probs, nprob, et);
     return 0;
 }
 int launch_expm(const ProblemDev* probs, int nprob, int mmax, cudaStream_t s, double hscale) {
