@@ -696,7 +696,7 @@ struct Ctx {
             }
         } else if (E->precision == EWV_F32 && a.transpose && a.fin_mode == FIN_NONE && a.d < 0 && !a.grad &&
                    !a.store_bf16 && E->d_tbase) {
-            const int set = tma_map_set(18);
+            const int set = tma_map_set(tma_transpose_height(a.u >= 0, a.a >= 0));
             if (launch_transpose_tma(E->R, E->d_probs, E->d_tbase + (size_t)set * (E->nprob + 1), E->nprob,
                                      E->ntiles_by[set], a, E->d_err, s) != 0)
                 launch_failed = 1;
@@ -2492,7 +2492,7 @@ static int adjoint_krylov(ewv_model* m, Engine* E, double t, double dt, int mm, 
         views[2 * ns + sh] = G;
     }
     // FP32: the products of both Arnoldi processes take the persistent TMA passes (the forward
-    // one the autotuned variant, the transposed one 64 x 18 tiles); the tensor maps describe the F and A views and are rebuilt when the buffers change.  The
+    // one the autotuned variant); the tensor maps describe the F and A views and are rebuilt when the buffers change.  The
     // gradient passes take the TMA gradient pass when the caller built maps of the G view
     // (the cotangent and the workspace from vector 0).
     bool tma = prec == EWV_F32 && E->tma_variant >= 0 && E->d_tbase && E->nprob == ns &&
@@ -2537,7 +2537,7 @@ static int adjoint_krylov(ewv_model* m, Engine* E, double t, double dt, int mm, 
     static const double kW[4] = {0.17392742256872693, 0.32607257743127307,
                                  0.32607257743127307, 0.17392742256872693};
     const int fset = tma ? tma_map_set(tma_variant_tile_height_for(E->tma_variant, false)) : 0;
-    const int trset = tma_map_set(18), gset = tma_map_set(30);
+    const int trset = tma_map_set(tma_transpose_height(false, false)), gset = tma_map_set(30);
     const int rc_gs = gs_ready(E, m->err);
     if (rc_gs != EWV_OK) return rc_gs;
     auto arnoldi = [&](const ProblemDev* v, bool transpose) {
@@ -2955,7 +2955,7 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
     auto tset_of = [&](const StageArgs& sa) {
         return tma_map_set(tma_variant_tile_height_for(E->tma_variant, sa.a >= 0));
     };
-    const int gset = tma_map_set(30), trset = tma_map_set(18);
+    const int gset = tma_map_set(30);
     auto stage = [&](const StageArgs& sa) {
         if (tma_adj && !sa.transpose && sa.grad && sa.fin_mode == FIN_NONE && sa.d < 0 &&
             launch_grad_tma(R, E->d_adj, E->d_tbase + (size_t)gset * (E->nprob + 1), ns, E->ntiles_by[gset], sa,
@@ -2963,6 +2963,7 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
             ++m->launches;
             return;
         }
+        const int trset = tma_map_set(tma_transpose_height(sa.u >= 0, sa.a >= 0));
         if (tma_adj && sa.transpose && !sa.grad && sa.fin_mode == FIN_NONE && sa.d < 0 &&
             launch_transpose_tma(R, E->d_adj, E->d_tbase + (size_t)trset * (E->nprob + 1), ns, E->ntiles_by[trset],
                                  sa, E->d_err, s) == 0) {

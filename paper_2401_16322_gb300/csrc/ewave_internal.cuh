@@ -208,8 +208,9 @@ int launch_leapfrog_tma(int R, const ProblemDev* probs, const int* tbase, int np
 // tiles, the 30-row map set).
 int launch_grad_tma(int R, const ProblemDev* probs, const int* tbase, int nprob, int ntiles,
                     const StageArgs& a, int* err, cudaStream_t s);
-// The transposed pass H^T through the persistent TMA pipeline (FP32, no dot partner, no
-// gradient; 64 x 18 tiles, the 18-row map set).
+// The transposed pass H^T through the persistent TMA pipeline (FP32, no gradient); tbase and
+// ntiles are those of the map set of tma_transpose_height rows.
+int tma_transpose_height(bool reads_u, bool reads_a);
 int launch_transpose_tma(int R, const ProblemDev* probs, const int* tbase, int nprob, int ntiles,
                          const StageArgs& a, int* err, cudaStream_t s);
 int launch_stage_tma(int variant, int R, const ProblemDev* probs, const int* tbase, int nprob,

@@ -10,6 +10,7 @@
 #include "ewave_internal.cuh"
 #include "flat_vec.cuh"
 #include "krylov_finalize.cuh"
+#include "pdl.cuh"
 
 namespace ewv {
 
@@ -161,6 +162,8 @@ between_kernel(const ProblemDev* probs, int nprob, int record, int vec, int kind
     __shared__ double sw[MAX_P];
     __shared__ double sr[MAX_SIGMA];
     const ProblemDev* P = probs + blockIdx.x;
+    pdl_trigger();
+    pdl_wait();
     const long long step = P->clk[0] + (record ? 1 : 0);
     const double dt = P->tclk[1];
     const double tn = P->tclk[0] + (double)step * dt;
@@ -692,33 +695,33 @@ __global__ void __launch_bounds__(EXPM_THREADS) expm_kernel(const ProblemDev* pr
         }
         __syncthreads();
     }
-    // X^(2^s) e_1 by products with e_1 or by squarings, whichever is less work
-    double* Rm = Q;
-    const long long nmv = s < 40 ? 1LL << s : 1LL << 40;
-    if ((double)nmv <= (double)s * n || s == 0) {
-        double* x = Um;
-        double* y = Wm;
-        for (int r = tid; r < n; r += blockDim.x) x[r] = (r == 0) ? 1.0 : 0.0;
-        __syncthreads();
-        for (long long it = 0; it < nmv; ++it) {
-            for (int r = tid; r < n; r += blockDim.x) y[r] = dot_strided(Rm + r * n, 1, x, 1, n);
-            __syncthreads();
-            double* t = x;
-            x = y;
-            y = t;
-        }
-        for (int r = tid; r < n; r += blockDim.x) eo[r] = x[r];
-    } else {
-        double* cur = Rm;
-        double* nxt = Um;
-        for (int it = 0; it < s; ++it) {
-            mat_mul(cur, cur, nxt, n);
-            double* t = cur;
-            cur = nxt;
-            nxt = t;
-        }
-        for (int r = tid; r < n; r += blockDim.x) eo[r] = cur[r * n + 0];
+    // X^(2^s) e_1: s - k squarings of X, then 2^k products with a vector, k by the cost of the two in
+    // cycles (a squaring is bound by the FP64 pipe, 2 products a cycle; a product with a vector by
+    // its latency, about 700: all 2^s of them, s = 7 for a step at 8 times the leap-frog step, were
+    // half of the kernel's 200 us)
+    const double cost_sq = 1500.0 + 0.6 * n * n * n, cost_mv = 700.0 + 0.6 * n * n;
+    int k = 0;
+    while (k < s && k < 20 && ldexp(cost_mv, k) < cost_sq) ++k;
+    double* cur = Q;
+    double* nxt = Um;
+    for (int it = 0; it < s - k; ++it) {
+        mat_mul(cur, cur, nxt, n);
+        double* t = cur;
+        cur = nxt;
+        nxt = t;
     }
+    double* x = Wm;
+    double* y = Tm;
+    for (int r = tid; r < n; r += blockDim.x) x[r] = (r == 0) ? 1.0 : 0.0;
+    __syncthreads();
+    for (int it = 0; it < 1 << k; ++it) {
+        if (tid < n) y[tid] = dot_strided(cur + tid * n, 1, x, 1, n);
+        __syncthreads();
+        double* t = x;
+        x = y;
+        y = t;
+    }
+    if (tid < n) eo[tid] = x[tid];
 }
 
 // ---------------------------------------------------------------- Faber coefficients
@@ -757,10 +760,8 @@ void launch_reset_cursor(const ProblemDev* probs, int nprob, cudaStream_t s) {
 }
 static void launch_between(int precision, const ProblemDev* probs, int nprob, int record, int vec, int kind, int m,
                            double gamma, double c0, double c1, cudaStream_t s) {
-    if (precision == 0)
-        between_kernel<float><<<nprob, PRO_THREADS, 0, s>>>(probs, nprob, record, vec, kind, m, gamma, c0, c1);
-    else
-        between_kernel<double><<<nprob, PRO_THREADS, 0, s>>>(probs, nprob, record, vec, kind, m, gamma, c0, c1);
+    launch_pdl(precision == 0 ? between_kernel<float> : between_kernel<double>, nprob, PRO_THREADS, 0, s, probs, nprob,
+               record, vec, kind, m, gamma, c0, c1);
 }
 void launch_prologue(const ProblemDev* probs, int nprob, int kind, int m, double gamma,
                      double c0, double c1, cudaStream_t s) {

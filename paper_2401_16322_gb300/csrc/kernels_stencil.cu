@@ -26,9 +26,9 @@
 // points a thread covered 14), damping looked up instead of evaluated, terms whose
 // coefficient is zero left out (the w rows of H vanish wherever no damping acts, the
 // epilogue's unused operands), and no shared memory, whose bandwidth is not the limit.
-// Measured on 601 x 301 in FP64: a Faber degree 37 us (102 us before), 65 FP64 instructions a
-// point (about 150), FP64 pipe 63 % busy; HORK 12 on 101 x 101, FP64: 8.5 us a pass (45 us).
-// FP32 on 601 x 301: H x 6.2 us and H^T x 10.2 us a call (29 us).
+// Measured on 601 x 301 in FP64: a Faber degree 35 us (102 us with four points a thread in shared
+// memory), 65 FP64 instructions a point (about 150), FP64 pipe 63 % busy; HORK 12 on 101 x 101,
+// FP64: 7.7 us a pass (45 us).  FP32 on 601 x 301: H x and H^T x 12.7 us for the pair (59 us).
 //
 // Epilogue (StageArgs), per field f at every output point:
 //   K   = cx X + ch xs (H X + sigma e_src)          (xs: per-problem scale, Krylov)
@@ -39,6 +39,7 @@
 #include <type_traits>
 
 #include "ewave_internal.cuh"
+#include "pdl.cuh"
 
 namespace ewv {
 
@@ -292,6 +293,7 @@ __device__ __forceinline__ void epilogue(const ProblemDev& P, const StageArgs& a
         ch *= xs;
         cax *= xs;
     }
+    pdl_trigger();
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
         const bool pad = (f == 2 && padx) || (f == 3 && pady);
@@ -455,6 +457,7 @@ __device__ __forceinline__ void transpose_point(const ProblemDev& P, const Stage
 template <typename T, int R, int PASS, int TERMS>
 __device__ __forceinline__ void stage_point(const ProblemDev& P, const StageArgs& a, int lt, int sub) {
     const PointAt q(P, lt, sub);
+    pdl_wait();
     if (q.i >= P.nx || q.j >= P.ny) return;
     const bool band = R == 4 && P.fs != 0 && q.j < 4;       // (a warp is one row)
     if constexpr (PASS == PASS_FORWARD) {
@@ -548,6 +551,7 @@ __device__ __forceinline__ void leapfrog_point(const ProblemDev& P, int i, int j
             wyp = variant != 1 ? ((T(1) - b.yh * dt) * wym + T(2) * dt * gy) / (T(1) + b.yh * dt)
                                : wym + T(2) * dt * (-b.yh * wy + gy);
     }
+    pdl_trigger();
     Pn[o] = up;
     Pn[2 * fstr + o] = wxp;
     Pn[3 * fstr + o] = wyp;
@@ -560,6 +564,7 @@ leapfrog_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ ti
     const int tile = blockIdx.x / DSUB;
     const ProblemDev& P = probs[tile_prob[tile]];
     const PointAt q(P, tile - P.tile_base, blockIdx.x % DSUB);
+    pdl_wait();
     if (q.i >= P.nx || q.j >= P.ny) return;
     if (R == 4 && P.fs != 0 && q.j < 4) leapfrog_point<T, R, R == 4>(P, q.i, q.j, cur, prev, variant, dt);
     else leapfrog_point<T, R, false>(P, q.i, q.j, cur, prev, variant, dt);
@@ -584,6 +589,16 @@ static void with_pass(int precision, int R, const StageArgs& a, F&& launch) {
     else with_type<PASS_FORWARD>(precision, R, launch);
 }
 
+// Programmatic dependent launch for grids that fill the chip several times over (1520 blocks of 601
+// x 301: 37.8 -> 35 us a Faber degree in FP64); a grid of a block per SM or less runs slower that
+// way (112 blocks of 101 x 101: 7.7 -> 8.2 us a pass), its blocks set up early end up sharing SMs.
+template <class... P, class... A>
+static void launch_plain(void (*kernel)(P...), int blocks, cudaStream_t s, A... args) {
+    const dim3 block(DBX, DBY);
+    if (blocks >= 600) launch_pdl(kernel, blocks, block, 0, s, args...);
+    else kernel<<<blocks, block, 0, s>>>(static_cast<P>(args)...);
+}
+
 void launch_stage(int precision, int R, int ntiles, const ProblemDev* probs, const int* tile_prob,
                   const StageArgs& a_in, cudaStream_t s) {
     if (ntiles <= 0) return;
@@ -593,18 +608,17 @@ void launch_stage(int precision, int R, int ntiles, const ProblemDev* probs, con
         using T = decltype(zero);
         constexpr int RR = decltype(r)::value, PASS = decltype(pass)::value;
         const int blocks = ntiles * DSUB;
-        const dim3 block(DBX, DBY);
         if constexpr (sizeof(T) == 8 && PASS == PASS_FORWARD) {
             constexpr int FABER = TERM_CX | TERM_CU | TERM_A | TERM_CAY, HORK = TERM_CX | TERM_A | TERM_CAY;
             switch (a.terms) {
-                case FABER: stage_kernel<T, RR, PASS, FABER><<<blocks, block, 0, s>>>(probs, tile_prob, a); return;
-                case HORK: stage_kernel<T, RR, PASS, HORK><<<blocks, block, 0, s>>>(probs, tile_prob, a); return;
-                case TERM_CU: stage_kernel<T, RR, PASS, TERM_CU><<<blocks, block, 0, s>>>(probs, tile_prob, a); return;
-                case TERM_XS: stage_kernel<T, RR, PASS, TERM_XS><<<blocks, block, 0, s>>>(probs, tile_prob, a); return;
+                case FABER: launch_plain(stage_kernel<T, RR, PASS, FABER>, blocks, s, probs, tile_prob, a); return;
+                case HORK: launch_plain(stage_kernel<T, RR, PASS, HORK>, blocks, s, probs, tile_prob, a); return;
+                case TERM_CU: launch_plain(stage_kernel<T, RR, PASS, TERM_CU>, blocks, s, probs, tile_prob, a); return;
+                case TERM_XS: launch_plain(stage_kernel<T, RR, PASS, TERM_XS>, blocks, s, probs, tile_prob, a); return;
                 default: break;
             }
         }
-        stage_kernel<T, RR, PASS, -1><<<blocks, block, 0, s>>>(probs, tile_prob, a);
+        launch_plain(stage_kernel<T, RR, PASS, -1>, blocks, s, probs, tile_prob, a);
     });
 }
 
@@ -614,8 +628,7 @@ int launch_stage_one(int precision, int R, const ProblemDev& P, const StageArgs&
     with_pass(precision, R, a, [&](auto zero, auto r, auto pass) {
         constexpr int PASS = decltype(pass)::value;
         if constexpr (PASS != PASS_GRADIENT)
-            stage_one_kernel<decltype(zero), decltype(r)::value, PASS, 0>
-                <<<P.ntiles * DSUB, dim3(DBX, DBY), 0, s>>>(P, a);
+            launch_plain(stage_one_kernel<decltype(zero), decltype(r)::value, PASS, 0>, P.ntiles * DSUB, s, P, a);
     });
     return 0;
 }
@@ -623,9 +636,8 @@ int launch_stage_one(int precision, int R, const ProblemDev& P, const StageArgs&
 void launch_leapfrog(int R, int ntiles, const ProblemDev* probs, const int* tile_prob, int cur, int prev,
                      int variant, double dt, cudaStream_t s) {
     if (ntiles <= 0) return;
-    const dim3 block(DBX, DBY);
-    if (R == 4) leapfrog_kernel<double, 4><<<ntiles * DSUB, block, 0, s>>>(probs, tile_prob, cur, prev, variant, dt);
-    else leapfrog_kernel<double, 2><<<ntiles * DSUB, block, 0, s>>>(probs, tile_prob, cur, prev, variant, dt);
+    if (R == 4) launch_plain(leapfrog_kernel<double, 4>, ntiles * DSUB, s, probs, tile_prob, cur, prev, variant, dt);
+    else launch_plain(leapfrog_kernel<double, 2>, ntiles * DSUB, s, probs, tile_prob, cur, prev, variant, dt);
 }
 
 // --------------------------------------------------------------------------------------

@@ -4,12 +4,12 @@
 // Appendix A / Sec. 2.2 free-surface rows, in-register damping, and the
 // K / Y / ACC epilogue of every integrator), organised for HBM bandwidth:
 //   - one CTA per SM walks the tile work list (tiles b, b + gridDim.x, ...);
-//   - warp 8 (one elected lane) is the producer: for each tile it issues TMA tensor loads
+//   - the last warp (one elected lane) is the producer: for each tile it issues TMA tensor loads
 //     (cp.async.bulk.tensor) of every operand into one of NST shared-memory stages and
 //     arms the stage's "full" mbarrier with the transaction byte count;
-//   - warps 0..15 are consumers: they wait on "full", compute the 64 x 16 tile from shared
-//     memory (2 consecutive rows per thread, y taps slid in registers), store Y / ACC with
-//     coalesced st.global, and arrive on the stage's "empty" mbarrier.
+//   - the other warps are consumers: they wait on "full", compute the tile from shared memory
+//     (two adjacent columns and one to four rows per thread), store Y / ACC with coalesced
+//     st.global, and arrive on the stage's "empty" mbarrier.
 // The TMA boxes (4D tensor maps over x, y, field, vector) start R rows above and 4 columns
 // left of the tile (16-byte aligned x); out-of-range elements are filled with zeros by
 // the TMA unit, which is exactly the zero extension of Sec. 2.1.
@@ -18,16 +18,15 @@
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
-#include <type_traits>
 #include <vector>
 
 #include "ewave_internal.cuh"
+#include "pdl.cuh"
 
 namespace ewv {
 
 constexpr int TX = 4;                 // staged x halo (>= R, keeps the box start 16-B aligned)
 constexpr int NMAP = 12;              // tensor maps per problem and tile height
-constexpr int MAX_NST = 5;
 
 // Shared-memory layout of one stage (floats) for tile height BYv; every buffer starts on a
 // 128-byte boundary.  HASU = false drops the U buffer (passes without a U operand, e.g. the
@@ -63,7 +62,8 @@ struct __align__(16) TileInfo {
     int x0, y0, nx, ny, pitch, pml, fs, src_i, src_j, shot;
     float beta0, inv_pml, idx1, idx2, sig, xs;   // xs: per-problem scale of H X (Krylov)
     const float* btab;       // damping at half-cell distances (ProblemDev::btab)
-    int nbtab, pad3;
+    int nbtab;
+    int xdamp;               // the tile's columns, and 8 more on each side, touch the damping layer
 };
 
 // The consumers read a stage's TileInfo with 16-byte shared loads into registers.
@@ -77,14 +77,6 @@ __device__ __forceinline__ TileInfo load_info(const TileInfo* p) {
     for (int q = 0; q < (int)(sizeof(TileInfo) / 16); ++q) u.v[q] = reinterpret_cast<const int4*>(p)[q];
     return u.t;
 }
-template <bool kRegs>
-__device__ __forceinline__ std::conditional_t<kRegs, TileInfo, const TileInfo&> tile_info(const TileInfo* p) {
-    if constexpr (kRegs)
-        return load_info(p);
-    else
-        return *p;
-}
-
 __device__ __forceinline__ uint32_t smem_addr(const void* p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
@@ -216,43 +208,19 @@ __device__ __forceinline__ float cent_tree(float u, const float (&p)[R]) {
         return fmaf(cent<R>(1), p[0], cent<R>(0) * u) + cent<R>(2) * p[1];
 }
 
-// Two-row arithmetic on packed FP32 pairs (one instruction for both rows of a consumer
-// thread; each component rounds exactly as the scalar operation does).
+// Arithmetic on packed FP32 pairs (one instruction for both columns of a consumer thread; each
+// component rounds exactly as the scalar operation does).
 __device__ __forceinline__ float2 f2(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ float2 f2s(float a) { return make_float2(a, a); }
 __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, f2s(-1.f), a); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-template <int R>
-__device__ __forceinline__ float2 stag_tree2(const float2 (&d)[R]) {
-    if constexpr (R == 4)
-        return add2(fma2(f2s(stag<4>(0)), d[0], mul2(f2s(stag<4>(1)), d[1])),
-                    fma2(f2s(stag<4>(2)), d[2], mul2(f2s(stag<4>(3)), d[3])));
-    else
-        return fma2(f2s(stag<R>(0)), d[0], mul2(f2s(stag<R>(1)), d[1]));
-}
-template <int R>
-__device__ __forceinline__ float2 cent_tree2(float2 u, const float2 (&p)[R]) {
-    if constexpr (R == 4)
-        return add2(add2(fma2(f2s(cent<4>(1)), p[0], mul2(f2s(cent<4>(0)), u)),
-                         fma2(f2s(cent<4>(3)), p[2], mul2(f2s(cent<4>(2)), p[1]))),
-                    mul2(f2s(cent<4>(4)), p[3]));
-    else
-        return add2(fma2(f2s(cent<R>(1)), p[0], mul2(f2s(cent<R>(0)), u)), mul2(f2s(cent<R>(2)), p[1]));
-}
-
 // beta at 2 d = k half cells from the first ghost line (zero beyond the layer).  Columns and
 // rows past the grid edge (ragged tiles, never stored) give k <= 0; the unsigned test sends
 // negative k to zero as well, so the table is never read outside its n entries.
 __device__ __forceinline__ float btab_at(const float* t, int n, int k) {
     return (unsigned)k < (unsigned)n ? __ldg(t + k) : 0.f;
-}
-
-__device__ __forceinline__ float dampf(float beta0, float inv_pml, float d, int pml) {
-    if (pml <= 0) return 0.f;
-    const float r = 1.f - d * inv_pml;
-    return (d <= (float)pml) ? beta0 * r * r : 0.f;
 }
 
 // Map of field box `kind` (0 u, 1 w_x, 2 w_y, 3 v, 4 four fields) for vector k.
@@ -293,6 +261,7 @@ __device__ __forceinline__ void fill_tile_info(TileInfo& ti, const ProblemDev* P
     ti.shot = P->shot;
     ti.btab = P->btab;
     ti.nbtab = P->nbtab;
+    ti.xdamp = x0 - 8 < P->pml || x0 + BX + 8 > P->nx - P->pml;
     ti.beta0 = P->fbeta0;
     ti.inv_pml = P->finv_pml;
     ti.idx1 = P->finv_dx;
@@ -316,17 +285,20 @@ __device__ __forceinline__ int tma_produce(const ProblemDev* __restrict__ probs,
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
         const int s = it % NSTv;
         const uint32_t ph = (uint32_t)(it / NSTv) & 1u;
-        if (!mbar_wait(&empty[s], ph ^ 1u, wait_lim)) {
-            *s_err = 1;
-            break;
-        }
+        // (the tile is resolved before the wait, so that a stage set free is refilled at once)
         const int pid = find_problem(tbase, nprob, tile);
         const ProblemDev* P = probs + pid;
         const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(P->tmaps) + mapset * NMAP;
         const int tiles_x = (P->nx + BX - 1) / BX;
         const int lt = tile - __ldg(tbase + pid);
         const int x0 = (lt % tiles_x) * BX, y0 = (lt / tiles_x) * BYv;
-        fill_tile_info(info[s], P, a, x0, y0);
+        TileInfo ti;
+        fill_tile_info(ti, P, a, x0, y0);
+        if (!mbar_wait(&empty[s], ph ^ 1u, wait_lim)) {
+            *s_err = 1;
+            break;
+        }
+        info[s] = ti;
         float* st = smem + (size_t)s * L::FLOATS;
         // the arrive below releases the tile info together with the copies
         mbar_expect_tx(&full[s], bytes);
@@ -370,361 +342,19 @@ __device__ __forceinline__ void tma_finish(int s_err, int issued, uint64_t* full
     }
 }
 
-// EPI 0: the general epilogue.  EPI 1: the steady-state form of the Faber and HORK passes,
-// ck = 1 and cau = cak = cax = 0:  Y = cu U + cx X + ch (H X + sigma),  ACC = ca A + cay Y.
-template <int R, int BYv, int NW, int NSTv, int EPI, bool HASU>
-__global__ void __launch_bounds__(NW * 32 + 32, 1)
-stage_tma_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ tbase, int nprob,
-                 int ntiles, int mapset, StageArgs a, int* err) {
-    using L = StageLayout<R, BYv, HASU>;
-    constexpr int NCONS = NW * 32;
-    constexpr int TPR = NCONS / BX;             // consumer thread rows
-    constexpr int NR = BYv / TPR;               // consecutive rows per consumer thread
-    static_assert(NR * TPR == BYv && NR >= 1, "tile rows must split evenly over threads");
-    extern __shared__ __align__(1024) unsigned char smem_raw[];
-    // TMA destinations need 128-byte alignment: align the dynamic base explicitly (the
-    // launch reserves 1 KB of slack for this).
-    float* smem = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    __shared__ __align__(8) uint64_t full[NSTv];
-    __shared__ __align__(8) uint64_t empty[NSTv];
-    __shared__ TileInfo info[NSTv];
-    __shared__ int s_err;
-
-    const int tid = threadIdx.x;
-    const int warp = tid >> 5, lane = tid & 31;
-    const uint64_t wait_lim = g_tma_wait_limit_ns;
-    if (tid == 0) {
-        for (int s = 0; s < NSTv; ++s) {
-            mbar_init(&full[s], 1);
-            mbar_init(&empty[s], NW);
-        }
-        s_err = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
-    __syncthreads();
-
-    const bool has_u = HASU && a.u >= 0, has_a = a.a >= 0;
-    const uint32_t bytes = tma_stage_bytes<R, BYv, EPI, HASU>(a);
-    int issued = 0;
-
-    if (warp == NW) {
-        // ------------------------------------------------------------ producer
-        if (lane == 0)
-            issued = tma_produce<R, BYv, NSTv, EPI, HASU>(probs, tbase, nprob, ntiles, mapset, a, smem, full,
-                                                          empty, info, &s_err, bytes, wait_lim);
-    } else {
-        // ------------------------------------------------------------ consumers
-        const int tx = tid & (BX - 1);    // x inside the tile
-        const int ty = tid / BX;          // rows NR ty .. NR ty + NR - 1
-#define cxf a.fcx
-#define chf a.fch
-#define cuf a.fcu
-#define ckf a.fck
-#define caf a.fca
-#define cauf a.fcau
-#define cakf a.fcak
-#define cayf a.fcay
-#define caxf a.fcax
-        int it = 0;
-        for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
-            const int s = it % NSTv;
-            const uint32_t ph = (uint32_t)(it / NSTv) & 1u;
-            if (!mbar_wait(&full[s], ph, wait_lim)) {
-                s_err = 1;
-                break;
-            }
-            // The tile descriptor: copied into registers where they are plentiful; read from
-            // shared memory field by field by the 20-warp variant (80 registers a thread).
-            using TI = std::conditional_t<(NW < 20), const TileInfo, const TileInfo&>;
-            TI ti = tile_info<(NW < 20)>(&info[s]);
-            const int nx = ti.nx, ny = ti.ny, pml = ti.pml;
-            const bool fs = ti.fs != 0;
-            const int y0 = ti.y0;
-            const long long fstr = ti.fstr;
-            const float beta0 = ti.beta0, inv_pml = ti.inv_pml, idx1 = ti.idx1, idx2 = ti.idx2;
-            float* Yg = ti.Y;
-            float* Ag = ti.A;
-            const float* st = smem + (size_t)s * L::FLOATS;
-            const float* su = st + L::U_OFF;
-            const float* swx = st + L::WX_OFF;
-            const float* swy = st + L::WY_OFF;
-            const float* sv = st + L::V_OFF;
-            const float* sc2 = st + L::C2_OFF;
-            const float* spu = st + L::PU_OFF;
-            const float* spa = st + L::PA_OFF;
-            const int i = ti.x0 + tx;
-            const int cxs = tx + TX;                     // staged column of this thread
-            float ucol[NR + 2 * R], wcol[NR + 2 * R - 1];
-#pragma unroll
-            for (int q = 0; q < NR + 2 * R; ++q) ucol[q] = su[(NR * ty + q) * L::SW + cxs];
-#pragma unroll
-            for (int q = 0; q < NR + 2 * R - 1; ++q) wcol[q] = swy[(NR * ty + q) * BX + tx];
-            const float* btab = ti.btab;
-            const int nbt = ti.nbtab;
-            const float bxn = btab_at(btab, nbt, 2 * min(i + 1, nx - i));
-            const float bxh = btab_at(btab, nbt, min(2 * i + 3, 2 * (nx - i) - 1));
-            const bool in_x = i < nx;
-            const float chx = chf * ti.xs;     // ch xs: K = cx X + ch xs (H X + sigma)
-            // EPI 2: one leap-frog step (Sec. 3.1) at a point.  X = level n; the A box holds
-            // level n - 1 (u^{n-1} or, in difference form, d^n in field 1, and w^{n-1});
-            // level n + 1 goes to Y (u, w_x, w_y) and, in difference form, d^{n+1} to field 1
-            // of level n (acc_out), which no thread of this step reads.
-            auto leapfrog_point = [&](int ii, int jj, int ptv, float uu, float c2v, float lap, float dws,
-                                      float dux, float duy, float bxnv, float bxhv, float bynv, float byhv,
-                                      float xwxv, float xwyv) {
-                const float dt = (float)a.dt, bsum = bxnv + bynv;
-                float rhs = -bxnv * bynv * uu + c2v * (lap * idx2 + dws * idx1);
-                if (ii == ti.src_i && jj == ti.src_j) rhs += ti.sig;
-                const float* pm = spa + ptv;
-                const long long o = (long long)jj * ti.pitch + ii;
-                // fast (2-ulp) divisions, as in the 3D step: the step's own error is far larger
-                float up;
-                if (a.m == 2) {
-                    const float hb = 0.5f * bsum * dt;
-                    const float dn = __fdividef(pm[BYv * BX] * (1.f - hb) + dt * dt * rhs, 1.f + hb);
-                    Ag[fstr + o] = dn;
-                    up = uu + dn;
-                } else {
-                    const float um = pm[0];
-                    const float inv_dt2 = 1.f / (dt * dt), inv_2dt = 1.f / (2.f * dt);
-                    up = __fdividef((2.f * uu - um) * inv_dt2 + bsum * um * inv_2dt + rhs, inv_dt2 + bsum * inv_2dt);
-                }
-                float wxp = 0.f, wyp = 0.f;
-                if (ii < nx - 1) {
-                    const float gx = (bynv - bxhv) * dux * idx1, wm = pm[2 * BYv * BX];
-                    wxp = a.m != 1 ? __fdividef((1.f - bxhv * dt) * wm + 2.f * dt * gx, 1.f + bxhv * dt)
-                                   : wm + 2.f * dt * (-bxhv * xwxv + gx);
-                }
-                if (jj < ny - 1) {
-                    const float gy = (bxnv - byhv) * duy * idx1, wm = pm[3 * BYv * BX];
-                    wyp = a.m != 1 ? __fdividef((1.f - byhv * dt) * wm + 2.f * dt * gy, 1.f + byhv * dt)
-                                   : wm + 2.f * dt * (-byhv * xwyv + gy);
-                }
-                Yg[o] = up;
-                Yg[2 * fstr + o] = wxp;
-                Yg[3 * fstr + o] = wyp;
-            };
-            bool paired = false;
-            if constexpr (NR == 2 && EPI >= 1) {
-                // Both rows of this thread as packed pairs (rows below the free-surface
-                // band: the interior stencils apply to both).
-                const int ly0 = 2 * ty;
-                const int j0 = y0 + ly0, j1 = j0 + 1;
-                paired = !(fs && j0 < 4);
-                if (paired && in_x && j0 < ny) {
-                    const float* urow0 = su + (ly0 + R) * L::SW + cxs;
-                    const float* urow1 = urow0 + L::SW;
-                    const float* wx0 = swx + ly0 * L::SW + cxs;
-                    const float* wx1 = wx0 + L::SW;
-                    const float2 uc = f2(ucol[R], ucol[R + 1]);
-                    // The pair sums and differences of the taps are packed; the products with
-                    // the stencil weights stay scalar (immediate operands, no registers held).
-                    // lap = 2 c_0 u + sum_k c_k (x pair sum + y pair sum); the divergence of w
-                    // and d_x u, d_y u accumulate their staggered differences the same way.
-                    float lap0 = (2.f * cent<R>(0)) * uc.x, lap1 = (2.f * cent<R>(0)) * uc.y;
-                    float dw0 = 0.f, dw1 = 0.f, ux0 = 0.f, ux1 = 0.f, uy0 = 0.f, uy1 = 0.f;
-#pragma unroll
-                    for (int k = 0; k < R; ++k) {
-                        const float2 ap = f2(urow0[k + 1], urow1[k + 1]);
-                        const float2 am = f2(urow0[-k - 1], urow1[-k - 1]);
-                        const float2 a0 = k == 0 ? uc : f2(urow0[-k], urow1[-k]);
-                        const float2 sl = add2(ap, am);
-                        const float2 sx = sub2(ap, a0);
-                        const float2 sw = sub2(f2(wx0[k], wx1[k]), f2(wx0[-1 - k], wx1[-1 - k]));
-                        lap0 = fmaf(cent<R>(k + 1), sl.x + (ucol[R + k + 1] + ucol[R - k - 1]), lap0);
-                        lap1 = fmaf(cent<R>(k + 1), sl.y + (ucol[R + k + 2] + ucol[R - k]), lap1);
-                        ux0 = fmaf(stag<R>(k), sx.x, ux0);
-                        ux1 = fmaf(stag<R>(k), sx.y, ux1);
-                        uy0 = fmaf(stag<R>(k), ucol[R - k] - ucol[R + 1 + k], uy0);
-                        uy1 = fmaf(stag<R>(k), ucol[R - k + 1] - ucol[R + 2 + k], uy1);
-                        dw0 = fmaf(stag<R>(k), sw.x + (wcol[R - 1 - k] - wcol[R + k]), dw0);
-                        dw1 = fmaf(stag<R>(k), sw.y + (wcol[R - k] - wcol[R + k + 1]), dw1);
-                    }
-                    if constexpr (EPI == 3) {
-                        // FWI gradient pass: grad += gscale q_v (L u + D w) of X (m = c^2)
-                        float* G = (float*)a.grad + (long long)ti.shot * fstr;
-                        const long long o0 = (long long)j0 * ti.pitch + i;
-                        const float gs = (float)a.gscale;
-                        G[o0] += gs * spa[BYv * BX + ly0 * BX + tx] * (lap0 * idx2 + dw0 * idx1);
-                        if (j1 < ny) G[o0 + ti.pitch] += gs * spa[BYv * BX + ly0 * BX + BX + tx] * (lap1 * idx2 + dw1 * idx1);
-                    } else {
-                    const float byn0 = btab_at(btab, nbt, 2 * (fs ? ny - j0 : min(j0 + 1, ny - j0)));
-                    const float byn1 = btab_at(btab, nbt, 2 * (fs ? ny - j1 : min(j1 + 1, ny - j1)));
-                    const float byh0 = btab_at(btab, nbt, fs ? 2 * (ny - j0) - 1 : min(2 * j0 + 3, 2 * (ny - j0) - 1));
-                    const float byh1 = btab_at(btab, nbt, fs ? 2 * (ny - j1) - 1 : min(2 * j1 + 3, 2 * (ny - j1) - 1));
-                    const int pt0 = ly0 * BX + tx, pt1 = pt0 + BX;
-                    if constexpr (EPI == 2) {
-                        leapfrog_point(i, j0, pt0, uc.x, sc2[pt0], lap0, dw0, ux0, uy0, bxn, bxh, byn0, byh0,
-                                       wx0[0], wcol[R]);
-                        if (j1 < ny)
-                            leapfrog_point(i, j1, pt1, uc.y, sc2[pt1], lap1, dw1, ux1, uy1, bxn, bxh, byn1, byh1,
-                                           wx1[0], wcol[R + 1]);
-                    } else {
-                    const float xv0 = sv[pt0], xv1 = sv[pt1];
-                    const float xwx0 = wx0[0], xwx1 = wx1[0];
-                    const float xwy0 = wcol[R], xwy1 = wcol[R + 1];
-                    // H v = -bx by u + c^2 (lap u / dx^2 + div w / dx) - (bx + by) v
-                    float hv0 = -bxn * byn0 * uc.x + sc2[pt0] * (lap0 * idx2 + dw0 * idx1) - (bxn + byn0) * xv0;
-                    float hv1 = -bxn * byn1 * uc.y + sc2[pt1] * (lap1 * idx2 + dw1 * idx1) - (bxn + byn1) * xv1;
-                    if (i == ti.src_i) {
-                        if (j0 == ti.src_j) hv0 += ti.sig;
-                        if (j1 == ti.src_j) hv1 += ti.sig;
-                    }
-                    const bool wxin = i < nx - 1;
-                    const float hwx0 = wxin ? (byn0 - bxh) * ux0 * idx1 - bxh * xwx0 : 0.f;
-                    const float hwx1 = wxin ? (byn1 - bxh) * ux1 * idx1 - bxh * xwx1 : 0.f;
-                    const float hwy0 = (j0 < ny - 1) ? (bxn - byh0) * uy0 * idx1 - byh0 * xwy0 : 0.f;
-                    const float hwy1 = (j1 < ny - 1) ? (bxn - byh1) * uy1 * idx1 - byh1 * xwy1 : 0.f;
-                    const bool row1 = j1 < ny;
-                    const long long o0 = (long long)j0 * ti.pitch + i;
-                    const float xf0[4] = {uc.x, xv0, xwx0, xwy0}, xf1[4] = {uc.y, xv1, xwx1, xwy1};
-                    const float hf0[4] = {xv0, hv0, hwx0, hwy0}, hf1[4] = {xv1, hv1, hwx1, hwy1};
-#pragma unroll
-                    for (int f = 0; f < 4; ++f) {
-                        float y0v = fmaf(cxf, xf0[f], chx * hf0[f]);
-                        float y1v = fmaf(cxf, xf1[f], chx * hf1[f]);
-                        if (has_u) {
-                            y0v = fmaf(cuf, spu[f * BYv * BX + pt0], y0v);
-                            y1v = fmaf(cuf, spu[f * BYv * BX + pt1], y1v);
-                        }
-                        if ((f == 2 && !wxin) || (f == 3 && j0 >= ny - 1)) y0v = 0.f;
-                        if ((f == 2 && !wxin) || (f == 3 && j1 >= ny - 1)) y1v = 0.f;
-                        if (Yg) {
-                            float* yp = Yg + f * fstr + o0;
-                            yp[0] = y0v;
-                            if (row1) yp[ti.pitch] = y1v;
-                        }
-                        if (Ag) {
-                            float a0v = cayf * y0v, a1v = cayf * y1v;
-                            if (has_a) {
-                                a0v = fmaf(cayf, y0v, caf * spa[f * BYv * BX + pt0]);
-                                a1v = fmaf(cayf, y1v, caf * spa[f * BYv * BX + pt1]);
-                            }
-                            float* ap = Ag + f * fstr + o0;
-                            ap[0] = a0v;
-                            if (row1) ap[ti.pitch] = a1v;
-                        }
-                    }
-                    }   // EPI 1
-                    }   // EPI 1, 2
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < NR; ++r) {
-                if (paired) break;
-                const int ly = NR * ty + r;
-                const int j = y0 + ly;
-                const float* urow = su + (ly + R) * L::SW + cxs;
-                const float* wxrow = swx + ly * L::SW + cxs;
-                float px[R], dx[R], dw[R];
-#pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    px[k] = urow[k + 1] + urow[-k - 1];
-                    dx[k] = urow[1 + k] - urow[-k];
-                    dw[k] = wxrow[k] - wxrow[-1 - k];
-                }
-                const float uxx = cent_tree<R>(ucol[r + R], px);
-                const float dux = stag_tree<R>(dx);
-                const float dwx = stag_tree<R>(dw);
-                float uyy, duy, dwy;
-                if (fs && j < 4) {
-                    uyy = 0.f;
-#pragma unroll
-                    for (int q = 0; q < 9; ++q) uyy += g_tma_fs[TFS_UYY + j * 9 + q] * su[(q + R) * L::SW + cxs];
-                    dwy = 0.f;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) dwy += g_tma_fs[TFS_DWY + j * 8 + q] * swy[(q + R) * BX + tx];
-                } else {
-                    float py[R], dwv[R];
-#pragma unroll
-                    for (int k = 0; k < R; ++k) {
-                        py[k] = ucol[r + R + k + 1] + ucol[r + R - k - 1];
-                        dwv[k] = wcol[r + R - 1 - k] - wcol[r + R + k];
-                    }
-                    uyy = cent_tree<R>(ucol[r + R], py);
-                    dwy = stag_tree<R>(dwv);
-                }
-                if (fs && j < 3) {
-                    duy = 0.f;
-#pragma unroll
-                    for (int q = 0; q < 8; ++q) duy += g_tma_fs[TFS_UY + j * 8 + q] * su[(q + R) * L::SW + cxs];
-                } else {
-                    float dy[R];
-#pragma unroll
-                    for (int k = 0; k < R; ++k) dy[k] = ucol[r + R - k] - ucol[r + R + 1 + k];
-                    duy = stag_tree<R>(dy);
-                }
-                if (!in_x || j >= ny) continue;
-                const float byn = btab_at(btab, nbt, 2 * (fs ? ny - j : min(j + 1, ny - j)));
-                const float byh = btab_at(btab, nbt, fs ? 2 * (ny - j) - 1 : min(2 * j + 3, 2 * (ny - j) - 1));
-                const int pt = ly * BX + tx;
-                if constexpr (EPI == 3) {
-                    float* G = (float*)a.grad + (long long)ti.shot * fstr;
-                    G[(long long)j * ti.pitch + i] += (float)a.gscale * spa[BYv * BX + pt] *
-                                                      ((uxx + uyy) * idx2 + (dwx + dwy) * idx1);
-                    continue;
-                }
-                if constexpr (EPI == 2) {
-                    leapfrog_point(i, j, pt, ucol[r + R], sc2[pt], uxx + uyy, dwx + dwy, dux, duy, bxn, bxh,
-                                   byn, byh, wxrow[0], wcol[r + R]);
-                    continue;
-                }
-                const float xu = ucol[r + R], xv = sv[pt], xwx = wxrow[0], xwy = wcol[r + R];
-                const float c2 = sc2[pt];
-                float hv = -bxn * byn * xu + c2 * ((uxx + uyy) * idx2 + (dwx + dwy) * idx1) - (bxn + byn) * xv;
-                if (i == ti.src_i && j == ti.src_j) hv += ti.sig;
-                const float hwx = (i < nx - 1) ? (byn - bxh) * dux * idx1 - bxh * xwx : 0.f;
-                const float hwy = (j < ny - 1) ? (bxn - byh) * duy * idx1 - byh * xwy : 0.f;
-                const float xf[4] = {xu, xv, xwx, xwy};
-                const float hf[4] = {xv, hv, hwx, hwy};
-                const long long o = (long long)j * ti.pitch + i;
-                float* yrow = Yg ? Yg + o : nullptr;
-                float* arow = Ag ? Ag + o : nullptr;
-#pragma unroll
-                for (int f = 0; f < 4; ++f) {
-                    const bool pad = (f == 2 && i >= nx - 1) || (f == 3 && j >= ny - 1);
-                    const float uval = has_u ? spu[f * BYv * BX + pt] : 0.f;
-                    const float aval = has_a ? spa[f * BYv * BX + pt] : 0.f;
-                    const float kf = fmaf(cxf, xf[f], chx * hf[f]);
-                    if constexpr (EPI == 1) {
-                        const float yf = pad ? 0.f : (has_u ? fmaf(cuf, uval, kf) : kf);
-                        if (yrow) yrow[f * fstr] = yf;
-                        if (arow) arow[f * fstr] = has_a ? fmaf(cayf, yf, caf * aval) : cayf * yf;
-                    } else {
-                        const float yf = pad ? 0.f : (cuf * uval + ckf * kf);
-                        if (yrow) yrow[f * fstr] = yf;
-                        if (arow) arow[f * fstr] = pad ? 0.f : (caf * aval + cauf * uval + cakf * kf + cayf * yf + caxf * xf[f]);
-                    }
-                }
-            }
-            __syncwarp();
-            if (lane == 0) mbar_arrive(&empty[s]);
-        }
-    }
-    __syncthreads();
-    // (issued is non-zero on the producer lane only)
-    tma_finish<NSTv>(s_err, issued, full, err);
-}
-
-#undef cxf
-#undef chf
-#undef cuf
-#undef ckf
-#undef caf
-#undef cauf
-#undef cakf
-#undef cayf
-#undef caxf
-
-// ---------------------------------------------------------------- column-pair consumers
-// The same pass with every consumer thread on two adjacent columns (x, x + 1) of NR
-// consecutive rows: the column pair of a staged row is one 8-byte shared load, and the
-// arithmetic runs on packed FP32 pairs (one instruction for both columns).  The y taps of
-// both columns slide in registers as pairs; the x taps of a row are the five pairs from
-// x - 4 to x + 5, and the taps that straddle two pairs (odd offsets) are formed with scalar
-// operations.  Per grid point this issues about a third of the shared loads of the
-// one-column form and shares each tile's setup over twice the points.  Rows of the
-// free-surface band (Appendix A stencils, top tile only) take a scalar path per point.
+// ---------------------------------------------------------------- consumers
+// Every consumer thread owns two adjacent columns (x, x + 1) of NR consecutive rows: the column
+// pair of a staged row is one 8-byte shared load, and the arithmetic runs on packed FP32 pairs (one
+// instruction for both columns).  The y taps of both columns slide in registers as pairs; the x
+// taps of a row are the five pairs from x - 4 to x + 5, and the taps that straddle two pairs (odd
+// offsets) are formed with scalar operations.  Per grid point this issues about a third of the
+// shared loads of one column per thread and shares each tile's setup over twice the points.
+// Every tile shape does the same arithmetic per point: the results do not depend on the variant
+// the autotuner picks.  Rows of the free-surface band (Appendix A stencils, top tile only) take a
+// scalar path per point.
+// EPI 0: the general epilogue.  EPI 1: the steady-state form of the Faber and HORK passes, ck = 1
+// and cau = cak = cax = 0:  Y = cu U + cx X + ch (H X + sigma),  ACC = ca A + cay Y.  EPI 2: one
+// leap-frog step.  EPI 3: the gradient pass.
 __device__ __forceinline__ float2 lds2(const float* p) { return *reinterpret_cast<const float2*>(p); }
 __device__ __forceinline__ void st2(float* p, float2 v, bool both) {
     if (both)
@@ -733,10 +363,10 @@ __device__ __forceinline__ void st2(float* p, float2 v, bool both) {
         p[0] = v.x;
 }
 
-// One leap-frog step (Sec. 3.1) at a point of the column-pair form: level n in registers,
-// level n - 1 (u^{n-1}, or d^n in field 1 in difference form, and w^{n-1}) from the A stage
-// box at pa (fields plane floats apart); level n + 1 (u, w_x, w_y) goes to Y and, in
-// difference form, d^{n+1} to field 1 of A.  Same arithmetic as the one-column form.
+// One leap-frog step (Sec. 3.1) at a damped point: level n in registers, level n - 1 (u^{n-1},
+// or d^n in field 1 in difference form, and w^{n-1}) from the A stage box at pa (fields plane
+// floats apart); level n + 1 (u, w_x, w_y) goes to Y and, in difference form, d^{n+1} to field 1
+// of A, which no thread of this step reads.
 __device__ __forceinline__ void lf_point(const TileInfo& ti, const StageArgs& a, const float* pa, int plane, int ii,
                                          int jj, float uu, float c2v, float lap, float dws, float dux, float duy,
                                          float bxnv, float bxhv, float bynv, float byhv, float xwxv, float xwyv) {
@@ -746,7 +376,7 @@ __device__ __forceinline__ void lf_point(const TileInfo& ti, const StageArgs& a,
     if (ii == ti.src_i && jj == ti.src_j) rhs += ti.sig;
     const long long o = (long long)jj * ti.pitch + ii;
     const long long fstr = ti.fstr;
-    // fast (2-ulp) divisions, as in the one-column form
+    // fast (2-ulp) divisions: the step's own error is far larger
     float up;
     if (a.m == 2) {
         const float hb = 0.5f * bsum * dt;
@@ -774,8 +404,8 @@ __device__ __forceinline__ void lf_point(const TileInfo& ti, const StageArgs& a,
     ti.Y[3 * fstr + o] = wyp;
 }
 
-// One point (tile column tc, tile row lr) from shared memory with the scalar formulas of the
-// one-column form, free-surface rows included, and its epilogue.
+// One point (tile column tc, tile row lr) from shared memory with scalar formulas, free-surface
+// rows included, and its epilogue.
 template <int R, int BYv, int EPI, bool HASU, bool HASA>
 __device__ __forceinline__ void tma_point_scalar(const float* st, const TileInfo& ti, const StageArgs& a, int tc,
                                              int lr, bool has_u, bool has_a) {
@@ -911,6 +541,8 @@ stage_tma_x2_kernel(const ProblemDev* __restrict__ probs, const int* __restrict_
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_trigger();
+    pdl_wait();
     const bool has_u = HASU && a.u >= 0, has_a = HASA && a.a >= 0;
     int issued = 0;
     if (warp == NW) {
@@ -963,11 +595,18 @@ stage_tma_x2_kernel(const ProblemDev* __restrict__ probs, const int* __restrict_
                     for (int q = 0; q < NR + 2 * R - 1; ++q) wcol[q] = lds2(swy + (r0 + q) * BX + c0);
                     const float* btab = ti.btab;
                     const int nbt = ti.nbtab;
-                    const float2 bxn = f2(btab_at(btab, nbt, 2 * min(i0 + 1, nx - i0)),
-                                          btab_at(btab, nbt, 2 * min(i0 + 2, nx - i0 - 1)));
-                    const float2 bxh = f2(btab_at(btab, nbt, min(2 * i0 + 3, 2 * (nx - i0) - 1)),
-                                          btab_at(btab, nbt, min(2 * i0 + 5, 2 * (nx - i0) - 3)));
-                    const float2 nbxh = f2(-bxh.x, -bxh.y);
+                    // Where nothing damps this thread's points, the w rows of H are zero and the v
+                    // row has no damping term: no look-ups, no half-point differences of u (the
+                    // results are the same to the bit; about a fifth of the instructions).
+                    const bool damped = ti.xdamp || jt + NR > ny - ti.pml || (!fs && jt < ti.pml);
+                    float2 bxn = f2s(0.f), bxh = f2s(0.f), nbxh = f2s(0.f);
+                    if (damped) {
+                        bxn = f2(btab_at(btab, nbt, 2 * min(i0 + 1, nx - i0)),
+                                 btab_at(btab, nbt, 2 * min(i0 + 2, nx - i0 - 1)));
+                        bxh = f2(btab_at(btab, nbt, min(2 * i0 + 3, 2 * (nx - i0) - 1)),
+                                 btab_at(btab, nbt, min(2 * i0 + 5, 2 * (nx - i0) - 3)));
+                        nbxh = f2(-bxh.x, -bxh.y);
+                    }
                     const bool wx0in = i0 < nx - 1, wx1in = i0 + 1 < nx - 1;
                     const float2 idx1 = f2s(ti.idx1), idx2 = f2s(ti.idx2);
                     const float chx = a.fch * ti.xs;
@@ -989,6 +628,18 @@ stage_tma_x2_kernel(const ProblemDev* __restrict__ probs, const int* __restrict_
                         const float2 uc = ucol[r + R];
                         float2 lap = mul2(f2s(2.f * cent<R>(0)), uc);
                         float2 dux = f2s(0.f), duy = f2s(0.f), dw = f2s(0.f);
+                        float byn = 0.f, byh = 0.f;
+                        if (EPI != 3 && damped) {
+                            byn = btab_at(btab, nbt, 2 * (fs ? ny - j : min(j + 1, ny - j)));
+                            byh = btab_at(btab, nbt, fs ? 2 * (ny - j) - 1 : min(2 * j + 3, 2 * (ny - j) - 1));
+                            // staggered differences: d_x u at x + 1/2, d_y u at y + 1/2
+#pragma unroll
+                            for (int k = 0; k < R; ++k) {
+                                const float2 dxu = f2(uo(1 + k) - uo(-k), uo(2 + k) - uo(1 - k));
+                                dux = fma2(f2s(stag<R>(k)), dxu, dux);
+                                duy = fma2(f2s(stag<R>(k)), sub2(ucol[r + R - k], ucol[r + R + 1 + k]), duy);
+                            }
+                        }
 #pragma unroll
                         for (int k = 0; k < R; ++k) {
                             // Laplacian: x and y pair sums at distance k + 1
@@ -997,18 +648,11 @@ stage_tma_x2_kernel(const ProblemDev* __restrict__ probs, const int* __restrict_
                                                        : add2(up[(kk + 4) >> 1], up[(4 - kk) >> 1]);
                             const float2 sy = add2(ucol[r + R + kk], ucol[r + R - kk]);
                             lap = fma2(f2s(cent<R>(kk)), add2(sx, sy), lap);
-                            // staggered differences: d_x u at x + 1/2, d_y u at y + 1/2,
                             // the divergence of w at the node
-                            const float2 dxu = f2(uo(1 + k) - uo(-k), uo(2 + k) - uo(1 - k));
-                            dux = fma2(f2s(stag<R>(k)), dxu, dux);
-                            duy = fma2(f2s(stag<R>(k)), sub2(ucol[r + R - k], ucol[r + R + 1 + k]), duy);
                             const float2 dxw = f2(wo(k) - wo(-1 - k), wo(1 + k) - wo(-k));
                             const float2 dyw = sub2(wcol[r + R - 1 - k], wcol[r + R + k]);
                             dw = fma2(f2s(stag<R>(k)), add2(dxw, dyw), dw);
                         }
-                        const float byn = btab_at(btab, nbt, 2 * (fs ? ny - j : min(j + 1, ny - j)));
-                        const float byh =
-                            btab_at(btab, nbt, fs ? 2 * (ny - j) - 1 : min(2 * j + 3, 2 * (ny - j) - 1));
                         const int pt = lr * BX + c0;
                         if constexpr (EPI == 3) {
                             // FWI gradient pass: grad += gscale q_v (L u + D w) of X (m = c^2);
@@ -1029,6 +673,33 @@ stage_tma_x2_kernel(const ProblemDev* __restrict__ probs, const int* __restrict_
                         if constexpr (EPI == 2) {
                             // one leap-frog step per column of the pair
                             const float2 c2l = lds2(sc2 + pt);
+                            if (!damped) {
+                                // no damping: w keeps its level n-1 values, u needs no division
+                                const float* pa = spa + pt;
+                                const long long o = (long long)j * ti.pitch + i0;
+                                const float2 dt2 = f2s((float)a.dt * (float)a.dt);
+                                float2 rhs = mul2(c2l, fma2(lap, idx2, mul2(dw, idx1)));
+                                if (j == ti.src_j) {
+                                    if (i0 == ti.src_i) rhs.x += ti.sig;
+                                    if (i0 + 1 == ti.src_i) rhs.y += ti.sig;
+                                }
+                                float2 up;
+                                if (a.m == 2) {
+                                    const float2 dn = fma2(dt2, rhs, lds2(pa + BYv * BX));
+                                    st2(ti.A + ti.fstr + o, dn, in1);
+                                    up = add2(uc, dn);
+                                } else {
+                                    up = fma2(dt2, rhs, fma2(f2s(2.f), uc, mul2(f2s(-1.f), lds2(pa))));
+                                }
+                                float2 wxp = lds2(pa + 2 * BYv * BX), wyp = lds2(pa + 3 * BYv * BX);
+                                if (!wx0in) wxp.x = 0.f;
+                                if (!wx1in) wxp.y = 0.f;
+                                if (j >= ny - 1) wyp = f2s(0.f);
+                                st2(ti.Y + o, up, in1);
+                                st2(ti.Y + 2 * ti.fstr + o, wxp, in1);
+                                st2(ti.Y + 3 * ti.fstr + o, wyp, in1);
+                                continue;
+                            }
                             lf_point(ti, a, spa + pt, BYv * BX, i0, j, uc.x, c2l.x, lap.x, dw.x, dux.x, duy.x,
                                      bxn.x, bxh.x, byn, byh, wp[2].x, wcol[r + R].x);
                             if (in1)
@@ -1039,18 +710,23 @@ stage_tma_x2_kernel(const ProblemDev* __restrict__ probs, const int* __restrict_
                         const float2 xv = lds2(sv + pt), c2 = lds2(sc2 + pt);
                         const float2 xwx = wp[2], xwy = wcol[r + R];
                         // H v = -bx by u + c^2 (lap u / dx^2 + div w / dx) - (bx + by) v
-                        const float2 t = fma2(mul2(bxn, f2s(-byn)), uc, mul2(sub2(f2s(-byn), bxn), xv));
-                        float2 hv = fma2(c2, fma2(lap, idx2, mul2(dw, idx1)), t);
+                        const float2 force = fma2(lap, idx2, mul2(dw, idx1));
+                        const bool wyin = j < ny - 1;
+                        float2 hv, hwx = f2s(0.f), hwy = f2s(0.f);
+                        if (damped) {
+                            const float2 t = fma2(mul2(bxn, f2s(-byn)), uc, mul2(sub2(f2s(-byn), bxn), xv));
+                            hv = fma2(c2, force, t);
+                            hwx = fma2(nbxh, xwx, mul2(mul2(sub2(f2s(byn), bxh), dux), idx1));
+                            if (!wx0in) hwx.x = 0.f;
+                            if (!wx1in) hwx.y = 0.f;
+                            if (wyin) hwy = fma2(f2s(-byh), xwy, mul2(mul2(sub2(bxn, f2s(byh)), duy), idx1));
+                        } else {
+                            hv = mul2(c2, force);
+                        }
                         if (j == ti.src_j) {
                             if (i0 == ti.src_i) hv.x += ti.sig;
                             if (i0 + 1 == ti.src_i) hv.y += ti.sig;
                         }
-                        float2 hwx = fma2(nbxh, xwx, mul2(mul2(sub2(f2s(byn), bxh), dux), idx1));
-                        if (!wx0in) hwx.x = 0.f;
-                        if (!wx1in) hwx.y = 0.f;
-                        const bool wyin = j < ny - 1;
-                        const float2 hwy =
-                            wyin ? fma2(f2s(-byh), xwy, mul2(mul2(sub2(bxn, f2s(byh)), duy), idx1)) : f2s(0.f);
                         const float2 xf[4] = {uc, xv, xwx, xwy};
                         const float2 hf[4] = {xv, hv, hwx, hwy};
                         const long long o = (long long)j * ti.pitch + i0;
@@ -1143,17 +819,20 @@ __device__ __forceinline__ int tma_produce_t(const ProblemDev* __restrict__ prob
     for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x, ++it) {
         const int s = it % NSTv;
         const uint32_t ph = (uint32_t)(it / NSTv) & 1u;
-        if (!mbar_wait(&empty[s], ph ^ 1u, wait_lim)) {
-            *s_err = 1;
-            break;
-        }
+        // (the tile is resolved before the wait, so that a stage set free is refilled at once)
         const int pid = find_problem(tbase, nprob, tile);
         const ProblemDev* P = probs + pid;
         const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(P->tmaps) + mapset * NMAP;
         const int tiles_x = (P->nx + BX - 1) / BX;
         const int lt = tile - __ldg(tbase + pid);
         const int x0 = (lt % tiles_x) * BX, y0 = (lt / tiles_x) * BYv;
-        fill_tile_info(info[s], P, a, x0, y0);
+        TileInfo ti;
+        fill_tile_info(ti, P, a, x0, y0);
+        if (!mbar_wait(&empty[s], ph ^ 1u, wait_lim)) {
+            *s_err = 1;
+            break;
+        }
+        info[s] = ti;
         float* st = smem + (size_t)s * L::FLOATS;
         mbar_expect_tx(&full[s], bytes);
         const int kx = a.x, cx = a.x == 0 ? 0 : a.x - 1;
@@ -1313,6 +992,8 @@ stage_tma_t_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_trigger();
+    pdl_wait();
     const bool has_u = HASU && a.u >= 0, has_a = HASA && a.a >= 0;
     int issued = 0;
     if (warp == NW) {
@@ -1356,31 +1037,38 @@ stage_tma_t_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                     const bool in1 = i0 + 1 < nx;
                     const float* btab = ti.btab;
                     const int nbt = ti.nbtab;
-                    const float2 bxn = f2(btab_at(btab, nbt, 2 * min(i0 + 1, nx - i0)),
-                                          btab_at(btab, nbt, 2 * min(i0 + 2, nx - i0 - 1)));
+                    // Where nothing damps the taps of this thread's points, z_x = z_y = 0 and the
+                    // damping terms vanish (same results to the bit).
+                    const bool damped = ti.xdamp || jt + NR + R >= ny - ti.pml || (!fs && jt - R <= ti.pml);
+                    float2 bxn = f2s(0.f);
                     // bx at the half columns i0 + d + 1/2, d = -4 .. 5 (the z_x taps)
                     float bxh[10];
-#pragma unroll
-                    for (int d = -4; d <= 5; ++d) {
-                        const int p = i0 + d;
-                        bxh[d + 4] = btab_at(btab, nbt, min(2 * p + 3, 2 * (nx - p) - 1));
-                    }
-                    const float2 bxhp = f2(bxh[4], bxh[5]);   // at this thread's two columns
                     unsigned xin = 0u;                           // half columns 0 .. nx - 2
+                    if (damped) {
+                        bxn = f2(btab_at(btab, nbt, 2 * min(i0 + 1, nx - i0)),
+                                 btab_at(btab, nbt, 2 * min(i0 + 2, nx - i0 - 1)));
 #pragma unroll
-                    for (int d = -4; d <= 5; ++d)
-                        if (i0 + d >= 0 && i0 + d < nx - 1) xin |= 1u << (d + 4);
+                        for (int d = -4; d <= 5; ++d) {
+                            const int p = i0 + d;
+                            bxh[d + 4] = btab_at(btab, nbt, min(2 * p + 3, 2 * (nx - p) - 1));
+                            if (p >= 0 && p < nx - 1) xin |= 1u << (d + 4);
+                        }
+                    }
                     // z_v = c^2 y_v and z_y = (bx - by^h) y_wy down this column pair
                     float2 zq[NR + 2 * R], zyq[NR + 2 * R - 1];
 #pragma unroll
                     for (int q = 0; q < NR + 2 * R; ++q)
                         zq[q] = mul2(lds2(zvp + (r0 + q) * L::SW + cs), lds2(c2p + (r0 + q) * L::SW + cs));
+                    if (damped) {
 #pragma unroll
-                    for (int q = 0; q < NR + 2 * R - 1; ++q) {
-                        const int h = ti.y0 + r0 + q - R;
-                        const float bh = btab_at(btab, nbt, fs ? 2 * (ny - h) - 1 : min(2 * h + 3, 2 * (ny - h) - 1));
-                        zyq[q] = (h >= 0 && h < ny - 1) ? mul2(sub2(bxn, f2s(bh)), lds2(wyp + (r0 + q) * BX + c0))
-                                                        : f2s(0.f);
+                        for (int q = 0; q < NR + 2 * R - 1; ++q) {
+                            const int h = ti.y0 + r0 + q - R;
+                            const float bh =
+                                btab_at(btab, nbt, fs ? 2 * (ny - h) - 1 : min(2 * h + 3, 2 * (ny - h) - 1));
+                            zyq[q] = (h >= 0 && h < ny - 1)
+                                         ? mul2(sub2(bxn, f2s(bh)), lds2(wyp + (r0 + q) * BX + c0))
+                                         : f2s(0.f);
+                        }
                     }
                     const bool wx0in = i0 < nx - 1, wx1in = i0 + 1 < nx - 1;
                     const float2 idx1 = f2s(ti.idx1), idx2 = f2s(ti.idx2);
@@ -1389,26 +1077,17 @@ stage_tma_t_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                     for (int r = 0; r < NR; ++r) {
                         const int lr = r0 + r, j = jt + r;
                         if (j >= ny) break;
-                        const float byn = btab_at(btab, nbt, 2 * (fs ? ny - j : min(j + 1, ny - j)));
-                        const float byh =
-                            btab_at(btab, nbt, fs ? 2 * (ny - j) - 1 : min(2 * j + 3, 2 * (ny - j) - 1));
-                        // x taps of z_v (pairs at column offsets -4 .. 5) and y_wx
+                        // x taps of z_v (pairs at column offsets -4 .. 5)
                         const float* zr = zvp + (lr + R) * L::SW + cs;
                         const float* cr = c2p + (lr + R) * L::SW + cs;
                         const float2 zp[5] = {mul2(lds2(zr - 4), lds2(cr - 4)), mul2(lds2(zr - 2), lds2(cr - 2)),
                                               zq[r + R], mul2(lds2(zr + 2), lds2(cr + 2)),
                                               mul2(lds2(zr + 4), lds2(cr + 4))};
                         const float* wr = wxp + lr * L::SW + cs;
-                        const float2 wp[5] = {lds2(wr - 4), lds2(wr - 2), lds2(wr), lds2(wr + 2), lds2(wr + 4)};
                         auto zo = [&](int d) { return ((d + 4) & 1) ? zp[(d + 4) >> 1].y : zp[(d + 4) >> 1].x; };
-                        // z_x at half column offset d: (by - bx^h) y_wx (zero off the w_x grid)
-                        auto xo = [&](int d) {
-                            const float wv = ((d + 4) & 1) ? wp[(d + 4) >> 1].y : wp[(d + 4) >> 1].x;
-                            return ((xin >> (d + 4)) & 1u) ? (byn - bxh[d + 4]) * wv : 0.f;
-                        };
                         const float2 zc = zq[r + R];
                         float2 lap = mul2(f2s(2.f * cent<R>(0)), zc);
-                        float2 gxt = f2s(0.f), gyt = f2s(0.f), dxt = f2s(0.f), dyt = f2s(0.f);
+                        float2 dxt = f2s(0.f), dyt = f2s(0.f);
 #pragma unroll
                         for (int k = 0; k < R; ++k) {
                             const int kk = k + 1;
@@ -1416,8 +1095,6 @@ stage_tma_t_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                                                        : add2(zp[(kk + 4) >> 1], zp[(4 - kk) >> 1]);
                             const float2 sy = add2(zq[r + R + kk], zq[r + R - kk]);
                             lap = fma2(f2s(cent<R>(kk)), add2(sx, sy), lap);
-                            gxt = fma2(f2s(stag<R>(k)), f2(xo(-1 - k) - xo(k), xo(-k) - xo(1 + k)), gxt);
-                            gyt = fma2(f2s(stag<R>(k)), sub2(zyq[r + R + k], zyq[r + R - 1 - k]), gyt);
                             dxt = fma2(f2s(stag<R>(k)), f2(zo(-k) - zo(1 + k), zo(1 - k) - zo(2 + k)), dxt);
                             dyt = fma2(f2s(stag<R>(k)), sub2(zq[r + R + 1 + k], zq[r + R - k]), dyt);
                         }
@@ -1425,18 +1102,39 @@ stage_tma_t_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                         const float2 yv = lds2(zvp + (lr + R) * L::SW + cs);
                         const float2 yu = lds2(yup + pt);
                         const bool wyin = j < ny - 1;
-                        float2 ywx = wp[2];
+                        float2 ywx = lds2(wr);
                         if (!wx0in) ywx.x = 0.f;
                         if (!wx1in) ywx.y = 0.f;
                         const float2 ywy = wyin ? lds2(wyp + (lr + R) * BX + c0) : f2s(0.f);
                         // (H^T y)_u, _v, _wx, _wy
-                        const float2 hu = fma2(mul2(bxn, f2s(-byn)), yv,
-                                               fma2(lap, idx2, mul2(add2(gxt, gyt), idx1)));
-                        const float2 hv = fma2(sub2(f2s(-byn), bxn), yv, yu);
-                        float2 hwx = fma2(dxt, idx1, mul2(f2(-bxhp.x, -bxhp.y), ywx));
+                        float2 hu, hv = yu, hwx, hwy = f2s(0.f);
+                        if (damped) {
+                            const float byn = btab_at(btab, nbt, 2 * (fs ? ny - j : min(j + 1, ny - j)));
+                            const float byh =
+                                btab_at(btab, nbt, fs ? 2 * (ny - j) - 1 : min(2 * j + 3, 2 * (ny - j) - 1));
+                            // z_x at half column offset d: (by - bx^h) y_wx (zero off the w_x grid)
+                            const float2 wp[5] = {lds2(wr - 4), lds2(wr - 2), lds2(wr), lds2(wr + 2), lds2(wr + 4)};
+                            auto xo = [&](int d) {
+                                const float wv = ((d + 4) & 1) ? wp[(d + 4) >> 1].y : wp[(d + 4) >> 1].x;
+                                return ((xin >> (d + 4)) & 1u) ? (byn - bxh[d + 4]) * wv : 0.f;
+                            };
+                            float2 gxt = f2s(0.f), gyt = f2s(0.f);
+#pragma unroll
+                            for (int k = 0; k < R; ++k) {
+                                gxt = fma2(f2s(stag<R>(k)), f2(xo(-1 - k) - xo(k), xo(-k) - xo(1 + k)), gxt);
+                                gyt = fma2(f2s(stag<R>(k)), sub2(zyq[r + R + k], zyq[r + R - 1 - k]), gyt);
+                            }
+                            hu = fma2(mul2(bxn, f2s(-byn)), yv, fma2(lap, idx2, mul2(add2(gxt, gyt), idx1)));
+                            hv = fma2(sub2(f2s(-byn), bxn), yv, yu);
+                            hwx = fma2(dxt, idx1, mul2(f2(-bxh[4], -bxh[5]), ywx));
+                            if (wyin) hwy = fma2(dyt, idx1, mul2(f2s(-byh), ywy));
+                        } else {
+                            hu = mul2(lap, idx2);
+                            hwx = mul2(dxt, idx1);
+                            if (wyin) hwy = mul2(dyt, idx1);
+                        }
                         if (!wx0in) hwx.x = 0.f;
                         if (!wx1in) hwx.y = 0.f;
-                        const float2 hwy = wyin ? fma2(dyt, idx1, mul2(f2s(-byh), ywy)) : f2s(0.f);
                         const float2 xf[4] = {yu, yv, ywx, ywy};
                         const float2 hf[4] = {hu, hv, hwx, hwy};
                         const long long o = (long long)j * ti.pitch + i0;
@@ -1563,25 +1261,18 @@ int build_tensor_maps(std::vector<ProblemDev>& probs, int R, const std::vector<i
     return 0;
 }
 
-// Kernel variants the autotuner chooses from: (tile height, consumer warps, stages).  Variant
-// 4 has no U buffer (4 stages of 64 x 16): passes with a U operand run variant 0 instead.
-// Variant 5 keeps two rows per consumer thread with 20 warps (64 x 20 tiles): 21 warps per
-// SM, which caps a thread at 80 registers (six warps share one scheduler's register file).
-// Variant 6 uses 18 warps (64 x 18 tiles): 19 warps per SM, still 96 registers a thread.
-// Variants 7 to 9 run the column-pair consumers (two columns per thread): 7 = 64 x 18 tiles
-// with 9 warps (two rows a thread), 8 = 64 x 16 with 8 warps (two rows), 9 = 64 x 18 with
-// 18 warps (one row), 10 = 64 x 24 with 12 warps and 2 stages (two rows).  11 and 12 are
-// composite: passes that read an A operand run variant 7, the others (Horner HORK passes,
-// Krylov products, leap-frog-free RK stages without an accumulator) drop the A buffer and
-// take taller tiles: 11 = 64 x 24 with 12 warps and 3 stages, 12 = 64 x 36 with 9 warps, four
-// rows a thread and 2 stages; 13 = 64 x 28 with 14 warps and 3 stages; 14 = 64 x 30 with 15
-// warps and 3 stages (512 threads at 128 registers: the whole register file).  The shape
-// reported for a composite is its no-A shape.
+// Kernel variants the autotuner chooses from: (tile height, consumer warps, stages).  One row a
+// thread where the warps equal the rows, else two (variant 12 four).  Variant 4 has no U buffer
+// (4 stages of 64 x 16): passes with a U operand run variant 0 instead.  11 to 14 are composite:
+// passes that read an A operand run variant 7, the others (Horner HORK passes, Krylov products,
+// leap-frog-free RK stages without an accumulator) drop the A buffer and take taller tiles (14:
+// 512 threads at 128 registers, the whole register file).  The shape reported for a composite is
+// its no-A shape.
 struct TmaVariant {
     int by, nw, nst;
 };
 constexpr TmaVariant kVariants[TMA_NUM_VARIANTS] = {
-    {16, 16, 3}, {16, 8, 3}, {8, 8, 5},  {8, 16, 5},  {16, 16, 4}, {20, 20, 3}, {18, 18, 3},
+    {16, 16, 3}, {16, 8, 3}, {8, 8, 5},  {8, 4, 5},  {16, 16, 4}, {20, 10, 3}, {18, 18, 3},
     {18, 9, 3},  {16, 8, 3}, {18, 18, 3}, {24, 12, 2}, {24, 12, 3}, {36, 9, 2}, {28, 14, 3}, {30, 15, 3}};
 
 static bool composite(int v) { return v >= 11 && v <= 14; }
@@ -1600,26 +1291,6 @@ void tma_variant_describe(int v, int* by, int* nw, int* nst) {
 
 static int g_num_sms = 0;
 
-template <int R, int BYv, int NW, int NSTv, int EPI, bool HASU = true>
-static int launch_variant(const ProblemDev* probs, const int* tbase, int nprob, int ntiles,
-                          const StageArgs& a, int* err, cudaStream_t s) {
-    const size_t smem = (size_t)NSTv * StageLayout<R, BYv, HASU>::BYTES + 1024;
-    // the shared-memory attribute is set once per instantiation and device
-    static unsigned long long configured = 0;
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return -1;
-    if (!(configured >> dev & 1ull)) {
-        if (cudaFuncSetAttribute(stage_tma_kernel<R, BYv, NW, NSTv, EPI, HASU>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return -1;
-        configured |= 1ull << dev;
-    }
-    const int grid = ntiles < g_num_sms ? ntiles : g_num_sms;
-    stage_tma_kernel<R, BYv, NW, NSTv, EPI, HASU><<<grid, NW * 32 + 32, smem, s>>>(
-        probs, tbase, nprob, ntiles, map_set_of(BYv), a, err);
-    return 0;
-}
-
 template <int R, int BYv, int NW, int NSTv, int EPI, bool HASA = true, bool HASU = true>
 static int launch_x2(const ProblemDev* probs, const int* tbase, int nprob, int ntiles, const StageArgs& a,
                      int* err, cudaStream_t s) {
@@ -1637,9 +1308,8 @@ static int launch_x2(const ProblemDev* probs, const int* tbase, int nprob, int n
         configured |= 1ull << dev;
     }
     const int grid = ntiles < g_num_sms ? ntiles : g_num_sms;
-    stage_tma_x2_kernel<R, BYv, NW, NSTv, EPI, HASU, HASA><<<grid, NW * 32 + 32, smem, s>>>(
-        probs, tbase, nprob, ntiles, map_set_of(BYv), a, err);
-    return 0;
+    return launch_pdl(stage_tma_x2_kernel<R, BYv, NW, NSTv, EPI, HASU, HASA>, grid, NW * 32 + 32, smem, s, probs, tbase,
+                      nprob, ntiles, map_set_of(BYv), a, err);
 }
 
 // One leap-frog step (EPI 2) on the column-pair consumers (64 x 30 tiles, 15 warps, 3
@@ -1691,10 +1361,10 @@ int launch_grad_tma(int R, const ProblemDev* probs, const int* tbase, int nprob,
     return -1;
 }
 
-template <int R, bool HASU, bool HASA>
+template <int R, int BYv, int NW, int NSTv, bool HASU, bool HASA>
 static int launch_t(const ProblemDev* probs, const int* tbase, int nprob, int ntiles, const StageArgs& a, int* err,
                     cudaStream_t s) {
-    constexpr int BYv = 18, NW = 9, NSTv = 3;
+    static_assert(map_set_of(BYv) >= 0, "tile height without a map set");
     const size_t smem = (size_t)NSTv * TLayout<R, BYv, HASU, HASA>::BYTES + 1024;
     static unsigned long long configured = 0;
     int dev = 0;
@@ -1706,13 +1376,15 @@ static int launch_t(const ProblemDev* probs, const int* tbase, int nprob, int nt
         configured |= 1ull << dev;
     }
     const int grid = ntiles < g_num_sms ? ntiles : g_num_sms;
-    stage_tma_t_kernel<R, BYv, NW, NSTv, HASU, HASA><<<grid, NW * 32 + 32, smem, s>>>(
-        probs, tbase, nprob, ntiles, map_set_of(BYv), a, err);
-    return 0;
+    return launch_pdl(stage_tma_t_kernel<R, BYv, NW, NSTv, HASU, HASA>, grid, NW * 32 + 32, smem, s, probs, tbase, nprob,
+                      ntiles, map_set_of(BYv), a, err);
 }
 
-// The transposed pass H^T (FP32, no dot partner, no gradient) on 64 x 18 tiles with 9
-// column-pair consumer warps; tbase and ntiles are those of the 18-row map set.
+// The transposed pass H^T (FP32, no gradient) on the column-pair consumers, two rows a thread.  The
+// tile is as tall as three stages fit shared memory, since the consumer warps hide the latency:
+// 64 x 18 with 9 warps for a pass with a U and an A operand, 64 x 24 with 12 for one of them, 64 x
+// 30 with 15 for the plain product; tbase and ntiles are those of that height's map set.
+int tma_transpose_height(bool reads_u, bool reads_a) { return reads_u && reads_a ? 18 : reads_u || reads_a ? 24 : 30; }
 int launch_transpose_tma(int R, const ProblemDev* probs, const int* tbase, int nprob, int ntiles,
                          const StageArgs& a_in, int* err, cudaStream_t s) {
     if (ntiles <= 0) return nprob > 0 ? -1 : 0;
@@ -1733,16 +1405,18 @@ int launch_transpose_tma(int R, const ProblemDev* probs, const int* tbase, int n
     a.fcay = (float)a.cay;
     a.fcax = (float)a.cax;
     const bool hu = a.u >= 0, ha = a.a >= 0;
-    if (R == 4)
-        return hu ? (ha ? launch_t<4, true, true>(probs, tbase, nprob, ntiles, a, err, s)
-                        : launch_t<4, true, false>(probs, tbase, nprob, ntiles, a, err, s))
-                  : (ha ? launch_t<4, false, true>(probs, tbase, nprob, ntiles, a, err, s)
-                        : launch_t<4, false, false>(probs, tbase, nprob, ntiles, a, err, s));
-    if (R == 2)
-        return hu ? (ha ? launch_t<2, true, true>(probs, tbase, nprob, ntiles, a, err, s)
-                        : launch_t<2, true, false>(probs, tbase, nprob, ntiles, a, err, s))
-                  : (ha ? launch_t<2, false, true>(probs, tbase, nprob, ntiles, a, err, s)
-                        : launch_t<2, false, false>(probs, tbase, nprob, ntiles, a, err, s));
+    if (R == 4) {
+        if (hu && ha) return launch_t<4, 18, 9, 3, true, true>(probs, tbase, nprob, ntiles, a, err, s);
+        if (hu) return launch_t<4, 24, 12, 3, true, false>(probs, tbase, nprob, ntiles, a, err, s);
+        if (ha) return launch_t<4, 24, 12, 3, false, true>(probs, tbase, nprob, ntiles, a, err, s);
+        return launch_t<4, 30, 15, 3, false, false>(probs, tbase, nprob, ntiles, a, err, s);
+    }
+    if (R == 2) {
+        if (hu && ha) return launch_t<2, 18, 9, 3, true, true>(probs, tbase, nprob, ntiles, a, err, s);
+        if (hu) return launch_t<2, 24, 12, 3, true, false>(probs, tbase, nprob, ntiles, a, err, s);
+        if (ha) return launch_t<2, 24, 12, 3, false, true>(probs, tbase, nprob, ntiles, a, err, s);
+        return launch_t<2, 30, 15, 3, false, false>(probs, tbase, nprob, ntiles, a, err, s);
+    }
     return -1;
 }
 
@@ -1767,60 +1441,33 @@ int launch_stage_tma(int variant, int R, const ProblemDev* probs, const int* tba
     }
     // the steady-state Faber / HORK form: Y = cu U + cx X + ch H, ACC = ca A + cay Y
     const bool epi = a.ck == 1.0 && a.cau == 0.0 && a.cak == 0.0 && a.cax == 0.0;
-#define EWV_TMA_CASE(V, RR, BYV, NWV, NSTV) \
-    if (variant == V && R == RR)                                                                \
-        return epi ? launch_variant<RR, BYV, NWV, NSTV, 1>(probs, tbase, nprob, ntiles, a, err, s) \
-                   : launch_variant<RR, BYV, NWV, NSTV, 0>(probs, tbase, nprob, ntiles, a, err, s);
-    EWV_TMA_CASE(0, 4, 16, 16, 3)
-    EWV_TMA_CASE(1, 4, 16, 8, 3)
-    EWV_TMA_CASE(2, 4, 8, 8, 5)
-    EWV_TMA_CASE(3, 4, 8, 16, 5)
-    EWV_TMA_CASE(5, 4, 20, 20, 3)
-    EWV_TMA_CASE(6, 4, 18, 18, 3)
-#define EWV_TMA_X2_CASE(V, RR, BYV, NWV, NSTV) \
-    if (variant == V && R == RR)                                                             \
-        return epi ? launch_x2<RR, BYV, NWV, NSTV, 1>(probs, tbase, nprob, ntiles, a, err, s) \
-                   : launch_x2<RR, BYV, NWV, NSTV, 0>(probs, tbase, nprob, ntiles, a, err, s);
     if (composite(variant) && a.a >= 0) variant = 7;   // composite, pass with A
-#define EWV_TMA_X2_NOA_CASE(V, RR, BYV, NWV, NSTV) \
-    if (variant == V && R == RR)                                                                    \
-        return epi ? launch_x2<RR, BYV, NWV, NSTV, 1, false>(probs, tbase, nprob, ntiles, a, err, s) \
-                   : launch_x2<RR, BYV, NWV, NSTV, 0, false>(probs, tbase, nprob, ntiles, a, err, s);
-    EWV_TMA_X2_CASE(7, 4, 18, 9, 3)
-    EWV_TMA_X2_CASE(8, 4, 16, 8, 3)
-    EWV_TMA_X2_CASE(9, 4, 18, 18, 3)
-    EWV_TMA_X2_CASE(10, 4, 24, 12, 2)
-    EWV_TMA_X2_NOA_CASE(11, 4, 24, 12, 3)
-    EWV_TMA_X2_NOA_CASE(12, 4, 36, 9, 2)
-    EWV_TMA_X2_NOA_CASE(13, 4, 28, 14, 3)
-    EWV_TMA_X2_NOA_CASE(14, 4, 30, 15, 3)
-    EWV_TMA_X2_CASE(7, 2, 18, 9, 3)
-    EWV_TMA_X2_CASE(8, 2, 16, 8, 3)
-    EWV_TMA_X2_CASE(9, 2, 18, 18, 3)
-    EWV_TMA_X2_CASE(10, 2, 24, 12, 2)
-    EWV_TMA_X2_NOA_CASE(11, 2, 24, 12, 3)
-    EWV_TMA_X2_NOA_CASE(12, 2, 36, 9, 2)
-    EWV_TMA_X2_NOA_CASE(13, 2, 28, 14, 3)
-    EWV_TMA_X2_NOA_CASE(14, 2, 30, 15, 3)
-#undef EWV_TMA_X2_NOA_CASE
-#undef EWV_TMA_X2_CASE
-    if (variant == 4) {   // no U buffer; a pass with a U operand runs variant 0
-        if (a.u >= 0) variant = 0;
-        else if (R == 4)
-            return epi ? launch_variant<4, 16, 16, 4, 1, false>(probs, tbase, nprob, ntiles, a, err, s)
-                       : launch_variant<4, 16, 16, 4, 0, false>(probs, tbase, nprob, ntiles, a, err, s);
-        else
-            return epi ? launch_variant<2, 16, 16, 4, 1, false>(probs, tbase, nprob, ntiles, a, err, s)
-                       : launch_variant<2, 16, 16, 4, 0, false>(probs, tbase, nprob, ntiles, a, err, s);
-    }
-    EWV_TMA_CASE(0, 4, 16, 16, 3)
-    EWV_TMA_CASE(0, 2, 16, 16, 3)
-    EWV_TMA_CASE(1, 2, 16, 8, 3)
-    EWV_TMA_CASE(2, 2, 8, 8, 5)
-    EWV_TMA_CASE(3, 2, 8, 16, 5)
-    EWV_TMA_CASE(5, 2, 20, 20, 3)
-    EWV_TMA_CASE(6, 2, 18, 18, 3)
+    if (variant == 4 && a.u >= 0) variant = 0;         // no U buffer
+    // the shapes that repeat another one's
+    if (variant == 1) variant = 8;
+    if (variant == 6) variant = 9;
+#define EWV_TMA_CASE2(V, RR, BYV, NWV, NSTV, HASA, HASU)                                                   \
+    if (variant == V && R == RR)                                                                         \
+        return epi ? launch_x2<RR, BYV, NWV, NSTV, 1, HASA, HASU>(probs, tbase, nprob, ntiles, a, err, s) \
+                   : launch_x2<RR, BYV, NWV, NSTV, 0, HASA, HASU>(probs, tbase, nprob, ntiles, a, err, s);
+#define EWV_TMA_CASE(V, BYV, NWV, NSTV, HASA, HASU)  \
+    EWV_TMA_CASE2(V, 4, BYV, NWV, NSTV, HASA, HASU) \
+    EWV_TMA_CASE2(V, 2, BYV, NWV, NSTV, HASA, HASU)
+    EWV_TMA_CASE(0, 16, 16, 3, true, true)
+    EWV_TMA_CASE(2, 8, 8, 5, true, true)
+    EWV_TMA_CASE(3, 8, 4, 5, true, true)
+    EWV_TMA_CASE(4, 16, 16, 4, true, false)
+    EWV_TMA_CASE(5, 20, 10, 3, true, true)
+    EWV_TMA_CASE(7, 18, 9, 3, true, true)
+    EWV_TMA_CASE(8, 16, 8, 3, true, true)
+    EWV_TMA_CASE(9, 18, 18, 3, true, true)
+    EWV_TMA_CASE(10, 24, 12, 2, true, true)
+    EWV_TMA_CASE(11, 24, 12, 3, false, true)
+    EWV_TMA_CASE(12, 36, 9, 2, false, true)
+    EWV_TMA_CASE(13, 28, 14, 3, false, true)
+    EWV_TMA_CASE(14, 30, 15, 3, false, true)
 #undef EWV_TMA_CASE
+#undef EWV_TMA_CASE2
     return -1;
 }
 
