@@ -2979,8 +2979,38 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
         launch_stage(prec, R, tb, E->d_adj, d_tp, sa, s);
         ++m->launches;
     };
+    // Faber and HORK adjoints in FP32: the forward recompute stores G(p_{j-1}) = L u + D w, the
+    // factor of the gradient, instead of the four fields of p_{j-1} (a pass has it anyway), and the
+    // transposed pass adds q_v G to the gradient while it reads q: no gradient pass, which
+    // recomputed the stencil from the stored vectors, and a tape of m fields instead of 4 m (the 16
+    // shots of 401 x 201 at m = 20: 103 MB, which the L2 cache holds, instead of 413 MB).
+    // Tape field i: field i % 4 of workspace vector 3 + i / 4; the recompute alternates between
+    // vectors 1 and 2.  (deg >= 4: below, those vectors would meet the cotangents'.)
+    const bool use_tape = tma_adj && deg >= 4 && (method == EWV_METHOD_FABER || method == EWV_METHOD_HORK);
+    bool tape_failed = false;
+    auto tape_pass = [&](StageArgs sa, int i) {
+        const int v = tma_tape_variant(E->tma_variant);
+        const int set = tma_map_set(tma_variant_tile_height_for(v, false));
+        sa.tape_vec = 3 + i / 4;
+        sa.tape_field = i % 4;
+        if (launch_stage_tma(v, R, E->d_adj, E->d_tbase + (size_t)set * (E->nprob + 1), ns, E->ntiles_by[set], sa,
+                             E->d_err, s) != 0)
+            tape_failed = true;
+        ++m->launches;
+    };
+    auto reverse_pass = [&](StageArgs sa, int i) {
+        const int set = tma_map_set(tma_transpose_height(sa.u >= 0, sa.a >= 0));
+        sa.tape_vec = 3 + i / 4;
+        sa.tape_field = i % 4;
+        sa.grad = grad;
+        if (launch_transpose_tma(R, E->d_adj, E->d_tbase + (size_t)set * (E->nprob + 1), ns, E->ntiles_by[set], sa,
+                                 E->d_err, s) != 0)
+            tape_failed = true;
+        ++m->launches;
+    };
     // launch errors, and the TMA pipeline's timeout flag when it ran
     auto adj_finish = [&]() {
+        if (tape_failed) return fail(m->err, EWV_ERR_CUDA, "an adjoint pass could not be launched");
         int rc2 = check_launch(m->err);
         if (rc2 != EWV_OK || !tma_adj) return rc2;
         int herr = 0;
@@ -3026,6 +3056,35 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
         launch_set_clock(E->d_adj, ns, t, dt, s);
         launch_prologue(E->d_adj, ns, 3 /* HORK */, deg, 0.0, 0.0, 0.0, s);
         m->launches += 2;
+        if (use_tape) {
+            auto kbuf = [](int i) { return 1 + (i & 1); };      // k_i: vectors 1 and 2 alternate
+            for (int i = 1; i <= deg; ++i) {
+                StageArgs sa = stage_defaults();
+                sa.x = kbuf(i - 1);
+                sa.y_out = i < deg ? kbuf(i) : -1;
+                sa.src_slot = i - 1;
+                sa.cx = 1.0;
+                sa.ch = dt;
+                sa.ck = 1.0;
+                tape_pass(sa, i - 1);
+            }
+            auto rbuf = [&](int k) { return k == 0 ? 0 : deg + 1 + ((deg - 1 - k) % 2); };
+            for (int i = deg; i >= 1; --i) {
+                const double sc = (i == deg) ? w(deg) : 1.0;
+                StageArgs tr = stage_defaults();
+                tr.transpose = 1;
+                tr.x = (i == deg) ? 0 : rbuf(i);
+                tr.cx = sc;
+                tr.ch = dt * sc;
+                tr.a = 0;
+                tr.ca = w(i - 1);
+                tr.cak = 1.0;
+                tr.acc_out = rbuf(i - 1);
+                tr.gscale = dt * sc;
+                reverse_pass(tr, i - 1);
+            }
+            return adj_finish();
+        }
         for (int j = 1; j <= deg - 1; ++j) {
             StageArgs sa = stage_defaults();
             sa.x = j;
@@ -3086,6 +3145,24 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
     launch_set_clock(E->d_adj, ns, t, dt, s);
     launch_prologue(E->d_adj, ns, 1 /* Faber */, deg, g, c0, c1, s);
     m->launches += 2;
+    if (use_tape) {
+        // p_j over p_{j-2}, as in the forward step
+        auto pbuf = [](int j) { return 1 + (j & 1); };
+        for (int j = 1; j <= deg; ++j) {
+            StageArgs sa = stage_defaults();
+            sa.x = pbuf(j - 1);
+            if (j < deg) {
+                sa.u = j >= 2 ? pbuf(j) : -1;
+                sa.y_out = pbuf(j);
+            }
+            sa.src_slot = j - 1;
+            sa.cx = -c0;
+            sa.ch = 1.0 / g;
+            sa.cu = -cprime(j);
+            sa.ck = 1.0;
+            tape_pass(sa, j - 1);
+        }
+    } else {
     // recompute the forward vectors p_1..p_{m-1} of this step into the tape (T_k = vector k+1)
     for (int j = 1; j <= deg - 1; ++j) {
         StageArgs sa = stage_defaults();
@@ -3099,16 +3176,20 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
         sa.ck = 1.0;
         stage(sa);
     }
+    }
     // reverse recurrence; ybar is vector 0, q_{m-k} lives in Q[(k-1) % 3] (vectors m+1..m+3)
     auto qbuf = [&](int jj) { return jj == 0 ? 0 : deg + 1 + ((deg - jj - 1) % 3); };
     for (int j = deg; j >= 1; --j) {
         // gradient: (1/gamma) q_{j,v} G(p_{j-1}); q_m = a_m ybar is not stored
-        StageArgs gr = stage_defaults();
-        gr.x = j;                              // T_{j-1}
-        gr.grad = grad;
-        gr.gq = (j == deg) ? 0 : qbuf(j);
-        gr.gscale = (j == deg) ? a[deg] / g : 1.0 / g;
-        stage(gr);
+        const double gscale = (j == deg) ? a[deg] / g : 1.0 / g;
+        if (!use_tape) {
+            StageArgs gr = stage_defaults();
+            gr.x = j;                          // T_{j-1}
+            gr.grad = grad;
+            gr.gq = (j == deg) ? 0 : qbuf(j);
+            gr.gscale = gscale;
+            stage(gr);
+        }
         // q_{j-1} = a_{j-1} ybar + B^T q_j - c'_{j+1} q_{j+1}
         StageArgs tr = stage_defaults();
         tr.transpose = 1;
@@ -3134,7 +3215,12 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
         }
         // degree 1: q_0 cannot overwrite ybar while ybar is read with a halo
         tr.acc_out = (j == 1 && deg == 1) ? deg + 1 : qbuf(j - 1);
-        stage(tr);
+        if (use_tape) {
+            tr.gscale = gscale;
+            reverse_pass(tr, j - 1);
+        } else {
+            stage(tr);
+        }
     }
     if (deg == 1) {
         PointArgs pa{};

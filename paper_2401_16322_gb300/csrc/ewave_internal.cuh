@@ -129,6 +129,9 @@ struct StageArgs {
     void* grad;                      // gradient mode: grad += gscale q_v G(X), per-shot fields
     int gq;                          // vector index of q (its v field is read)
     double gscale;
+    // gradient tape (2D TMA passes): field tape_field of workspace vector tape_vec.  A forward pass
+    // writes L u + D w of X there; a transposed pass with grad set adds gscale X_v times it to grad.
+    int tape_vec, tape_field;
     int terms;                       // plain kernels: which coefficients are not 0 or 1 (set at launch)
     int store_bf16;                  // 1: round every stored Y / ACC value to bfloat16 (RN)
     // FP32 copies of cx .. cax, filled by the FP32 TMA launcher (the kernel reads them from
@@ -216,6 +219,7 @@ int launch_transpose_tma(int R, const ProblemDev* probs, const int* tbase, int n
 int launch_stage_tma(int variant, int R, const ProblemDev* probs, const int* tbase, int nprob,
                      int ntiles, const StageArgs& a, int* err, cudaStream_t s);
 int tma_variant_tile_height(int v);
+int tma_tape_variant(int v);   // the variant that writes a gradient tape when v is selected (column pairs)
 // Tile height of variant v for a pass that does (reads_a) or does not read an A operand
 // (composite variants pick their tile by it).
 int tma_variant_tile_height_for(int v, bool reads_a);

@@ -58,6 +58,8 @@ struct StageLayout {
 struct __align__(16) TileInfo {
     float* Y;
     float* A;
+    float* T;                // field of the gradient tape (adjoint steps), or null
+    float* G;                // this shot's gradient field, or null
     long long fstr;
     int x0, y0, nx, ny, pitch, pml, fs, src_i, src_j, shot;
     float beta0, inv_pml, idx1, idx2, sig, xs;   // xs: per-problem scale of H X (Krylov)
@@ -248,6 +250,10 @@ __device__ __forceinline__ void fill_tile_info(TileInfo& ti, const ProblemDev* P
     ti.A = a.acc_out >= 0 ? (a.acc_out == 0 ? (float*)P->state
                                             : (float*)P->work + (long long)(a.acc_out - 1) * P->vec_stride)
                           : nullptr;
+    ti.T = a.tape_vec > 0 ? (float*)P->work + (long long)(a.tape_vec - 1) * P->vec_stride +
+                                (long long)a.tape_field * P->field_stride
+                          : nullptr;
+    ti.G = a.grad ? (float*)a.grad + (long long)P->shot * P->field_stride : nullptr;
     ti.fstr = P->field_stride;
     ti.x0 = x0;
     ti.y0 = y0;
@@ -483,6 +489,7 @@ __device__ __forceinline__ void tma_point_scalar(const float* st, const TileInfo
         return;
     }
     const float idx1 = ti.idx1, idx2 = ti.idx2;
+    if (ti.T) ti.T[(long long)j * ti.pitch + i] = (uxx + uyy) * idx2 + (dwx + dwy) * idx1;
     const float xu = uc, xv = sv[pt], xwx = wxrow[0], xwy = wcolv(R);
     float hv = -bxn * byn * xu + sc2[pt] * ((uxx + uyy) * idx2 + (dwx + dwy) * idx1) - (bxn + byn) * xv;
     if (i == ti.src_i && j == ti.src_j) hv += ti.sig;
@@ -711,6 +718,8 @@ stage_tma_x2_kernel(const ProblemDev* __restrict__ probs, const int* __restrict_
                         const float2 xwx = wp[2], xwy = wcol[r + R];
                         // H v = -bx by u + c^2 (lap u / dx^2 + div w / dx) - (bx + by) v
                         const float2 force = fma2(lap, idx2, mul2(dw, idx1));
+                        // tape pass of an adjoint step: L u + D w, the gradient's factor of this vector
+                        if (ti.T) st2(ti.T + (long long)j * ti.pitch + i0, force, in1);
                         const bool wyin = j < ny - 1;
                         float2 hv, hwx = f2s(0.f), hwy = f2s(0.f);
                         if (damped) {
@@ -962,7 +971,9 @@ __device__ __forceinline__ void tma_point_scalar_t(const float* st, const TileIn
         uv[f] = has_u ? st[L::PU_OFF + f * BYv * BX + pt] : 0.f;
         av[f] = has_a ? st[L::PA_OFF + f * BYv * BX + pt] : 0.f;
     }
-    tma_epilogue_point(ti, a, (long long)j * ti.pitch + i, xf, hf, uv, av, i >= nx - 1, j >= ny - 1);
+    const long long o = (long long)j * ti.pitch + i;
+    if (ti.T) ti.G[o] += (float)a.gscale * yv * ti.T[o];
+    tma_epilogue_point(ti, a, o, xf, hf, uv, av, i >= nx - 1, j >= ny - 1);
 }
 
 template <int R, int BYv, int NW, int NSTv, bool HASU, bool HASA>
@@ -1101,6 +1112,18 @@ stage_tma_t_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                         const int pt = lr * BX + c0;
                         const float2 yv = lds2(zvp + (lr + R) * L::SW + cs);
                         const float2 yu = lds2(yup + pt);
+                        if (ti.T) {
+                            // grad += gscale y_v (L u + D w), the factor from the step's tape
+                            const long long o = (long long)j * ti.pitch + i0;
+                            const float2 gy = mul2(f2s((float)a.gscale), yv);
+                            if (in1) {
+                                const float2 g = *reinterpret_cast<const float2*>(ti.T + o);
+                                float2* G = reinterpret_cast<float2*>(ti.G + o);
+                                *G = add2(*G, mul2(gy, g));
+                            } else {
+                                ti.G[o] += gy.x * ti.T[o];
+                            }
+                        }
                         const bool wyin = j < ny - 1;
                         float2 ywx = lds2(wr);
                         if (!wx0in) ywx.x = 0.f;
@@ -1283,6 +1306,7 @@ int tma_variant_tile_height_for(int v, bool reads_a) {
 }
 
 int tma_variant_tile_height(int v) { return kVariants[v].by; }
+int tma_tape_variant(int v) { return v >= 7 ? v : 14; }
 void tma_variant_describe(int v, int* by, int* nw, int* nst) {
     *by = kVariants[v].by;
     *nw = kVariants[v].nw;
@@ -1433,6 +1457,7 @@ int launch_stage_tma(int variant, int R, const ProblemDev* probs, const int* tba
     a.fcay = (float)a.cay;
     a.fcax = (float)a.cax;
     if (ntiles <= 0) return nprob > 0 ? -1 : 0;   // problems but no tiles: inconsistent lists
+    if (a.tape_vec > 0 && (tma_tape_variant(variant) != variant || a.a >= 0)) return -1;
     if (!g_num_sms) {
         int dev = 0;
         cudaGetDevice(&dev);
