@@ -47,8 +47,57 @@ __device__ __forceinline__ void fma16(double2& acc, double c, const double2& q) 
     acc.x = fma(c, q.x, acc.x);
     acc.y = fma(c, q.y, acc.y);
 }
-// dot product of one 16-byte vector, widened to FP64 for the accumulation
-__device__ __forceinline__ double dotv(const float4& a, const float4& b) { return (double)dot16(a, b); }
-__device__ __forceinline__ double dotv(const double2& a, const double2& b) { return dot16d(a, b); }
+// hi + lo += x, the rounding of hi + x kept in lo (Knuth's TwoSum)
+__device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
+    const float s = hi + x;
+    const float b = s - hi;
+    lo += (hi - (s - b)) + (x - b);
+    hi = s;
+}
+
+// Sum of dot products of 16-byte vectors.  FP64 vectors: an FP64 sum.  FP32 vectors: the products
+// of four elements are added in FP32 (dot16), those sums accumulated as an unevaluated pair of
+// FP32 numbers (48 bits) that is widened to FP64 once: an FP64 conversion and addition for every
+// 16 bytes would occupy the FP64 pipe (16 cycles each) longer than memory takes to deliver them.
+template <typename V>
+struct DotSum;
+template <>
+struct DotSum<double2> {
+    double s = 0.0;
+    __device__ __forceinline__ void add(const double2& a, const double2& b) { s += dot16d(a, b); }
+    // sum over the warp, valid on lane 0
+    __device__ __forceinline__ double warp_total() const {
+        double v = s;
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        return v;
+    }
+};
+template <>
+struct DotSum<float4> {
+    float hi = 0.f, lo = 0.f;
+    __device__ __forceinline__ void add(const float4& a, const float4& b) { two_sum_add(hi, lo, dot16(a, b)); }
+    __device__ __forceinline__ double warp_total() const {
+        float h = hi, l = lo;
+        for (int o = 16; o > 0; o >>= 1) {
+            const float oh = __shfl_down_sync(0xffffffffu, h, o), ol = __shfl_down_sync(0xffffffffu, l, o);
+            two_sum_add(h, l, oh);
+            l += ol;
+        }
+        return (double)h + (double)l;
+    }
+};
+// Block-wide total (fixed order), valid on thread 0; red: one double per warp.  Called by all threads.
+template <typename V>
+__device__ __forceinline__ double block_total(const DotSum<V>& d, double* red) {
+    const int tid = threadIdx.y * blockDim.x + threadIdx.x;
+    const double w = d.warp_total();
+    if ((tid & 31) == 0) red[tid >> 5] = w;
+    __syncthreads();
+    double s = 0.0;
+    if (tid == 0)
+        for (int i = 0; i < NTHREADS / 32; ++i) s += red[i];
+    __syncthreads();
+    return s;
+}
 
 }  // namespace ewv

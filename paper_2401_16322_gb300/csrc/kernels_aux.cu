@@ -405,24 +405,24 @@ point_flat_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
         }
         return;
     }
-    double accd = 0.0;
+    DotSum<V> acc;
     if (pa.mode == 0) {
         const V* Q = reinterpret_cast<const V*>(vptr<T>(P, 0));
         for (long long q = q0 + tid; q < q1; q += NTHREADS) {
             const V a = Q[q];
-            accd += dotv(a, a);
+            acc.add(a, a);
         }
     } else if (pa.mode == 7) {
         const V* W = reinterpret_cast<const V*>(vptr<T>(P, pa.j));      // slot j+1
         for (long long q = q0 + tid; q < q1; q += NTHREADS) {
             const V w = W[q];
-            accd += dotv(w, w);
+            acc.add(w, w);
         }
     } else if (pa.mode == 5) {
         // <q_{j+1}, q_k> after the matrix-vector product (its finalisation is FIN_MATVEC)
         const V* W = reinterpret_cast<const V*>(vptr<T>(P, pa.j));      // slot j+1
         const V* D = reinterpret_cast<const V*>(vptr<T>(P, pa.k - 1));  // slot k
-        for (long long q = q0 + tid; q < q1; q += NTHREADS) accd += dotv(W[q], D[q]);
+        for (long long q = q0 + tid; q < q1; q += NTHREADS) acc.add(W[q], D[q]);
     } else {
         V* W = reinterpret_cast<V*>(vptr<T>(P, pa.j));                  // slot j+1
         const V* Qk = reinterpret_cast<const V*>(vptr<T>(P, pa.k - 1));   // slot k
@@ -436,11 +436,11 @@ point_flat_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
             const V qn = Qn ? Qn[q] : V{};
             const V w = axpy16(wq, coef, qk);
             W[q] = w;
-            accd += dotv(w, Qn ? qn : w);
+            acc.add(w, Qn ? qn : w);
         }
     }
     if (pa.mode == 1 && pa.k == pa.j && pa.j == pa.m) return;   // h_{m+1,m} unused
-    const double bsum = block_sum_fixed(accd, red);
+    const double bsum = block_total(acc, red);
     StageArgs a{};
     a.fin_mode = pa.mode == 0 ? (pa.notail == 2 ? FIN_NORM0_TAIL : pa.notail ? FIN_NORM0_NOTAIL : FIN_NORM0)
                : pa.mode == 7 ? FIN_STORE_NORM

@@ -47,14 +47,6 @@ constexpr int GS_VPT = PCHUNK / 4 / NTHREADS;   // 16-byte vectors of a chunk pe
 constexpr int GS_BATCH = NTHREADS / 32 / 2;     // basis vectors per reduction (two sums each, one per warp)
 static_assert(GS_VPT * 4 * NTHREADS == PCHUNK, "a chunk is a whole number of vectors per thread");
 
-// s + e = a + b exactly (Knuth)
-__device__ __forceinline__ void two_sum_add(float& hi, float& lo, float x) {
-    const float s = hi + x;
-    const float b = s - hi;
-    lo += (hi - (s - b)) + (x - b);
-    hi = s;
-}
-
 // The chunk of this block: its problem and 16-byte vectors [q0, q1).
 struct Chunk {
     int pid, slot, base, count;
@@ -247,13 +239,13 @@ gs_update_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ p
 #pragma unroll
         for (int i = 0; i < GS_VPT; ++i) w[i] = axpy16(w[i], h, v[i]);
     }
-    double acc = 0.0;
+    DotSum<float4> acc;
 #pragma unroll
     for (int i = 0; i < GS_VPT; ++i) {
         if (tid + i * NTHREADS < c.n) W[c.q0 + tid + i * NTHREADS] = w[i];
-        acc += dotv(w[i], w[i]);
+        acc.add(w[i], w[i]);
     }
-    const double bsum = block_sum_fixed(acc, red);
+    const double bsum = block_total(acc, red);
     StageArgs a{};
     a.fin_mode = FIN_MGS;
     a.fin_j = j;

@@ -14,8 +14,10 @@
 //
 // Layout: block b owns the flat passes' chunks b cpb .. b cpb + cpb - 1 (PCHUNK elements of one
 // problem's padded vector each, found through the chunk table), with the same thread-to-element
-// mapping, the same per-chunk partial sums and the same fixed-order totals as the flat passes,
-// so both forms give the same values bit for bit.  Each step's partials go to a buffer of
+// mapping, the same per-chunk partial sums and totals to FP64 rounding as the flat passes: the
+// FP32 vectors agree bit for bit.  What a step costs besides its two vectors is FP64 work, at 16
+// cycles a warp instruction: FP32 sums are carried as FP32 pairs, and one warp per block forms
+// the totals and the tails (a lane per entry).  Each step's partials go to a buffer of
 // their own (two, alternating), a grid barrier makes them visible, and every block sums its
 // problems' partials and replays the scalar recurrence on a private copy of tail_{j+1} and of
 // column j of H; the block that owns a problem's chunk 0 writes the results back.
@@ -80,13 +82,17 @@ __device__ bool grid_barrier(unsigned int* bar, unsigned int nblocks, unsigned l
     return *s_ok != 0;
 }
 
-// Fixed-order total of a problem's partials (the order of partial_and_finalize_at); valid on
-// thread 0.
-__device__ __forceinline__ double problem_total(const double* partials, int base, int count, double* red,
-                                               int tid) {
+// Fixed-order total of a problem's partials, by one warp; valid on every lane.
+__device__ __forceinline__ double problem_total(const double* partials, int base, int count, int lane) {
     double v = 0.0;
-    for (int t = tid; t < count; t += NTHREADS) v += __ldcg(partials + base + t);
-    return block_sum_fixed(v, red);
+    for (int t = lane; t < count; t += 32) v += __ldcg(partials + base + t);
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+// Sum over the warp of one value per tail entry (lane q), valid on every lane.
+__device__ __forceinline__ double tail_sum(double v) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
 }
 
 // (at most 48 registers a thread: five blocks per SM keep one chunk per block co-resident
@@ -139,13 +145,13 @@ mgs_column_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
         const V* W = reinterpret_cast<const V*>(vptr<T>(P, j));
         const V* D = reinterpret_cast<const V*>(vptr<T>(P, ma.k0 - 1));
         V* ws = wsh + (size_t)sl * QPC;
-        double accd = 0.0;
+        DotSum<V> acc;
         for (long long q = q0 + tid; q < q1; q += NTHREADS) {
             const V w = W[q];
             ws[q - q0] = w;
-            accd += dotv(w, D[q]);
+            acc.add(w, D[q]);
         }
-        const double bsum = block_sum_fixed(accd, red);
+        const double bsum = block_total(acc, red);
         if (tid == 0) ma.partials[g] = bsum;
         double* kry = P->kry;
         if (tid < P->p) {
@@ -168,31 +174,27 @@ mgs_column_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
         const int g = blockIdx.x * cpb + sl;
         const int2 pc = __ldg(table + g);
         const ProblemDev* P = probs + pc.x;
-        const double tot = problem_total(ma.partials, g - pc.y, P->pchunks, red, tid);
-        if (tid == 0) {
+        if (tid < 32) {            // one warp: lane q holds tail entry q (p <= MAX_P < 32)
+            const double tot = problem_total(ma.partials, g - pc.y, P->pchunks, tid);
             double* kry = P->kry;
-            const bool writer = pc.y == 0;
+            const bool writer = pc.y == 0 && tid == 0;
             const int p = P->p;
             if (!isfinite(tot)) {
-                s_act[sl] = 0;
+                if (tid == 0) s_act[sl] = 0;
                 if (writer) {
                     kry[KRY_NONFINITE] = 1.0;
                     kry[KRY_ACTIVE] = 0.0;
                 }
             } else {
                 const int k0 = ma.k0;
-                const double sj = s_sc[sl][0];
-                const double* tj = s_ta[sl];
-                const double* tk0 = s_tb[sl];
-                double* a = s_tw[sl];
-                for (int q = 0; q < p; ++q) a[q] = tj[q];
-                for (int q = 0; q < p - 1; ++q) a[q] = sj * a[q + 1];
-                a[p - 1] = 0.0;
-                double d = 0.0;
-                for (int q = 0; q < p; ++q) d += a[q] * tk0[q];
+                const double a = tid < p - 1 ? s_sc[sl][0] * s_ta[sl][tid + 1] : 0.0;
+                const double d = tail_sum(tid < p ? a * s_tb[sl][tid] : 0.0);
+                if (tid < p) s_tw[sl][tid] = a;
                 const double h = s_sc[sl][1] * (tot + d);
-                s_h[sl][k0 - 1] = h;
-                s_tail[sl] = 1;
+                if (tid == 0) {
+                    s_h[sl][k0 - 1] = h;
+                    s_tail[sl] = 1;
+                }
                 if (writer) kry[KRY_H + (k0 - 1) * MAX_M + (j - 1)] = h;
             }
         }
@@ -215,16 +217,16 @@ mgs_column_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
             const V* Qk = reinterpret_cast<const V*>(vptr<T>(P, k - 1));
             const V* Qn = k < j ? reinterpret_cast<const V*>(vptr<T>(P, k)) : nullptr;
             V* ws = wsh + (size_t)sl * QPC;
-            double accd = 0.0;
+            DotSum<V> acc;
 #pragma unroll 2
             for (long long q = q0 + tid; q < q1; q += NTHREADS) {
                 const V qk = Qk[q];
                 const V qn = Qn ? Qn[q] : V{};
                 const V w = axpy16(ws[q - q0], coef, qk);
                 ws[q - q0] = w;
-                accd += dotv(w, Qn ? qn : w);
+                acc.add(w, Qn ? qn : w);
             }
-            const double bsum = block_sum_fixed(accd, red);
+            const double bsum = block_total(acc, red);
             if (tid == 0) part[g] = bsum;
             double* kry = P->kry;
             if (tid < P->p) {
@@ -246,46 +248,37 @@ mgs_column_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
             const int g = blockIdx.x * cpb + sl;
             const int2 pc = __ldg(table + g);
             const ProblemDev* P = probs + pc.x;
-            const double tot = problem_total(part, g - pc.y, P->pchunks, red, tid);
-            if (tid == 0) {
+            if (tid < 32) {
+                const double tot = problem_total(part, g - pc.y, P->pchunks, tid);
                 double* kry = P->kry;
-                const bool writer = pc.y == 0;
+                const bool writer = pc.y == 0 && tid == 0;
                 const int p = P->p;
                 if (!isfinite(tot)) {
-                    s_act[sl] = 0;
+                    if (tid == 0) s_act[sl] = 0;
                     if (writer) {
                         kry[KRY_NONFINITE] = 1.0;
                         kry[KRY_ACTIVE] = 0.0;
                     }
                 } else {
-                    const double hkj = s_h[sl][k - 1];
-                    const double sk = s_sc[sl][0];
-                    const double* tk = s_ta[sl];
-                    double* w = s_tw[sl];
-                    for (int q = 0; q < p; ++q) w[q] -= hkj * sk * tk[q];
+                    const double hs = s_h[sl][k - 1] * s_sc[sl][0];
+                    const double w = tid < p ? s_tw[sl][tid] - hs * s_ta[sl][tid] : 0.0;
+                    if (tid < p) s_tw[sl][tid] = w;
+                    const double tb = tid < p ? s_tb[sl][tid] : 0.0;
                     if (k < j) {
-                        const double* tn = s_tb[sl];
-                        double d = 0.0;
-                        for (int q = 0; q < p; ++q) d += w[q] * tn[q];
-                        const double h = s_sc[sl][1] * (tot + d);
-                        s_h[sl][k] = h;
+                        const double h = s_sc[sl][1] * (tot + tail_sum(w * tb));
+                        if (tid == 0) s_h[sl][k] = h;
                         if (writer) kry[KRY_H + k * MAX_M + (j - 1)] = h;
-                    } else {
-                        double d = 0.0;
-                        for (int q = 0; q < p; ++q) d += w[q] * w[q];
-                        const double h = sqrt(tot + d);
-                        if (j < ma.m) {
-                            if (writer) kry[KRY_H + j * MAX_M + (j - 1)] = h;
-                            if (!(h > ma.tol)) {
-                                s_act[sl] = 0;
-                                if (writer) {
-                                    kry[KRY_ACTIVE] = 0.0;
-                                    kry[KRY_MEFF] = (double)j;
-                                }
-                            } else if (writer) {
+                    } else if (j < ma.m) {
+                        const double h = sqrt(tot + tail_sum(w * w)), sg = tail_sum(tb * w);
+                        const bool on = h > ma.tol;
+                        if (tid == 0 && !on) s_act[sl] = 0;
+                        if (writer) {
+                            kry[KRY_H + j * MAX_M + (j - 1)] = h;
+                            if (!on) {
+                                kry[KRY_ACTIVE] = 0.0;
+                                kry[KRY_MEFF] = (double)j;
+                            } else {
                                 kry[KRY_S + j + 1] = 1.0 / h;
-                                double sg = 0.0;
-                                for (int q = 0; q < p; ++q) sg += s_tb[sl][q] * w[q];
                                 P->sigma[j + 1] = P->has_src ? sg : 0.0;
                             }
                         }
