@@ -56,7 +56,7 @@ struct ProblemDev {
     int nz, nfields;      // 2D: 1 and 4 (u, v, w_x, w_y); 3D: nz and 6 (w_z, psi added)
     int src_k, tiles_z;   // 3D: source plane, tiles along z (KC3 planes each); 2D: 0, 1
     int pchunks, pchunk_base;   // flat pointwise passes: chunks of this problem's vector, first
-    int nbtab, pad2;      // entries of btab
+    int nbtab, kc3;       // entries of btab; 3D TMA passes: planes per task
     double beta0, inv_dx, inv_dx2, inv_pml;
     double f_peak, t0, amp;
     long long field_stride, vec_stride;
@@ -190,6 +190,7 @@ void launch_leapfrog3d(int precision, int R, int nblocks, const ProblemDev* prob
 // kernels_tma3d.cu: persistent TMA-fed FP32 forward pass of three-dimensional problems.
 int upload_tma3d_tables(const double* fs_uzz, const double* fs_uz, const double* fs_dwz);
 int tma3d_tasks_of(const ProblemDev& P);
+void tma3d_choose_chunk(std::vector<ProblemDev>& probs, int R);   // sets kc3
 int build_tensor_maps3d(std::vector<ProblemDev>& probs, int R, const std::vector<int>& work_vecs,
                         void** d_maps_inout);
 int launch_stage_tma3d(int R, int warps, const ProblemDev* probs, const int* tbase, int nprob,

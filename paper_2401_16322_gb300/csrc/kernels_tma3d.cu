@@ -5,8 +5,8 @@
 // with the auxiliary field psi, Sec. 2.1 stencils, Appendix A / Sec. 2.2 rows on the vertical
 // axis, damping from the per-model table, and the integrators' K / Y / ACC epilogue),
 // organised for HBM bandwidth:
-//   - a task is one 64 x 8 column tile of one problem over a chunk of KC3 planes; one CTA per
-//     SM walks the task list (tasks b, b + gridDim.x, ...);
+//   - a task is one 64 x 8 column tile of one problem over a chunk of planes (tma3d_choose_chunk);
+//     one CTA per SM walks the task list (tasks b, b + gridDim.x, ...);
 //   - the producer lane streams the chunk plane by plane through NST shared-memory stages
 //     (cp.async.bulk.tensor over 5D maps: x, y, z, field, vector).  The stage for compute
 //     plane c holds u(c) with its x / y halo, w_x(c) (x halo), w_y(c) (y halo), v(c), c^2(c),
@@ -28,6 +28,7 @@
 #include <vector>
 
 #include "ewave_internal.cuh"
+#include "pdl.cuh"
 
 namespace ewv {
 
@@ -61,14 +62,17 @@ struct Stage3 {
                   "TMA destinations must be 128-byte aligned");
 };
 
+// What the producer resolves once per task and hands to the consumers.  Two slots alternate:
+// a task has at least 2 R + 1 stages, more than the ring holds, so the consumers have left task
+// t before the producer starts task t + 2.
 struct __align__(16) Info3 {
     float* Y;
     float* A;
     const float* X;          // u field of the input vector (free-surface column taps)
     long long fstr, ps;
-    int x0, y0, c, warm;     // compute plane c; warm = 1: front values only
-    int nx, ny, nz, pitch, pml, fs, src_i, src_j, src_k, pad0;
-    float beta0, inv_pml, idx1, idx2, sig, xs;   // xs: per-problem scale of H X (Krylov)
+    int x0, y0;
+    int nx, ny, nz, pitch, fs, src_i, src_j, src_k;
+    float idx1, idx2, sig, xs;   // xs: per-problem scale of H X (Krylov)
 };
 
 __device__ __forceinline__ uint32_t saddr(const void* p) {
@@ -173,12 +177,6 @@ __device__ __forceinline__ float bt3(const float* t, int n, int k) {
     return (unsigned)k < (unsigned)n ? __ldg(t + k) : 0.f;
 }
 
-__device__ __forceinline__ float dmp(float beta0, float inv_pml, float d, int pml) {
-    if (pml <= 0) return 0.f;
-    const float r = 1.f - d * inv_pml;
-    return (d <= (float)pml) ? beta0 * r * r : 0.f;
-}
-
 // Half-point derivative of psi along one axis (unscaled), plain loads: p points at psi of the
 // output node, `stride` is the axis stride, idx the node index and n the extent (zero
 // extension); up = true for the vertical axis (sum_q s_q (psi_{k-q} - psi_{k+1+q})).
@@ -210,7 +208,9 @@ __device__ __forceinline__ int find_task_problem(const int* __restrict__ base, i
     return lo;
 }
 
-// MODE 0: integrator pass (epilogue above).  MODE 1: leap-frog step (Sec. 3.1's scheme on
+// MODE 0: integrator pass (epilogue above).  MODE 2: its steady-state form (ck = 1 and cau = cak =
+// cax = 0: the Faber and HORK passes), Y = cu U + cx X + ch (H X + sigma), ACC = ca A + cay Y.
+// MODE 1: leap-frog step (Sec. 3.1's scheme on
 // the 3D system): a.x = level n (cur), a.a = level n-1 (prev, overwritten with level n+1 in
 // fields u, w_x, w_y, w_z and psi), a.m = damping variant (0 time-averaged, 1 explicit),
 // a.dt; psi^{n+1} = psi^n + dt (u^n + u^{n+1}) / 2.
@@ -226,8 +226,9 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
     float* smem = reinterpret_cast<float*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     __shared__ __align__(8) uint64_t full[NST];
     __shared__ __align__(8) uint64_t empty[NST];
-    __shared__ Info3 info[NST];
+    __shared__ Info3 info[2];
     __shared__ int s_err;
+    static_assert(NST < 2 * R + 1, "the task info needs a ring shorter than a task");
 
     const int tid = threadIdx.x;
     const int warp = tid >> 5, lane = tid & 31;
@@ -240,6 +241,8 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_trigger();
+    pdl_wait();
 
     const bool has_u = a.u >= 0, has_a = a.a >= 0;
     const uint32_t bytes_warm = 2u * L::PL * 4u;
@@ -251,9 +254,9 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
     if (warp == NW) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
-            int it = 0;
+            int it = 0, tslot = 0;
             bool stop = false;
-            for (int task = blockIdx.x; task < ntasks && !stop; task += gridDim.x) {
+            for (int task = blockIdx.x; task < ntasks && !stop; task += gridDim.x, tslot ^= 1) {
                 const int pid = find_task_problem(tbase, nprob, task);
                 const ProblemDev* P = probs + pid;
                 const CUtensorMap* maps = reinterpret_cast<const CUtensorMap*>(P->tmaps);
@@ -263,17 +266,34 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                 const int x0 = (lt % tiles_x) * BX;
                 const int r = lt / tiles_x;
                 const int y0 = (r % tiles_y) * BY3;
-                const int k0 = (r / tiles_y) * KC3;
-                const int k1 = min(k0 + KC3, P->nz);
+                const int k0 = (r / tiles_y) * P->kc3;
+                const int k1 = min(k0 + P->kc3, P->nz);
                 const int kx = a.x, vx = a.x == 0 ? 0 : a.x - 1;
-                float* Yp = a.y_out >= 0 ? (a.y_out == 0 ? (float*)P->state
-                                                         : (float*)P->work + (long long)(a.y_out - 1) * P->vec_stride)
-                                         : nullptr;
-                float* Ap = a.acc_out >= 0 ? (a.acc_out == 0 ? (float*)P->state
-                                                             : (float*)P->work + (long long)(a.acc_out - 1) * P->vec_stride)
-                                           : nullptr;
-                const float* Xp = a.x == 0 ? (const float*)P->state
-                                           : (const float*)P->work + (long long)(a.x - 1) * P->vec_stride;
+                Info3 ti;
+                ti.Y = a.y_out >= 0 ? (a.y_out == 0 ? (float*)P->state
+                                                    : (float*)P->work + (long long)(a.y_out - 1) * P->vec_stride)
+                                    : nullptr;
+                ti.A = a.acc_out >= 0 ? (a.acc_out == 0 ? (float*)P->state
+                                                        : (float*)P->work + (long long)(a.acc_out - 1) * P->vec_stride)
+                                      : nullptr;
+                ti.X = a.x == 0 ? (const float*)P->state
+                                : (const float*)P->work + (long long)(a.x - 1) * P->vec_stride;
+                ti.fstr = P->field_stride;
+                ti.ps = (long long)P->ny * P->pitch;
+                ti.x0 = x0;
+                ti.y0 = y0;
+                ti.nx = P->nx;
+                ti.ny = P->ny;
+                ti.nz = P->nz;
+                ti.pitch = P->pitch;
+                ti.fs = P->fs;
+                ti.src_i = P->src_i;
+                ti.src_j = P->src_j;
+                ti.src_k = P->src_k;
+                ti.idx1 = P->finv_dx;
+                ti.idx2 = P->finv_dx2;
+                ti.sig = (a.src_slot >= 0 && P->has_src) ? (float)P->sigma[a.src_slot] : 0.f;
+                ti.xs = a.x_scale_slot >= 0 ? (float)P->kry[a.x_scale_slot] : 1.f;
                 // stages: front planes f = k0 - R .. k1 - 1 + R; compute plane c = f - R >= k0
                 for (int f = k0 - R; f < k1 + R; ++f, ++it) {
                     const int s = it % NST;
@@ -285,31 +305,8 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                     }
                     const int c = f - R;
                     const bool warm = c < k0;
-                    Info3& ti = info[s];
-                    ti.Y = Yp;
-                    ti.A = Ap;
-                    ti.X = Xp;
-                    ti.fstr = P->field_stride;
-                    ti.ps = (long long)P->ny * P->pitch;
-                    ti.x0 = x0;
-                    ti.y0 = y0;
-                    ti.c = c;
-                    ti.warm = warm ? 1 : 0;
-                    ti.nx = P->nx;
-                    ti.ny = P->ny;
-                    ti.nz = P->nz;
-                    ti.pitch = P->pitch;
-                    ti.pml = P->pml;
-                    ti.fs = P->fs;
-                    ti.src_i = P->src_i;
-                    ti.src_j = P->src_j;
-                    ti.src_k = P->src_k;
-                    ti.beta0 = P->fbeta0;
-                    ti.inv_pml = P->finv_pml;
-                    ti.idx1 = P->finv_dx;
-                    ti.idx2 = P->finv_dx2;
-                    ti.sig = (a.src_slot >= 0 && P->has_src) ? (float)P->sigma[a.src_slot] : 0.f;
-                    ti.xs = a.x_scale_slot >= 0 ? (float)P->kry[a.x_scale_slot] : 1.f;
+                    // (released to the consumers by the arrive below, like the copies)
+                    if (f == k0 - R) info[tslot] = ti;
                     float* st = smem + (size_t)s * L::FLOATS;
                     bar_expect_tx(&full[s], warm ? bytes_warm : bytes_full);
                     tma5(st + L::UF_OFF, map3(maps, kx, 3), x0, y0, f, 0, vx, &full[s]);
@@ -318,7 +315,7 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                         tma5(st + L::U_OFF, map3(maps, kx, 0), x0 - TX3, y0 - R, c, 0, vx, &full[s]);
                         tma5(st + L::WX_OFF, map3(maps, kx, 1), x0 - TX3, y0, c, 2, vx, &full[s]);
                         tma5(st + L::WY_OFF, map3(maps, kx, 2), x0, y0 - R, c, 3, vx, &full[s]);
-                        if (MODE == 0) tma5(st + L::V_OFF, map3(maps, kx, 3), x0, y0, c, 1, vx, &full[s]);
+                        if (MODE != 1) tma5(st + L::V_OFF, map3(maps, kx, 3), x0, y0, c, 1, vx, &full[s]);
                         tma3(st + L::C2_OFF, maps + 10, x0, y0, c, &full[s]);
                         tma5(st + L::PS_OFF, map3(maps, kx, 3), x0, y0, c, 5, vx, &full[s]);
                         if (has_u)
@@ -349,9 +346,9 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
 #pragma unroll
             for (int q = 0; q < 2 * R; ++q) wq[r][q] = 0.f;
         }
-        int it = 0;
+        int it = 0, tslot = 0;
         bool stop = false;
-        for (int task = blockIdx.x; task < ntasks && !stop; task += gridDim.x) {
+        for (int task = blockIdx.x; task < ntasks && !stop; task += gridDim.x, tslot ^= 1) {
             // the number of stages of this task is known from its geometry: recompute it
             const int pid = find_task_problem(tbase, nprob, task);
             const ProblemDev* P = probs + pid;
@@ -360,8 +357,8 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
             const int tiles_x = (P->nx + BX - 1) / BX;
             const int tiles_y = (P->ny + BY3 - 1) / BY3;
             const int lt = task - __ldg(tbase + pid);
-            const int k0 = ((lt / tiles_x) / tiles_y) * KC3;
-            const int k1 = min(k0 + KC3, P->nz);
+            const int k0 = ((lt / tiles_x) / tiles_y) * P->kc3;
+            const int k1 = min(k0 + P->kc3, P->nz);
             // the horizontal damping of this thread's column and rows is fixed for the task:
             // looked up once, not per plane
             const int ti_ = (lt % tiles_x) * BX + tx;
@@ -383,7 +380,7 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                     stop = true;
                     break;
                 }
-                const Info3& ti = info[s];   // field loads on use (a register copy would spill)
+                const Info3& ti = info[tslot];   // field loads on use (a register copy would spill)
                 const float* st = smem + (size_t)s * L::FLOATS;
                 // push the front values into the queues
 #pragma unroll
@@ -396,10 +393,11 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                     uq[r][2 * R] = st[L::UF_OFF + pt];
                     wq[r][2 * R - 1] = st[L::WZ_OFF + pt];
                 }
-                if (!ti.warm) {
-                    const int nx = ti.nx, ny = ti.ny, nz = ti.nz, pml = ti.pml, c = ti.c;
+                const int c = f - R;
+                if (c >= k0) {
+                    const int nx = ti.nx, ny = ti.ny, nz = ti.nz;
                     const bool fs = ti.fs != 0;
-                    const float beta0 = ti.beta0, inv_pml = ti.inv_pml, idx1 = ti.idx1, idx2 = ti.idx2;
+                    const float idx1 = ti.idx1, idx2 = ti.idx2;
                     const long long fstr = ti.fstr, ps = ti.ps;
                     const int i = ti.x0 + tx;
                     const float* su = st + L::U_OFF;
@@ -416,20 +414,17 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                         const float* urow = su + (ly + R) * L::SW + cxs;
                         const float* wxrow = swx + ly * L::SW + cxs;
                         const float u = uq[r][R];
-                        float px[R], py[R], dx[R], dy[R], dwxv[R], dwyv[R];
+                        float px[R], py[R], dwxv[R], dwyv[R];
 #pragma unroll
                         for (int q = 0; q < R; ++q) {
                             px[q] = urow[q + 1] + urow[-q - 1];
                             py[q] = urow[(q + 1) * L::SW] + urow[-(q + 1) * L::SW];
-                            dx[q] = urow[1 + q] - urow[-q];
-                            dy[q] = urow[(1 + q) * L::SW] - urow[-q * L::SW];
                             dwxv[q] = wxrow[q] - wxrow[-1 - q];
                             dwyv[q] = swy[(ly + R + q) * BX + tx] - swy[(ly + R - 1 - q) * BX + tx];
                         }
                         const float uxx = ce_tree<R>(u, px), uyy = ce_tree<R>(u, py);
-                        const float dux = st_tree<R>(dx), duy = st_tree<R>(dy);
                         const float dwx = st_tree<R>(dwxv), dwy = st_tree<R>(dwyv);
-                        float uzz, dwz, duz;
+                        float uzz, dwz;
                         const long long oc = (long long)j * ti.pitch + i;
                         if (fs && c < 4) {
                             const float* ucol = ti.X + oc;
@@ -452,18 +447,6 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                             uzz = ce_tree<R>(u, pz);
                             dwz = st_tree<R>(dwzv);
                         }
-                        if (fs && c < 3) {
-                            const float* ucol = ti.X + oc;
-                            duz = 0.f;
-#pragma unroll
-                            for (int q = 0; q < 8; ++q)
-                                duz += g3t_fs[T3_UZ + c * 8 + q] * (q < nz ? __ldg(ucol + q * ps) : 0.f);
-                        } else {
-                            float dz[R];
-#pragma unroll
-                            for (int q = 0; q < R; ++q) dz[q] = uq[r][R - q] - uq[r][R + 1 + q];
-                            duz = st_tree<R>(dz);
-                        }
                         const float byn = byn_t[r], byh = byh_t[r];
                         const int pt = ly * BX + tx;
                         const float xwx = wxrow[0];
@@ -473,13 +456,41 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                         const float xpsi = st[L::PS_OFF + pt];
                         const bool at_src = i == ti.src_i && j == ti.src_j && c == ti.src_k;
                         const long long o = (long long)c * ps + oc;
-                        // psi terms: (product of the other two b's) d_a psi, zero off the edges
-                        float gp[3] = {0.f, 0.f, 0.f};
-                        {
+                        const float force = c2 * ((uxx + uyy + uzz) * idx2 + (dwx + dwy + dwz) * idx1);
+                        // damped points only (elsewhere the w rows of H are zero and the v row has
+                        // no damping term): the half-point differences of u, and the psi terms
+                        // (product of the other two b's) d_a psi, zero off the edges of the layer
+                        const bool damped = bxn + bxh + byn + byh + bzn + bzh != 0.f;   // (none is negative)
+                        const float gco[3] = {byn + bzn - bxh, bxn + bzn - byh, bxn + byn - bzh};
+                        float gw[3] = {0.f, 0.f, 0.f};
+                        float hdamp = 0.f;
+                        if (damped) {
+                            float dx[R], dy[R];
+#pragma unroll
+                            for (int q = 0; q < R; ++q) {
+                                dx[q] = urow[1 + q] - urow[-q];
+                                dy[q] = urow[(1 + q) * L::SW] - urow[-q * L::SW];
+                            }
+                            gw[0] = gco[0] * st_tree<R>(dx) * idx1;
+                            gw[1] = gco[1] * st_tree<R>(dy) * idx1;
+                            float duz;
+                            if (fs && c < 3) {
+                                const float* ucol = ti.X + oc;
+                                duz = 0.f;
+#pragma unroll
+                                for (int q = 0; q < 8; ++q)
+                                    duz += g3t_fs[T3_UZ + c * 8 + q] * (q < nz ? __ldg(ucol + q * ps) : 0.f);
+                            } else {
+                                float dz[R];
+#pragma unroll
+                                for (int q = 0; q < R; ++q) dz[q] = uq[r][R - q] - uq[r][R + 1 + q];
+                                duz = st_tree<R>(dz);
+                            }
+                            gw[2] = gco[2] * duz * idx1;
                             const float pyz = byn * bzn, pxz = bxn * bzn, pxy = bxn * byn;
                             const float* pc = ti.X + 5 * fstr + o;
-                            if (pyz != 0.f && i < nx - 1) gp[0] = pyz * dpsi3<R>(pc, 1, i, nx, false) * idx1;
-                            if (pxz != 0.f && j < ny - 1) gp[1] = pxz * dpsi3<R>(pc, ti.pitch, j, ny, false) * idx1;
+                            if (pyz != 0.f && i < nx - 1) gw[0] += pyz * dpsi3<R>(pc, 1, i, nx, false) * idx1;
+                            if (pxz != 0.f && j < ny - 1) gw[1] += pxz * dpsi3<R>(pc, ti.pitch, j, ny, false) * idx1;
                             if (pxy != 0.f && c < nz - 1) {
                                 float d = 0.f;
                                 if (fs && c < 3) {
@@ -490,18 +501,17 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                                 } else {
                                     d = dpsi3<R>(pc, ps, c, nz, true);
                                 }
-                                gp[2] = pxy * d * idx1;
+                                gw[2] += pxy * d * idx1;
                             }
+                            hdamp = -(pxy + pyz + pxz) * u - pxy * bzn * xpsi;
                         }
-                        if constexpr (MODE == 0) {
+                        if constexpr (MODE != 1) {
                             const float xv = st[L::V_OFF + pt];
-                            float hv = -(bxn * byn + byn * bzn + bxn * bzn) * u - (bxn + byn + bzn) * xv
-                                       - bxn * byn * bzn * xpsi
-                                       + c2 * ((uxx + uyy + uzz) * idx2 + (dwx + dwy + dwz) * idx1);
+                            float hv = force + hdamp - (bxn + byn + bzn) * xv;
                             if (at_src) hv += ti.sig;
-                            const float hwx = (i < nx - 1) ? (byn + bzn - bxh) * dux * idx1 + gp[0] - bxh * xwx : 0.f;
-                            const float hwy = (j < ny - 1) ? (bxn + bzn - byh) * duy * idx1 + gp[1] - byh * xwy : 0.f;
-                            const float hwz = (c < nz - 1) ? (bxn + byn - bzh) * duz * idx1 + gp[2] - bzh * xwz : 0.f;
+                            const float hwx = (i < nx - 1) ? gw[0] - bxh * xwx : 0.f;
+                            const float hwy = (j < ny - 1) ? gw[1] - byh * xwy : 0.f;
+                            const float hwz = (c < nz - 1) ? gw[2] - bzh * xwz : 0.f;
                             const float xf[6] = {u, xv, xwx, xwy, xwz, xpsi};
                             const float hf[6] = {xv, hv, hwx, hwy, hwz, u};
                             float* yp = ti.Y ? ti.Y + o : nullptr;
@@ -513,6 +523,12 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                                 const float uval = has_u ? st[L::PU_OFF + fld * L::PL + pt] : 0.f;
                                 const float aval = has_a ? st[L::PA_OFF + fld * L::PL + pt] : 0.f;
                                 const float kf = cxf * xf[fld] + (chf * ti.xs) * hf[fld];
+                                if constexpr (MODE == 2) {
+                                    const float yf = pad ? 0.f : (has_u ? fmaf(cuf, uval, kf) : kf);
+                                    if (yp) yp[fld * fstr] = yf;
+                                    if (ap) ap[fld * fstr] = has_a ? fmaf(cayf, yf, caf * aval) : cayf * yf;
+                                    continue;
+                                }
                                 const float yf = pad ? 0.f : (cuf * uval + ckf * kf);
                                 if (yp) yp[fld * fstr] = yf;
                                 if (ap) ap[fld * fstr] = pad ? 0.f : (caf * aval + cauf * uval + cakf * kf + cayf * yf + caxf * xf[fld]);
@@ -521,8 +537,7 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                             const float dt = (float)a.dt;
                             const float inv_dt2 = 1.f / (dt * dt), inv_2dt = 1.f / (2.f * dt);
                             const float bsum = bxn + byn + bzn;
-                            float rhs = -(bxn * byn + byn * bzn + bxn * bzn) * u - bxn * byn * bzn * xpsi
-                                        + c2 * ((uxx + uyy + uzz) * idx2 + (dwx + dwy + dwz) * idx1);
+                            float rhs = force + hdamp;
                             if (at_src) rhs += ti.sig;
                             const float* pm = st + L::PA_OFF + pt;   // level n-1, six fields
                             const float um = pm[0];
@@ -531,8 +546,6 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                                                         inv_dt2 + bsum * inv_2dt);
                             const bool has[3] = {i < nx - 1, j < ny - 1, c < nz - 1};
                             const float bh[3] = {bxh, byh, bzh};
-                            const float gco[3] = {byn + bzn - bxh, bxn + bzn - byh, bxn + byn - bzh};
-                            const float du[3] = {dux, duy, duz};
                             const float wcur[3] = {xwx, xwy, xwz};
                             float* out = ti.Y + o;
                             out[0] = up;
@@ -541,8 +554,9 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                                 float wn = 0.f;
                                 if (has[a3]) {
                                     const float wm = pm[(2 + a3) * L::PL];
-                                    const float g = gco[a3] * du[a3] * idx1 + gp[a3];
-                                    wn = a.m == 0 ? __fdividef((1.f - bh[a3] * dt) * wm + 2.f * dt * g, 1.f + bh[a3] * dt)
+                                    const float g = gw[a3];
+                                    wn = !damped  ? wm
+                                         : a.m == 0 ? __fdividef((1.f - bh[a3] * dt) * wm + 2.f * dt * g, 1.f + bh[a3] * dt)
                                                   : wm + 2.f * dt * (-bh[a3] * wcur[a3] + g);
                                 }
                                 out[(2 + a3) * fstr] = wn;
@@ -625,8 +639,7 @@ int launch3(const ProblemDev* probs, const int* tbase, int nprob, int ntasks, co
         if (g_sms3 <= 0) g_sms3 = 1;
     }
     const int grid = ntasks < g_sms3 ? ntasks : g_sms3;
-    stage_tma3d_kernel<R, NW, NST, MODE><<<grid, NW * 32 + 32, smem, s>>>(probs, tbase, nprob, ntasks, a, err);
-    return 0;
+    return launch_pdl(stage_tma3d_kernel<R, NW, NST, MODE>, grid, NW * 32 + 32, smem, s, probs, tbase, nprob, ntasks, a, err);
 }
 
 }  // namespace
@@ -640,7 +653,39 @@ int upload_tma3d_tables(const double* fs_uzz, const double* fs_uz, const double*
 }
 
 int tma3d_tasks_of(const ProblemDev& P) {
-    return ((P.nx + BX - 1) / BX) * ((P.ny + BY3 - 1) / BY3) * ((P.nz + KC3 - 1) / KC3);
+    return ((P.nx + BX - 1) / BX) * ((P.ny + BY3 - 1) / BY3) * ((P.nz + P.kc3 - 1) / P.kc3);
+}
+
+// Planes per task, the same for every problem of an engine.  A task of kc planes costs about as
+// much as kc + R full stages (its 2 R warm-up stages carry two planes instead of twenty), and the
+// pass as many rounds of tasks as the busiest SM gets: take the chunk that makes rounds x stages
+// smallest.  251 x 229 x 197: 5 chunks of 40 planes (4 rounds of 44) instead of chunks of 32 (6
+// rounds of 36); with the undamped points' shorter form and the dependent launch, Faber degree 40
+// takes 12.7 ms instead of 13.0, and 100 x 95 x 260, whose 32-plane chunks left a second round
+// nearly empty, 4.1 instead of 6.1.  Chunks shorter than 16 planes are not worth their warm-up.
+void tma3d_choose_chunk(std::vector<ProblemDev>& probs, int R) {
+    int dev = 0, nsm = 0, nz = 1;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
+        nsm = 1;
+    for (const ProblemDev& P : probs) nz = P.nz > nz ? P.nz : nz;
+    const int warm = R;
+    long long best = -1;
+    int best_kc = nz;
+    for (int n = 1; n == 1 || nz / n >= 16; ++n) {
+        const int kc = (nz + n - 1) / n;
+        long long tasks = 0;
+        for (ProblemDev& P : probs) {
+            P.kc3 = kc;
+            tasks += tma3d_tasks_of(P);
+        }
+        const long long cost = (tasks + nsm - 1) / nsm * (kc + warm);
+        if (best < 0 || cost < best) {
+            best = cost;
+            best_kc = kc;
+        }
+    }
+    for (ProblemDev& P : probs) P.kc3 = best_kc;
 }
 
 // NMAP3 maps per problem: state and workspace, each with the u halo box, the w_x box, the w_y
@@ -680,8 +725,11 @@ int build_tensor_maps3d(std::vector<ProblemDev>& probs, int R, const std::vector
 int launch_stage_tma3d(int R, int warps, const ProblemDev* probs, const int* tbase, int nprob,
                        int ntasks, const StageArgs& a, int* err, cudaStream_t s) {
     if (ntasks <= 0) return nprob > 0 ? -1 : 0;
+    const bool steady = a.ck == 1.0 && a.cau == 0.0 && a.cak == 0.0 && a.cax == 0.0;
     if (warps == 16) {
-        if (R == 4) return launch3<4, 16, 4, 0>(probs, tbase, nprob, ntasks, a, err, s);
+        if (R == 4)
+            return steady ? launch3<4, 16, 4, 2>(probs, tbase, nprob, ntasks, a, err, s)
+                          : launch3<4, 16, 4, 0>(probs, tbase, nprob, ntasks, a, err, s);
         if (R == 2) return launch3<2, 16, 4, 0>(probs, tbase, nprob, ntasks, a, err, s);
     } else {
         if (R == 4) return launch3<4, 8, 4, 0>(probs, tbase, nprob, ntasks, a, err, s);
