@@ -113,8 +113,10 @@ int ensure_tables() {
     return 0;
 }
 
-// Minimum over theta of the centred second-derivative symbol.
-double symbol_min(int order) {
+// Minimum over theta of the centred second-derivative symbol, a constant of the order: found once a
+// process (the scan takes 0.57 ms, and every Faber call with the default ellipse ran it: one step
+// of degree 20 on 301 x 201 took 615 us, 122 without it).
+double scan_symbol_min(int order) {
     const double c8[5] = {-205.0 / 72.0, 8.0 / 5.0, -1.0 / 5.0, 8.0 / 315.0, -1.0 / 560.0};
     const double c4[3] = {-5.0 / 2.0, 4.0 / 3.0, -1.0 / 12.0};
     const double* c = order == 8 ? c8 : c4;
@@ -127,6 +129,10 @@ double symbol_min(int order) {
         best = std::min(best, v);
     }
     return best;
+}
+double symbol_min(int order) {
+    static const double min8 = scan_symbol_min(8), min4 = scan_symbol_min(4);
+    return order == 8 ? min8 : min4;
 }
 
 struct Shot {
