@@ -1317,7 +1317,9 @@ int build_tensor_maps(std::vector<ProblemDev>& probs, int R, const std::vector<i
 // passes that read an A operand run variant 7, the others (Horner HORK passes, Krylov products,
 // leap-frog-free RK stages without an accumulator) drop the A buffer and take taller tiles (14:
 // 512 threads at 128 registers, the whole register file).  The shape reported for a composite is
-// its no-A shape.
+// its no-A shape.  Variant 10, two stages with the A buffer, is the better A shape where a pass is
+// a few tiles per SM (16 shots of 401 x 201: 20 us against 22 of variant 7), but without an A
+// operand it lost to 14 there (21 against 18): those passes run 14's shape.
 struct TmaVariant {
     int by, nw, nst;
 };
@@ -1329,6 +1331,7 @@ static bool composite(int v) { return v >= 11 && v <= 14; }
 
 int tma_variant_tile_height_for(int v, bool reads_a) {
     if (composite(v) && reads_a) return kVariants[7].by;
+    if (v == 10 && !reads_a) return kVariants[14].by;
     return kVariants[v].by;
 }
 
@@ -1503,6 +1506,7 @@ int launch_stage_tma(int variant, int R, const ProblemDev* probs, const int* tba
     // the steady-state Faber / HORK form: Y = cu U + cx X + ch H, ACC = ca A + cay Y
     const bool epi = a.ck == 1.0 && a.cau == 0.0 && a.cak == 0.0 && a.cax == 0.0;
     if (composite(variant) && a.a >= 0) variant = 7;   // composite, pass with A
+    if (variant == 10 && a.a < 0) variant = 14;
     if (variant == 4 && a.u >= 0) variant = 0;         // no U buffer
     // the shapes that repeat another one's
     if (variant == 1) variant = 8;
