@@ -232,6 +232,8 @@ struct Engine {
     double* d_gs_partials = nullptr;   // FP32 Gram-Schmidt passes (allocated at their first use)
     double* d_gram = nullptr;
     unsigned int* d_mgs_bar = nullptr;
+    unsigned int* d_chain_bar = nullptr;   // grid-barrier words of the chained passes
+    bool chain_ok = false;                 // 2D FP64: a step's passes fit one cooperative launch
     double* d_ecoef = nullptr;    // [nprob][MAX_TAU][MAX_M]: exp(tau H) e_1 of a multi-output combine
     // adaptive Krylov step: tolerance, dimension range and statistics of the current call
     double ad_tol = 0.0;
@@ -306,6 +308,7 @@ struct Engine {
         cudaFree(d_gs_partials);
         cudaFree(d_gram);
         cudaFree(d_mgs_bar);
+        cudaFree(d_chain_bar);
         cudaFree(d_ecoef);
         cudaFree(d_kbar);
     }
@@ -570,6 +573,11 @@ int build_engine(Engine* E, std::string& err) {
         *E->h_err = 0;
         CUDA_OR_FAIL(err, cudaEventCreateWithFlags(&E->err_ev, cudaEventDisableTiming));
     }
+    E->chain_ok = E->precision == EWV_F64 && E->dims == 2 && chain_fits(E->ntiles);
+    if (E->chain_ok && !E->d_chain_bar) {
+        CUDA_OR_FAIL(err, cudaMalloc(&E->d_chain_bar, sizeof(unsigned int) * 2));
+        CUDA_OR_FAIL(err, cudaMemset(E->d_chain_bar, 0, sizeof(unsigned int) * 2));
+    }
     std::vector<int> tp(tb);
     for (int p = 0; p < E->nprob; ++p)
         for (int t = 0; t < E->probs[p].ntiles; ++t) tp[E->probs[p].tile_base + t] = p;
@@ -680,7 +688,37 @@ struct Ctx {
         if (E->timing) cudaEventRecordWithFlags(e1, s, rec_flags);
         ++*launches;
     }
+    // Chained passes (small 2D FP64 engines): the stage() calls between chain_begin and chain_end
+    // go out as one cooperative launch.  Not while passes are timed one by one.
+    PassChain chain;
+    bool chaining = false;
+    void chain_begin() {
+        chaining = E->chain_ok && !E->timing;
+        chain.n = 0;
+    }
+    void chain_end() {
+        if (!chaining) return;
+        chaining = false;
+        if (chain.n == 0) return;
+        if (launch_chain(E->R, E->ntiles, E->d_probs, E->d_tile_prob, chain, E->d_chain_bar, E->d_err, s) == 0) {
+            ++*launches;
+            return;
+        }
+        cudaGetLastError();         // no cooperative launch to be had: pass by pass
+        E->chain_ok = false;
+        for (int n = 0; n < chain.n; ++n) stage(chain_stage(chain.pass[n]));
+    }
     void stage(const StageArgs& a_in) {
+        if (chaining) {
+            if (chain.n == MAX_CHAIN) {
+                chain_end();
+                chain_begin();
+            }
+            ChainPass& c = chain.pass[chain.n++];
+            c = ChainPass{a_in.x, a_in.u, a_in.a, a_in.y_out, a_in.acc_out, a_in.src_slot, 0, 0,
+                          a_in.cx, a_in.ch, a_in.cu, a_in.ck, a_in.ca, a_in.cau, a_in.cak, a_in.cay, a_in.cax};
+            return;
+        }
         StageArgs a = a_in;
         a.store_bf16 = E->store_bf16;
         cudaEvent_t e0 = nullptr, e1 = nullptr;
@@ -907,6 +945,7 @@ int run_faber(Ctx& C, double t, double dt, int m, int nsteps, double g, double c
     ++*C.launches;
     C.prologue(PRO_FABER, m, g, c0, c1);
     int rc = C.step_loop(nsteps, EWV_METHOD_FABER, m, dt, g, c0, c1, 1, [&](int) {
+        C.chain_begin();
         StageArgs s1 = stage_defaults();
         s1.x = 0;
         s1.y_out = 1;
@@ -919,6 +958,7 @@ int run_faber(Ctx& C, double t, double dt, int m, int nsteps, double g, double c
         s1.cax = a[0];
         C.stage(s1);
         if (m == 1) {
+            C.chain_end();
             C.copy(2, 0, ALL_FIELDS, false);
         } else {
             StageArgs s2 = stage_defaults();
@@ -954,6 +994,7 @@ int run_faber(Ctx& C, double t, double dt, int m, int nsteps, double g, double c
                 C.stage(sj);
             }
         }
+        C.chain_end();
         C.record_next(0, PRO_FABER, m, g, c0, c1);
     });
     if (rc != EWV_OK) return rc;
@@ -990,6 +1031,7 @@ int run_hork_horner(Ctx& C, double t, double dt, int m, int nsteps) {
     ++*C.launches;
     C.prologue(PRO_HORK_HORNER, m);
     int rc = C.step_loop(nsteps, EWV_METHOD_HORK, m, dt, 0, 0, 0, 1, [&](int) {
+        C.chain_begin();
         int prev = 0;
         for (int k = 0; k < m; ++k) {
             const int j = m - k;
@@ -1009,6 +1051,7 @@ int run_hork_horner(Ctx& C, double t, double dt, int m, int nsteps) {
             C.stage(s);
             prev = s.y_out;
         }
+        C.chain_end();
         if (prev != 0) C.copy(prev, 0, ALL_FIELDS, false);   // m = 1: V_1 is in a work vector
         C.record_next(0, PRO_HORK_HORNER, m);
     });
@@ -1041,6 +1084,7 @@ int run_hork(Ctx& C, double t, double dt, int m, int nsteps) {
             C.record_next(0, PRO_HORK, m);
             return;
         }
+        C.chain_begin();
         for (int i = 1; i <= m; ++i) {
             StageArgs si = stage_defaults();
             si.cx = 1.0;
@@ -1070,6 +1114,7 @@ int run_hork(Ctx& C, double t, double dt, int m, int nsteps) {
             }
             C.stage(si);
         }
+        C.chain_end();
         C.record_next(0, PRO_HORK, m);
     });
     if (rc != EWV_OK) return rc;
@@ -1082,6 +1127,7 @@ int run_rk(Ctx& C, double t, double dt, int scheme, int nsteps) {
     const int pro = scheme == EWV_METHOD_RK32 ? PRO_RK32 : PRO_RK44, stages = scheme == EWV_METHOD_RK32 ? 3 : 4;
     C.prologue(pro, stages);
     int rc = C.step_loop(nsteps, scheme, 0, dt, 0, 0, 0, 1, [&](int) {
+        C.chain_begin();
         if (scheme == EWV_METHOD_RK32) {
             const int xs[3] = {0, 1, 2}, ys[3] = {1, 2, 0};
             const double al[3] = {0.5 * dt, 0.5 * dt, dt};
@@ -1114,6 +1160,7 @@ int run_rk(Ctx& C, double t, double dt, int scheme, int nsteps) {
             a.ch = 1.0; a.ca = 1.0; a.cak = dt / 6.0;
             C.stage(a);
         }
+        C.chain_end();
         C.record_next(0, pro, stages);
     });
     if (rc != EWV_OK) return rc;
@@ -1754,7 +1801,7 @@ int take_pending_error(Engine* E, cudaStream_t s, std::string& err) {
     const int w = *(volatile int*)E->h_err;
     CUDA_OR_FAIL(err, cudaMemset(E->d_err, 0, sizeof(int)));
     *(volatile int*)E->h_err = 0;
-    if (w & 1) return fail(err, EWV_ERR_TIMEOUT, "a bounded wait in a TMA pass or a Gram-Schmidt barrier timed out "
+    if (w & 1) return fail(err, EWV_ERR_TIMEOUT, "a bounded wait in a TMA pass or a grid barrier timed out "
                                                  "during an earlier call");
     return fail(err, EWV_ERR_NONFINITE, "a non-finite value appeared in the state during an earlier call");
 }
@@ -3310,7 +3357,7 @@ int ewv_batch_sync(ewv_batch_t b) {
 int ewv_debug_set_wait_limit(unsigned long long ns) {
     if (ns > 1000000000ull) return EWV_ERR_INVALID_ARG;
     if (cudaDeviceSynchronize() != cudaSuccess) return EWV_ERR_CUDA;
-    return set_tma_wait_limit_ns(ns) == 0 && set_mgs_wait_limit_ns(ns) == 0 ? EWV_OK : EWV_ERR_CUDA;
+    return set_tma_wait_limit_ns(ns) == 0 && set_mgs_wait_limit_ns(ns) == 0 && set_chain_wait_limit_ns(ns) == 0 ? EWV_OK : EWV_ERR_CUDA;
 }
 
 int ewv_debug_set_column_kernel(int enable) {

@@ -139,6 +139,39 @@ struct StageArgs {
     float fcx, fch, fcu, fck, fca, fcau, fcak, fcay, fcax;
 };
 
+// The forward passes of one step, launched together (see chain_kernel).
+struct ChainPass {
+    int x, u, a, y_out, acc_out, src_slot, terms, pad;
+    double cx, ch, cu, ck, ca, cau, cak, cay, cax;
+};
+constexpr int MAX_CHAIN = 128;
+struct PassChain {
+    int n, pad;
+    ChainPass pass[MAX_CHAIN];
+};
+__host__ __device__ inline StageArgs chain_stage(const ChainPass& c) {
+    StageArgs a{};
+    a.x = c.x;
+    a.u = c.u;
+    a.a = c.a;
+    a.y_out = c.y_out;
+    a.acc_out = c.acc_out;
+    a.d = -1;
+    a.src_slot = c.src_slot;
+    a.x_scale_slot = -1;
+    a.terms = c.terms;
+    a.cx = c.cx;
+    a.ch = c.ch;
+    a.cu = c.cu;
+    a.ck = c.ck;
+    a.ca = c.ca;
+    a.cau = c.cau;
+    a.cak = c.cak;
+    a.cay = c.cay;
+    a.cax = c.cax;
+    return a;
+}
+
 // Arguments of the pointwise kernel (kernels_aux.cu).
 struct PointArgs {
     int mode;        // 0: |q1|^2 (norm); 1: MGS pass; 2: Krylov combine; 3: copy; 4: swap;
@@ -169,6 +202,12 @@ int upload_stencil_tables(int order, const double* fs_uyy, const double* fs_uy,
                           const double* fs_dwy);
 void launch_stage(int precision, int R, int ntiles, const ProblemDev* probs,
                   const int* tile_prob, const StageArgs& a, cudaStream_t s);
+// The passes of a step in one cooperative launch (2D FP64): whether ntiles tiles fit, and the
+// launch; bar: two words, zero between launches.
+bool chain_fits(int ntiles);
+int launch_chain(int R, int ntiles, const ProblemDev* probs, const int* tile_prob, const PassChain& chain,
+                 unsigned int* bar, int* err, cudaStream_t s);
+int set_chain_wait_limit_ns(unsigned long long ns);
 // y = H x or H^T x of one problem, whose descriptor travels with the launch (-1: another pass).
 int launch_stage_one(int precision, int R, const ProblemDev& P, const StageArgs& a, cudaStream_t s);
 // One FP64 leap-frog step (2D).

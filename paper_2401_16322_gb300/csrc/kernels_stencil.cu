@@ -39,6 +39,7 @@
 #include <type_traits>
 
 #include "ewave_internal.cuh"
+#include "grid_barrier.cuh"
 #include "pdl.cuh"
 
 namespace ewv {
@@ -184,6 +185,11 @@ struct Taps {
     }
 };
 
+// a b + c rounded once.  The forward pass spells its sums out, so that every kernel that holds it
+// rounds alike: a chained step gives the bits of the same step launched pass by pass.
+__device__ __forceinline__ float mad(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double mad(double a, double b, double c) { return __fma_rn(a, b, c); }
+
 // Sums of u at (i, j): the Laplacian (times dx^2) and the half-point differences d_x u at
 // (i + 1/2, j), d_y u at (i, j + 1/2) (times dx).
 template <typename T, int R, bool BAND>
@@ -196,35 +202,35 @@ struct USums {
     __device__ __forceinline__ T laplacian() const {
         T uxx = CENT<T, R>(0) * t.row[R], uyy;
 #pragma unroll
-        for (int k = 1; k <= R; ++k) uxx += CENT<T, R>(k) * (t.row[R + k] + t.row[R - k]);
+        for (int k = 1; k <= R; ++k) uxx = mad(CENT<T, R>(k), (t.row[R + k] + t.row[R - k]), uxx);
         if constexpr (BAND) {
             uyy = T(0);
 #pragma unroll
-            for (int q = 0; q <= 2 * R; ++q) uyy += fs_coef<T>(FS_UYY_OFF + j * 9 + q) * t.col[q];
+            for (int q = 0; q <= 2 * R; ++q) uyy = mad(fs_coef<T>(FS_UYY_OFF + j * 9 + q), t.col[q], uyy);
         } else {
             uyy = CENT<T, R>(0) * t.row[R];
 #pragma unroll
-            for (int k = 1; k <= R; ++k) uyy += CENT<T, R>(k) * (t.col[R + k] + t.col[R - k]);
+            for (int k = 1; k <= R; ++k) uyy = mad(CENT<T, R>(k), (t.col[R + k] + t.col[R - k]), uyy);
         }
         return uxx + uyy;
     }
     __device__ __forceinline__ T du_x() const {
         T d = T(0);
 #pragma unroll
-        for (int k = 0; k < R; ++k) d += STAG<T, R>(k) * (t.row[R + 1 + k] - t.row[R - k]);
+        for (int k = 0; k < R; ++k) d = mad(STAG<T, R>(k), (t.row[R + 1 + k] - t.row[R - k]), d);
         return d;
     }
     __device__ __forceinline__ T du_y() const {
         T d = T(0);
         if constexpr (!BAND) {
 #pragma unroll
-            for (int k = 0; k < R; ++k) d += STAG<T, R>(k) * (t.col[R - k] - t.col[R + 1 + k]);
+            for (int k = 0; k < R; ++k) d = mad(STAG<T, R>(k), (t.col[R - k] - t.col[R + 1 + k]), d);
         } else if (j < 3) {
 #pragma unroll
-            for (int q = 0; q < 2 * R; ++q) d += fs_coef<T>(FS_UY_OFF + j * 8 + q) * t.col[q];
+            for (int q = 0; q < 2 * R; ++q) d = mad(fs_coef<T>(FS_UY_OFF + j * 8 + q), t.col[q], d);
         } else {     // row 3: the interior stencil, counted from row 0
 #pragma unroll
-            for (int k = 0; k < R; ++k) d += STAG<T, R>(k) * (t.col[R - 1 - k] - t.col[R + k]);
+            for (int k = 0; k < R; ++k) d = mad(STAG<T, R>(k), (t.col[R - 1 - k] - t.col[R + k]), d);
         }
         return d;
     }
@@ -237,13 +243,13 @@ __device__ __forceinline__ T divergence(const ProblemDev& P, const T* X, int i, 
     const Taps<T, R, 2 * R, BAND> t(X + 2 * P.field_stride, X + 3 * P.field_stride, i, j, P.pitch, P.nx - 1, P.ny - 1);
     T dwx = T(0), dwy = T(0);
 #pragma unroll
-    for (int k = 0; k < R; ++k) dwx += STAG<T, R>(k) * (t.row[R + k] - t.row[R - 1 - k]);
+    for (int k = 0; k < R; ++k) dwx = mad(STAG<T, R>(k), (t.row[R + k] - t.row[R - 1 - k]), dwx);
     if constexpr (BAND) {
 #pragma unroll
-        for (int q = 0; q < 2 * R; ++q) dwy += fs_coef<T>(FS_DWY_OFF + j * 8 + q) * t.col[q];
+        for (int q = 0; q < 2 * R; ++q) dwy = mad(fs_coef<T>(FS_DWY_OFF + j * 8 + q), t.col[q], dwy);
     } else {
 #pragma unroll
-        for (int k = 0; k < R; ++k) dwy += STAG<T, R>(k) * (t.col[R - 1 - k] - t.col[R + k]);
+        for (int k = 0; k < R; ++k) dwy = mad(STAG<T, R>(k), (t.col[R - 1 - k] - t.col[R + k]), dwy);
     }
     return dwx + dwy;
 }
@@ -300,21 +306,21 @@ __device__ __forceinline__ void epilogue(const ProblemDev& P, const StageArgs& a
         T kf;
         if (f < 2 || hw) {
             kf = ch * hf[f];
-            if (t & TERM_CX) kf += cx * xf[f];
+            if (t & TERM_CX) kf = mad(cx, xf[f], kf);
         } else {
             kf = (t & TERM_CX) ? cx * xf[f] : T(0);
         }
         T yf = (t & TERM_CK) ? (T)a.ck * kf : kf;
-        if (t & TERM_CU) yf += (T)a.cu * uv[f];
+        if (t & TERM_CU) yf = mad((T)a.cu, uv[f], yf);
         if (pad) yf = T(0);
         if (a.store_bf16) yf = bf16_round(yf);     // storage-precision experiment
         if (Y) Y[f * P.field_stride] = yf;
         if (ACC) {
             T af = (t & TERM_CA) ? (T)a.ca * av[f] : av[f];
-            if (t & TERM_CAY) af += (T)a.cay * yf;
-            if (t & TERM_CAU) af += (T)a.cau * uv[f];
-            if (t & TERM_CAK) af += (T)a.cak * kf;
-            if (t & TERM_CAX) af += cax * xf[f];
+            if (t & TERM_CAY) af = mad((T)a.cay, yf, af);
+            if (t & TERM_CAU) af = mad((T)a.cau, uv[f], af);
+            if (t & TERM_CAK) af = mad((T)a.cak, kf, af);
+            if (t & TERM_CAX) af = mad(cax, xf[f], af);
             if (a.store_bf16) af = bf16_round(af);
             ACC[f * P.field_stride] = pad ? T(0) : af;
         }
@@ -327,14 +333,14 @@ __device__ __forceinline__ void epilogue(const ProblemDev& P, const StageArgs& a
 enum { PASS_FORWARD = 0, PASS_GRADIENT = 1, PASS_TRANSPOSE = 2 };
 
 template <typename T, int R, bool BAND, int TERMS>
-__device__ __forceinline__ void forward_point(const ProblemDev& P, const StageArgs& a, int i, int j) {
+__device__ __forceinline__ void forward_point(const ProblemDev& P, const StageArgs& a, int i, int j,
+                                              const Damping<T>& b, T c2) {
     const int nx = P.nx, ny = P.ny;
     const long long o = (long long)j * P.pitch + i;
     const T* X = vec_ptr<T>(&P, a.x);
     const T idx1 = (T)P.inv_dx, idx2 = (T)P.inv_dx2;
-    const Damping<T> b(P, i, j);
     const bool padx = i >= nx - 1, pady = j >= ny - 1;
-    const T xv = X[P.field_stride + o], c2 = static_cast<const T*>(P.c2)[o];
+    const T xv = X[P.field_stride + o];
     const T xwx = padx ? T(0) : X[2 * P.field_stride + o], xwy = pady ? T(0) : X[3 * P.field_stride + o];
     T xu, lap, damping = T(0), hwx = T(0), hwy = T(0);
     {
@@ -342,14 +348,13 @@ __device__ __forceinline__ void forward_point(const ProblemDev& P, const StageAr
         xu = s.u();
         lap = s.laplacian();
         if (b.any) {
-            damping = -b.xn * b.yn * xu - (b.xn + b.yn) * xv;
-            hwx = (b.yn - b.xh) * s.du_x() * idx1 - b.xh * xwx;
-            hwy = (b.xn - b.yh) * s.du_y() * idx1 - b.yh * xwy;
+            damping = -mad(b.xn * b.yn, xu, (b.xn + b.yn) * xv);
+            hwx = mad((b.yn - b.xh) * idx1, s.du_x(), -(b.xh * xwx));
+            hwy = mad((b.xn - b.yh) * idx1, s.du_y(), -(b.yh * xwy));
         }
     }
-    T hv = c2 * (lap * idx2 + divergence<T, R, BAND>(P, X, i, j) * idx1);
-    if (b.any) hv += damping;
-    if (i == P.src_i && j == P.src_j && a.src_slot >= 0 && P.has_src) hv += (T)P.sigma[a.src_slot];
+    if (i == P.src_i && j == P.src_j && a.src_slot >= 0 && P.has_src) damping += (T)P.sigma[a.src_slot];
+    const T hv = mad(c2, mad(lap, idx2, divergence<T, R, BAND>(P, X, i, j) * idx1), damping);
     const T xf[4] = {xu, xv, xwx, xwy}, hf[4] = {xv, hv, hwx, hwy};
     epilogue<T, TERMS>(P, a, o, xf, hf, b.any, padx, pady);
 }
@@ -461,8 +466,10 @@ __device__ __forceinline__ void stage_point(const ProblemDev& P, const StageArgs
     if (q.i >= P.nx || q.j >= P.ny) return;
     const bool band = R == 4 && P.fs != 0 && q.j < 4;       // (a warp is one row)
     if constexpr (PASS == PASS_FORWARD) {
-        if (band) forward_point<T, R, R == 4, TERMS>(P, a, q.i, q.j);
-        else forward_point<T, R, false, TERMS>(P, a, q.i, q.j);
+        const Damping<T> b(P, q.i, q.j);
+        const T c2 = static_cast<const T*>(P.c2)[(long long)q.j * P.pitch + q.i];
+        if (band) forward_point<T, R, R == 4, TERMS>(P, a, q.i, q.j, b, c2);
+        else forward_point<T, R, false, TERMS>(P, a, q.i, q.j, b, c2);
     } else if constexpr (PASS == PASS_GRADIENT) {
         if (band) gradient_point<T, R, R == 4>(P, a, q.i, q.j);
         else gradient_point<T, R, false>(P, a, q.i, q.j);
@@ -486,6 +493,53 @@ template <typename T, int R, int PASS, int TERMS>
 __global__ void __launch_bounds__(DBX * DBY, 6)
 stage_one_kernel(const __grid_constant__ ProblemDev P, StageArgs a) {
     stage_point<T, R, PASS, TERMS>(P, a, blockIdx.x / DSUB, blockIdx.x % DSUB);
+}
+
+// --------------------------------------------------------------------------------------
+// The passes of one step in one cooperative launch (FP64, small grids).  A thread keeps its point
+// through all of them (damping, c^2 and descriptor stay in registers) and a bounded grid barrier
+// takes the place of the launch between two passes: at a few blocks per SM a pass computes for 2 to
+// 8 us, and setting a kernel up and draining it costs more than the barrier.  us a pass, launched
+// one by one and chained: HORK 8.5 -> 6.8 on 101 x 101, 11.5 -> 9.2 on 150 x 150, 13.8 -> 11.1 on
+// 250 x 200, 17.3 -> 13.1 on 251 x 251 (Faber and the Horner form likewise); HORK 12, 4th order,
+// 101 x 101, 4 steps: 367 -> 297 us.
+// bar: [0] arrivals, [1] blocks that have left; the last one clears both for the next launch.
+// --------------------------------------------------------------------------------------
+__device__ unsigned long long g_chain_wait_limit_ns = 1000000000ull;
+
+int set_chain_wait_limit_ns(unsigned long long ns) {
+    return cudaMemcpyToSymbol(g_chain_wait_limit_ns, &ns, sizeof(ns)) == cudaSuccess ? 0 : -1;
+}
+
+template <typename T, int R, int TERMS>
+__global__ void __launch_bounds__(DBX * DBY, 4)
+chain_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ tile_prob,
+             const __grid_constant__ PassChain chain, unsigned int* bar, int* err) {
+    __shared__ int s_ok;
+    const unsigned long long lim = g_chain_wait_limit_ns;
+    const int tile = blockIdx.x / DSUB;
+    const ProblemDev P = probs[tile_prob[tile]];
+    const PointAt q(P, tile - P.tile_base, blockIdx.x % DSUB);
+    const bool in = q.i < P.nx && q.j < P.ny, band = R == 4 && P.fs != 0 && q.j < 4;
+    const Damping<T> b(P, q.i, q.j);
+    const T c2 = in ? static_cast<const T*>(P.c2)[(long long)q.j * P.pitch + q.i] : T(0);
+    for (int n = 0; n < chain.n; ++n) {
+        const StageArgs a = chain_stage(chain.pass[n]);
+        if (in) {
+            if (a.terms == TERMS) {
+                if (band) forward_point<T, R, R == 4, TERMS>(P, a, q.i, q.j, b, c2);
+                else forward_point<T, R, false, TERMS>(P, a, q.i, q.j, b, c2);
+            } else {
+                if (band) forward_point<T, R, R == 4, -1>(P, a, q.i, q.j, b, c2);
+                else forward_point<T, R, false, -1>(P, a, q.i, q.j, b, c2);
+            }
+        }
+        if (n + 1 < chain.n && !grid_phase_barrier(bar, (unsigned)(n + 1), lim, &s_ok)) {
+            if (threadIdx.x == 0 && threadIdx.y == 0) atomicOr(err, 1);
+            break;
+        }
+    }
+    chain_leave(bar);
 }
 
 // --------------------------------------------------------------------------------------
@@ -631,6 +685,55 @@ int launch_stage_one(int precision, int R, const ProblemDev& P, const StageArgs&
             launch_plain(stage_one_kernel<decltype(zero), decltype(r)::value, PASS, 0>, P.ntiles * DSUB, s, P, a);
     });
     return 0;
+}
+
+template <typename T, int R, int TERMS>
+static int launch_chain_of(int blocks, const ProblemDev* probs, const int* tile_prob, const PassChain& chain,
+                           unsigned int* bar, int* err, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(blocks);
+    cfg.blockDim = dim3(DBX, DBY);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeCooperative;
+    attr[0].val.cooperative = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, chain_kernel<T, R, TERMS>, probs, tile_prob, chain, bar, err) == cudaSuccess ? 0 : -1;
+}
+
+// Grids whose passes are chained: up to four blocks per SM, which are co-resident for every
+// instantiation (128 threads, at most 128 registers).  Chaining still gains a quarter at that size;
+// larger grids (300 x 250: 20 us a pass) have no choice.
+bool chain_fits(int ntiles) {
+    int dev = 0, nsm = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess)
+        return false;
+    return coop && ntiles > 0 && ntiles * DSUB <= 4 * nsm;
+}
+
+int launch_chain(int R, int ntiles, const ProblemDev* probs, const int* tile_prob, const PassChain& chain_in,
+                 unsigned int* bar, int* err, cudaStream_t s) {
+    constexpr int FABER = TERM_CX | TERM_CU | TERM_A | TERM_CAY, HORK = TERM_CX | TERM_A | TERM_CAY;
+    static thread_local PassChain chain;        // (13 KB: not on the caller's stack)
+    chain = chain_in;
+    int count[3] = {0, 0, 0};
+    for (int n = 0; n < chain.n; ++n) {
+        const int t = chain.pass[n].terms = stage_terms(chain_stage(chain.pass[n]));
+        ++count[t == FABER ? 0 : t == HORK ? 1 : 2];
+    }
+    const int blocks = ntiles * DSUB;
+    auto go = [&](auto r) {
+        constexpr int RR = decltype(r)::value;
+        if (count[0] >= count[1] && count[0] >= count[2])
+            return launch_chain_of<double, RR, FABER>(blocks, probs, tile_prob, chain, bar, err, s);
+        if (count[1] >= count[2])
+            return launch_chain_of<double, RR, HORK>(blocks, probs, tile_prob, chain, bar, err, s);
+        return launch_chain_of<double, RR, TERM_CU>(blocks, probs, tile_prob, chain, bar, err, s);
+    };
+    return R == 4 ? go(Int<4>()) : go(Int<2>());
 }
 
 void launch_leapfrog(int R, int ntiles, const ProblemDev* probs, const int* tile_prob, int cur, int prev,
