@@ -173,8 +173,8 @@ TMA_SOURCE = os.path.join(ROOT, "paper_2401_16322_gb300", "csrc", "kernels_tma.c
 
 
 def tma_kernel_name(variant):
-    """The 2D TMA kernel a variant runs: variants 7 and up use the column-pair consumers."""
-    return "stage_tma_x2_kernel" if variant >= 7 else "stage_tma_kernel"
+    """The 2D TMA kernel a variant runs (one kernel template; the variants are tile shapes)."""
+    return "stage_tma_x2_kernel"
 
 
 def ncu_traffic_per_point(method, variant):

@@ -454,9 +454,10 @@ int ewv_batch_enable_graphs(ewv_batch_t batch, int enable);
  * 10 = (24, 12, 2); each consumer thread owns two adjacent columns (8-byte shared loads, packed
  * FP32 pair arithmetic).  11 = (24, 12, 3), 12 = (36, 9, 2), 13 = (28, 14, 3) and 14 =
  * (30, 15, 3) are composite: passes without an A operand (Horner HORK passes, Krylov products)
- * run these shapes without the A stage buffer, passes with one run variant 7 (the reported
- * shape is the no-A one), and so does 10 (passes without an A operand run 14's shape; the
- * reported shape is the one with it).  Every variant does the same arithmetic per point.  The autotuner's
+ * run these shapes without the A stage buffer, passes with A and no U (low-storage HORK stages)
+ * 14's shape without the U buffer, passes with both variant 7 (the reported shape is the no-A
+ * one).  10 is composite too: passes with both operands run its own shape (the reported one), the
+ * others 14's.  Every variant does the same arithmetic per point.  The autotuner's
  * score is the sum of a probe pass with and one without an A operand.  The leap-frog step and
  * the FWI gradient pass always run 64 x 30 tiles with 15 warps, the transposed pass 64 x 18, 24
  * or 30 by the operands it reads;

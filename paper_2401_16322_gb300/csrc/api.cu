@@ -751,7 +751,7 @@ struct Ctx {
             if (E->tma_variant < 0) {
                 launch_failed = 1;
             } else {
-                const int set = tma_map_set(tma_variant_tile_height_for(E->tma_variant, a.a >= 0));
+                const int set = tma_map_set(tma_variant_tile_height_for(E->tma_variant, a.u >= 0, a.a >= 0));
                 if (launch_stage_tma(E->tma_variant, E->R, E->d_probs, E->d_tbase + (size_t)set * (E->nprob + 1),
                                      E->nprob, E->ntiles_by[set], a, E->d_err, s) != 0)
                     launch_failed = 1;
@@ -768,16 +768,19 @@ struct Ctx {
             launch_point(E->precision, E->ntiles, E->d_probs, E->d_tile_prob, pa, s);
         ++*launches;
     }
-    // Tile-shape autotuner: time every persistent-kernel variant on two idempotent probe
-    // passes (read the state, write workspace vectors 1 and 2, which every FP32 method
-    // overwrites before reading): one with a U and an A operand (the Faber and low-storage
-    // HORK form) and one with U only (the Horner HORK form); keep the variant with the
-    // smallest sum.  Runs once per engine, outside graph capture.
+    // Tile-shape autotuner: time every persistent-kernel variant on two probe passes (read the
+    // state and workspace vectors 1 and 2, write the latter two in place, which every FP32 method
+    // overwrites before reading): one with a U and an A operand (the Faber form) and one with U only
+    // (the Horner HORK form); keep the variant with the smallest sum.  The operands are vectors of
+    // their own, as in the passes (with the state as U and A the second and third read came from the
+    // caches, and Faber 80 on 16 shots of 1001 x 501 got a shape that takes 8.88 ms instead of 8.52).
+    // The two probes are timed apart.  Runs once per engine, outside graph capture: one untimed and
+    // two timed launches each (the 72-shot batch: a first pass of 38 ms instead of 50 with three).
     void autotune() {
         StageArgs p = stage_defaults();
         p.x = 0;
-        p.u = 0;
-        p.a = 0;
+        p.u = 1;
+        p.a = 2;
         p.y_out = 1;
         p.acc_out = 2;
         p.cx = 1.0;
@@ -791,51 +794,63 @@ struct Ctx {
         pn.acc_out = -1;
         pn.ca = 0.0;
         pn.cay = 0.0;
-        cudaEvent_t e0, e1;
-        cudaEventCreate(&e0);
-        cudaEventCreate(&e1);
-        int best = -1;
-        double best_us = 1e300;
+        cudaEvent_t ev[3];
+        for (cudaEvent_t& e : ev) cudaEventCreate(&e);
+        double ta[TMA_NUM_VARIANTS], tn[TMA_NUM_VARIANTS];      // probe with A, without
         for (int v = 0; v < TMA_NUM_VARIANTS; ++v) {
-            const int set = tma_map_set(tma_variant_tile_height_for(v, true));
-            const int setn = tma_map_set(tma_variant_tile_height_for(v, false));
+            ta[v] = tn[v] = -1.0;
+            if (tma_variant_shape(v) != v) continue;            // timed under the variant it repeats
+            const int set = tma_map_set(tma_variant_tile_height_for(v, true, true));
+            const int setn = tma_map_set(tma_variant_tile_height_for(v, true, false));
             const int* tb = E->d_tbase + (size_t)set * (E->nprob + 1);
             const int* tbn = E->d_tbase + (size_t)setn * (E->nprob + 1);
             if (launch_stage_tma(v, E->R, E->d_probs, tb, E->nprob, E->ntiles_by[set], p, E->d_err, s) != 0 ||
                 launch_stage_tma(v, E->R, E->d_probs, tbn, E->nprob, E->ntiles_by[setn], pn, E->d_err, s) != 0 ||
-                cudaGetLastError() != cudaSuccess) {
-                E->tma_variant_us[v] = -1.0;
+                cudaGetLastError() != cudaSuccess)
                 continue;
-            }
-            double best_v = 1e300;
-            for (int rep = 0; rep < 3; ++rep) {
-                cudaEventRecord(e0, s);
+            double best_a = 1e300, best_n = 1e300;
+            for (int rep = 0; rep < 2; ++rep) {
+                cudaEventRecord(ev[0], s);
                 launch_stage_tma(v, E->R, E->d_probs, tb, E->nprob, E->ntiles_by[set], p, E->d_err, s);
+                cudaEventRecord(ev[1], s);
                 launch_stage_tma(v, E->R, E->d_probs, tbn, E->nprob, E->ntiles_by[setn], pn, E->d_err, s);
-                cudaEventRecord(e1, s);
-                cudaEventSynchronize(e1);
-                float ms = 0.f;
-                cudaEventElapsedTime(&ms, e0, e1);
-                best_v = std::min(best_v, 1e3 * (double)ms);
+                cudaEventRecord(ev[2], s);
+                cudaEventSynchronize(ev[2]);
+                float ma = 0.f, mn = 0.f;
+                cudaEventElapsedTime(&ma, ev[0], ev[1]);
+                cudaEventElapsedTime(&mn, ev[1], ev[2]);
+                best_a = std::min(best_a, 1e3 * (double)ma);
+                best_n = std::min(best_n, 1e3 * (double)mn);
             }
+            *launches += 6;
             // a variant whose pipeline wait gave up is not a candidate (clear its flag)
             int flag = 0;
             if (cudaMemcpyAsync(&flag, E->d_err, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
                 cudaStreamSynchronize(s) != cudaSuccess || flag != 0) {
                 cudaMemsetAsync(E->d_err, 0, sizeof(int), s);
-                E->tma_variant_us[v] = -1.0;
                 continue;
             }
-            E->tma_variant_us[v] = best_v;
-            if (best_v < best_us) {
-                best_us = best_v;
-                best = v;
-            }
+            ta[v] = best_a;
+            tn[v] = best_n;
         }
-        cudaEventDestroy(e0);
-        cudaEventDestroy(e1);
+        for (cudaEvent_t& e : ev) cudaEventDestroy(e);
+        // a shape's time is the smallest seen of it: variants that run a pass on the same shape
+        // differ only by the other pass, not by noise
+        auto same_shape = [&](double* t, bool reads_a) {
+            for (int v = 0; v < TMA_NUM_VARIANTS; ++v)
+                for (int w = 0; w < TMA_NUM_VARIANTS; ++w)
+                    if (t[v] > 0.0 && t[w] > 0.0 && tma_pass_shape(v, true, reads_a) == tma_pass_shape(w, true, reads_a))
+                        t[v] = t[w] = std::min(t[v], t[w]);
+        };
+        same_shape(ta, true);
+        same_shape(tn, false);
+        int best = -1;
+        for (int v = 0; v < TMA_NUM_VARIANTS; ++v) {
+            const int w = tma_variant_shape(v);
+            E->tma_variant_us[v] = ta[w] > 0.0 ? ta[w] + tn[w] : -1.0;
+            if (ta[w] > 0.0 && (best < 0 || E->tma_variant_us[v] < E->tma_variant_us[best])) best = v;
+        }
         E->tma_variant = best;
-        *launches += 8 * TMA_NUM_VARIANTS;
     }
     void copy(int src, int dst, int fmask, bool swap) {
         PointArgs pa{};
@@ -2590,7 +2605,7 @@ static int adjoint_krylov(ewv_model* m, Engine* E, double t, double dt, int mm, 
                                    0.66999052179242813, 0.93056815579702629};
     static const double kW[4] = {0.17392742256872693, 0.32607257743127307,
                                  0.32607257743127307, 0.17392742256872693};
-    const int fset = tma ? tma_map_set(tma_variant_tile_height_for(E->tma_variant, false)) : 0;
+    const int fset = tma ? tma_map_set(tma_variant_tile_height_for(E->tma_variant, false, false)) : 0;
     const int trset = tma_map_set(tma_transpose_height(false, false)), gset = tma_map_set(30);
     const int rc_gs = gs_ready(E, m->err);
     if (rc_gs != EWV_OK) return rc_gs;
@@ -3007,7 +3022,7 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
                                              cudaMemcpyHostToDevice, s));
     }
     auto tset_of = [&](const StageArgs& sa) {
-        return tma_map_set(tma_variant_tile_height_for(E->tma_variant, sa.a >= 0));
+        return tma_map_set(tma_variant_tile_height_for(E->tma_variant, sa.u >= 0, sa.a >= 0));
     };
     const int gset = tma_map_set(30);
     auto stage = [&](const StageArgs& sa) {
@@ -3044,7 +3059,7 @@ static int adjoint_step_impl(ewv_model_t m, int method, double t, double dt, int
     bool tape_failed = false;
     auto tape_pass = [&](StageArgs sa, int i) {
         const int v = tma_tape_variant(E->tma_variant);
-        const int set = tma_map_set(tma_variant_tile_height_for(v, false));
+        const int set = tma_map_set(tma_variant_tile_height_for(v, sa.u >= 0, false));
         sa.tape_vec = 3 + i / 4;
         sa.tape_field = i % 4;
         if (launch_stage_tma(v, R, E->d_adj, E->d_tbase + (size_t)set * (E->nprob + 1), ns, E->ntiles_by[set], sa,

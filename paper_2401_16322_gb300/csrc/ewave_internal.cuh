@@ -262,7 +262,9 @@ int tma_variant_tile_height(int v);
 int tma_tape_variant(int v);   // the variant that writes a gradient tape when v is selected (column pairs)
 // Tile height of variant v for a pass that does (reads_a) or does not read an A operand
 // (composite variants pick their tile by it).
-int tma_variant_tile_height_for(int v, bool reads_a);
+int tma_variant_tile_height_for(int v, bool reads_u, bool reads_a);
+int tma_variant_shape(int v);       // the variant whose shapes v repeats (v itself: its own)
+int tma_pass_shape(int v, bool reads_u, bool reads_a);   // the shape a pass runs on under variant v
 // Tile heights of the 2D TMA map sets (set k has tile height TMA_SET_HEIGHTS[k]).
 constexpr int TMA_NUM_SETS = 8;
 constexpr int TMA_SET_HEIGHTS[TMA_NUM_SETS] = {16, 8, 20, 18, 24, 36, 28, 30};

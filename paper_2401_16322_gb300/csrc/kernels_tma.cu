@@ -1329,10 +1329,25 @@ constexpr TmaVariant kVariants[TMA_NUM_VARIANTS] = {
 
 static bool composite(int v) { return v >= 11 && v <= 14; }
 
-int tma_variant_tile_height_for(int v, bool reads_a) {
-    if (composite(v) && reads_a) return kVariants[7].by;
-    if (v == 10 && !reads_a) return kVariants[14].by;
-    return kVariants[v].by;
+// A pass with an A operand and no U (the low-storage HORK stages) needs as many stage buffers as
+// one with U and no A: the composite variants and 10 run it on 14's tall tiles.  HORK 20, 16 shots of
+// 803 x 397: 1240 us a step (24 rows with both buffers and two stages: 1272; variant 7's shape: 1302).
+static bool a_only_on_tall(int v, bool reads_u, bool reads_a) {
+    return (composite(v) || v == 10) && reads_a && !reads_u;
+}
+
+constexpr int A_ONLY_TALL = TMA_NUM_VARIANTS;   // (64 x 30, 15 warps, 3 stages, no U buffer)
+int tma_variant_shape(int v) { return v == 1 ? 8 : v == 6 ? 9 : v; }
+int tma_pass_shape(int v, bool reads_u, bool reads_a) {
+    if (a_only_on_tall(v, reads_u, reads_a)) return A_ONLY_TALL;
+    if (composite(v) && reads_a) return 7;
+    if (v == 10 && !reads_a) return 14;
+    if (v == 4 && reads_u) return 0;                // no U buffer
+    return tma_variant_shape(v);
+}
+int tma_variant_tile_height_for(int v, bool reads_u, bool reads_a) {
+    const int shape = tma_pass_shape(v, reads_u, reads_a);
+    return shape == A_ONLY_TALL ? 30 : kVariants[shape].by;
 }
 
 int tma_variant_tile_height(int v) { return kVariants[v].by; }
@@ -1505,12 +1520,7 @@ int launch_stage_tma(int variant, int R, const ProblemDev* probs, const int* tba
     }
     // the steady-state Faber / HORK form: Y = cu U + cx X + ch H, ACC = ca A + cay Y
     const bool epi = a.ck == 1.0 && a.cau == 0.0 && a.cak == 0.0 && a.cax == 0.0;
-    if (composite(variant) && a.a >= 0) variant = 7;   // composite, pass with A
-    if (variant == 10 && a.a < 0) variant = 14;
-    if (variant == 4 && a.u >= 0) variant = 0;         // no U buffer
-    // the shapes that repeat another one's
-    if (variant == 1) variant = 8;
-    if (variant == 6) variant = 9;
+    variant = tma_pass_shape(variant, a.u >= 0, a.a >= 0);
 #define EWV_TMA_CASE2(V, RR, BYV, NWV, NSTV, HASA, HASU)                                                   \
     if (variant == V && R == RR)                                                                         \
         return epi ? launch_x2<RR, BYV, NWV, NSTV, 1, HASA, HASU>(probs, tbase, nprob, ntiles, a, err, s) \
@@ -1518,6 +1528,7 @@ int launch_stage_tma(int variant, int R, const ProblemDev* probs, const int* tba
 #define EWV_TMA_CASE(V, BYV, NWV, NSTV, HASA, HASU)  \
     EWV_TMA_CASE2(V, 4, BYV, NWV, NSTV, HASA, HASU) \
     EWV_TMA_CASE2(V, 2, BYV, NWV, NSTV, HASA, HASU)
+    EWV_TMA_CASE(A_ONLY_TALL, 30, 15, 3, true, false)
     EWV_TMA_CASE(0, 16, 16, 3, true, true)
     EWV_TMA_CASE(2, 8, 8, 5, true, true)
     EWV_TMA_CASE(3, 8, 4, 5, true, true)
