@@ -359,10 +359,16 @@ class Model:
 
     # ---------------------------------------------------------------- compute
     def apply_device(self, x, y, transpose=False):
+        """y = H x (or H^T x) on the model's stream, for padded device vectors of the caller's.
+        Where the caller's current stream is another one, the product starts after what is queued
+        there (x may still be being written, y still read) and is complete on return."""
+        caller = self.torch.cuda.current_stream(self.stream.device_index)
+        if caller != self.stream:
+            self.stream.wait_stream(caller)
         self._check(self.lib.ewv_apply_operator(self.h, int(transpose), x.data_ptr(), y.data_ptr()),
                     "apply_operator")
-        if self.stream.cuda_stream != self.torch._C._cuda_getCurrentRawStream(self.stream.device_index):
-            self.stream.synchronize()    # x and y belong to the caller's stream
+        if caller != self.stream:
+            self.stream.synchronize()
 
     def apply(self, compact, transpose=False):
         x, y = self.new_vector(), self.new_vector()

@@ -1,0 +1,57 @@
+"""H x on a caller's vectors when other work is queued: a model whose stream is not the caller's
+takes x when the caller's stream has written it and overwrites y when the caller's stream has
+read it."""
+import numpy as np
+import pytest
+
+from _helpers import TOL, flatten, oracle_model, rel_l2
+from oracle.operator import assemble_H
+from paper_2401_16322_gb300.workloads import layered, smooth_random_state
+
+pytestmark = pytest.mark.gpu
+
+
+def _busy():
+    """Some tens of milliseconds of work on the current stream."""
+    import torch
+    a = torch.full((4096, 4096), 1e-4, device="cuda")
+    b = a
+    for _ in range(30):
+        b = b @ a
+    return b
+
+
+def _case(stream):
+    import torch
+    from paper_2401_16322_gb300 import Model
+    om = oracle_model(97, 65, layered(97, 65, 3), pml=10, fs=True)
+    g = Model(om.nx, om.ny, om.dx, om.order, om.pml, om.beta0, True, precision="f64", stream=stream)
+    g.set_velocity(om.c)
+    x = flatten(smooth_random_state([f.shape for f in om.zeros_state()], 11))
+    src, dx, dy = g.new_vector(), g.new_vector(), g.new_vector()
+    g.pack(x, src)
+    _busy()                                        # (loads the library's kernels)
+    g.apply_device(src, dy)
+    dy.fill_(3.0)
+    torch.cuda.synchronize()
+    return om, g, x, src, dx, dy
+
+
+@pytest.mark.parametrize("model_on", ["own stream", "current stream"])
+@pytest.mark.parametrize("transpose", [False, True])
+def test_operands_are_ordered_against_the_callers_stream(model_on, transpose):
+    """No synchronisation between the caller's work and the product, on either side."""
+    import torch
+    om, g, x, src, dx, dy = _case(torch.cuda.Stream() if model_on == "own stream" else None)
+    caller = torch.cuda.current_stream() if model_on == "own stream" else torch.cuda.Stream()
+    with torch.cuda.stream(caller):
+        _busy()
+        old = dy.clone()                           # reads y before the product
+        dx.copy_(src)                              # writes x before the product
+        g.apply_device(dx, dy, transpose)
+        new = dy.clone()                           # reads y after it
+    torch.cuda.synchronize()
+    H = assemble_H(om)
+    assert bool((old == 3.0).all())
+    assert rel_l2(g.unpack(new), (H.T if transpose else H) @ x) < TOL["f64"]
+    g.close()
