@@ -211,6 +211,9 @@ class Model:
             self._check(self.lib.ewv_create_model(ctypes.byref(d), ctypes.byref(h)), "create_model")
         self.h = h
         self.stream = stream if stream is not None else torch.cuda.current_stream(self.device)
+        # the current stream's handle: the public call builds a Stream object, 1.1 us against 0.05
+        self._raw_current = (getattr(torch._C, "_cuda_getCurrentRawStream", None)
+                             or (lambda index: torch.cuda.current_stream(index).cuda_stream))
         self._check(self.lib.ewv_set_stream(self.h, ctypes.c_void_p(self.stream.cuda_stream)))
         lay = LayoutInfo()
         self._check(self.lib.ewv_layout(self.h, ctypes.byref(lay)))
@@ -361,14 +364,20 @@ class Model:
     def apply_device(self, x, y, transpose=False):
         """y = H x (or H^T x) on the model's stream, for padded device vectors of the caller's.
         Where the caller's current stream is another one, the product starts after what is queued
-        there (x may still be being written, y still read) and is complete on return."""
-        caller = self.torch.cuda.current_stream(self.stream.device_index)
-        if caller != self.stream:
-            self.stream.wait_stream(caller)
-        self._check(self.lib.ewv_apply_operator(self.h, int(transpose), x.data_ptr(), y.data_ptr()),
-                    "apply_operator")
-        if caller != self.stream:
-            self.stream.synchronize()
+        there (x may still be being written, y still read) and is complete on return.  Otherwise it
+        is only enqueued, and x and y may be freed at once, whichever stream they come from."""
+        s = self.stream
+        other = self._raw_current(s.device_index) != s.cuda_stream
+        if other:
+            s.wait_stream(self.torch.cuda.current_stream(s.device_index))
+        rc = self.lib.ewv_apply_operator(self.h, 1 if transpose else 0, x.data_ptr(), y.data_ptr())
+        if other:
+            s.synchronize()
+        else:
+            x.record_stream(s)     # (nothing to do for memory of this stream)
+            y.record_stream(s)
+        if rc:
+            self._check(rc, "apply_operator")
 
     def apply(self, compact, transpose=False):
         x, y = self.new_vector(), self.new_vector()

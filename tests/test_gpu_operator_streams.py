@@ -1,6 +1,6 @@
 """H x on a caller's vectors when other work is queued: a model whose stream is not the caller's
 takes x when the caller's stream has written it and overwrites y when the caller's stream has
-read it."""
+read it; and vectors that come from another stream's memory outlive the product."""
 import numpy as np
 import pytest
 
@@ -54,4 +54,32 @@ def test_operands_are_ordered_against_the_callers_stream(model_on, transpose):
     H = assemble_H(om)
     assert bool((old == 3.0).all())
     assert rel_l2(g.unpack(new), (H.T if transpose else H) @ x) < TOL["f64"]
+    g.close()
+
+
+@pytest.mark.parametrize("which", ["x", "y"])
+def test_vectors_of_another_stream_may_be_freed_after_the_call(which):
+    """The vector is allocated on a side stream, whose next allocation would take its place while
+    the product waits behind other work."""
+    import torch
+    om, g, x, src, dx, dy = _case(None)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        v = torch.empty_like(src)
+        if which == "x":
+            v.copy_(src)
+    torch.cuda.synchronize()
+    _busy()
+    if which == "x":
+        g.apply_device(v, dy)
+        del v
+    else:
+        g.apply_device(src, v)
+        del v
+    with torch.cuda.stream(side):
+        other = [torch.full_like(src, 5.0) for _ in range(4)]
+    torch.cuda.synchronize()
+    if which == "x":
+        assert rel_l2(g.unpack(dy), assemble_H(om) @ x) < TOL["f64"]
+    assert all(bool((o == 5.0).all()) for o in other)     # (y: written by nobody else)
     g.close()
