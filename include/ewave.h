@@ -224,8 +224,13 @@ int ewv_set_storage_rounding(ewv_model_t model, int mode);
 /* ---- operator (Eq. 1, Secs. 2.1-2.2) ------------------------------------------------- */
 
 /* y = H x (transpose = 0) or y = H^T x (transpose = 1) for padded device vectors x, y of
- * this model (no source term).  x and y must not overlap. */
+ * this model (no source term).  x and y must not overlap.  The product runs on the model's
+ * stream after what is queued there (work of other streams on x or y is the caller's to order
+ * before it), and the call returns with y complete. */
 int ewv_apply_operator(ewv_model_t model, int transpose, const void* x, void* y);
+/* The same without the wait at the end: the product is enqueued on the model's stream, and x
+ * and y must stay valid until that stream has passed it.  (3D models: the call waits.) */
+int ewv_apply_operator_async(ewv_model_t model, int transpose, const void* x, void* y);
 
 /* ---- time integrators: advance every shot by nsteps steps of dt from time t --------- */
 

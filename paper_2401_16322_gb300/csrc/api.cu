@@ -2230,6 +2230,13 @@ int ewv_get_state(ewv_model_t m, int shot, double* host, size_t n) {
 }
 
 int ewv_apply_operator(ewv_model_t m, int transpose, const void* x, void* y) {
+    const int rc = ewv_apply_operator_async(m, transpose, x, y);
+    if (rc != EWV_OK) return rc;
+    CUDA_OR_FAIL(m->err, cudaStreamSynchronize(m->stream));
+    return EWV_OK;
+}
+
+int ewv_apply_operator_async(ewv_model_t m, int transpose, const void* x, void* y) {
     if (!m || !x || !y || x == y) return EWV_ERR_INVALID_ARG;
     if (!aligned(x) || !aligned(y)) return fail(m->err, EWV_ERR_BAD_SIZE_OR_ALIGNMENT, "x, y must be 256-B aligned");
     if (!m->params || !m->velocity_set) return fail(m->err, EWV_ERR_NOT_BOUND, "velocity not set");

@@ -31,7 +31,8 @@ EXPORTS = [
     "ewv_workspace_bytes", "ewv_bind_buffers", "ewv_bind_workspace", "ewv_bind_seismogram",
     "ewv_reset_recording", "ewv_set_velocity", "ewv_set_source_receivers",
     "ewv_set_faber_ellipse", "ewv_get_faber_ellipse", "ewv_set_state", "ewv_get_state",
-    "ewv_pack_vector", "ewv_unpack_vector", "ewv_apply_operator", "ewv_step_faber",
+    "ewv_pack_vector", "ewv_unpack_vector", "ewv_apply_operator", "ewv_apply_operator_async",
+    "ewv_step_faber",
     "ewv_step_krylov", "ewv_step_rk", "ewv_step_leapfrog", "ewv_set_leapfrog_variant",
     "ewv_create_batch", "ewv_destroy_batch", "ewv_batch_set_stream", "ewv_batch_step_faber",
     "ewv_batch_step_krylov", "ewv_batch_step_rk", "ewv_batch_step_leapfrog", "ewv_last_error",
@@ -117,6 +118,7 @@ def load_library(path=LIB_PATH):
         "ewv_pack_vector": ([vp, dp, sz, vp], i),
         "ewv_unpack_vector": ([vp, vp, dp, sz], i),
         "ewv_apply_operator": ([vp, i, vp, vp], i),
+        "ewv_apply_operator_async": ([vp, i, vp, vp], i),
         "ewv_step_faber": ([vp, d, d, i, i], i),
         "ewv_step_krylov": ([vp, d, d, i, i, ctypes.POINTER(i)], i),
         "ewv_step_rk": ([vp, d, d, i, i, i], i),
@@ -370,7 +372,7 @@ class Model:
         other = self._raw_current(s.device_index) != s.cuda_stream
         if other:
             s.wait_stream(self.torch.cuda.current_stream(s.device_index))
-        rc = self.lib.ewv_apply_operator(self.h, 1 if transpose else 0, x.data_ptr(), y.data_ptr())
+        rc = self.lib.ewv_apply_operator_async(self.h, 1 if transpose else 0, x.data_ptr(), y.data_ptr())
         if other:
             s.synchronize()
         else:

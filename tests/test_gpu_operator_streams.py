@@ -1,6 +1,7 @@
 """H x on a caller's vectors when other work is queued: a model whose stream is not the caller's
 takes x when the caller's stream has written it and overwrites y when the caller's stream has
-read it; and vectors that come from another stream's memory outlive the product."""
+read it; and vectors that come from another stream's memory outlive the product; and the
+C entry returns with y complete."""
 import numpy as np
 import pytest
 
@@ -82,4 +83,22 @@ def test_vectors_of_another_stream_may_be_freed_after_the_call(which):
     if which == "x":
         assert rel_l2(g.unpack(dy), assemble_H(om) @ x) < TOL["f64"]
     assert all(bool((o == 5.0).all()) for o in other)     # (y: written by nobody else)
+    g.close()
+
+
+@pytest.mark.parametrize("transpose", [0, 1])
+def test_c_entry_returns_with_y_complete(transpose):
+    """The model's stream is busy when the product is asked for; on return y can be read on any
+    stream."""
+    import torch
+    s = torch.cuda.Stream()
+    om, g, x, src, dx, dy = _case(s)
+    with torch.cuda.stream(s):
+        _busy()
+        dx.copy_(src)
+    assert g.lib.ewv_apply_operator(g.h, transpose, dx.data_ptr(), dy.data_ptr()) == 0
+    assert s.query()
+    y = dy.clone()
+    H = assemble_H(om)
+    assert rel_l2(g.unpack(y), (H.T if transpose else H) @ x) < TOL["f64"]
     g.close()
