@@ -16,6 +16,7 @@
 
 #include "../../include/ewave.h"
 #include "ewave_internal.cuh"
+#include "pass_queue.hpp"
 
 
 using namespace ewv;
@@ -689,36 +690,32 @@ struct Ctx {
         ++*launches;
     }
     // Chained passes (small 2D FP64 engines): the stage() calls between chain_begin and chain_end
-    // go out as one cooperative launch.  Not while passes are timed one by one.
-    PassChain chain;
-    bool chaining = false;
-    void chain_begin() {
-        chaining = E->chain_ok && !E->timing;
-        chain.n = 0;
-    }
+    // go out as one cooperative launch.  Not while passes are timed one by one.  Where no
+    // cooperative launch is to be had, pass by pass, for this engine from then on.
+    PassQueue<PassChain> queue;
+    void chain_begin() { queue.begin(E->chain_ok && !E->timing); }
     void chain_end() {
-        if (!chaining) return;
-        chaining = false;
-        if (chain.n == 0) return;
-        if (launch_chain(E->R, E->ntiles, E->d_probs, E->d_tile_prob, chain, E->d_chain_bar, E->d_err, s) == 0) {
-            ++*launches;
-            return;
-        }
-        cudaGetLastError();         // no cooperative launch to be had: pass by pass
-        E->chain_ok = false;
-        for (int n = 0; n < chain.n; ++n) stage(chain_stage(chain.pass[n]));
+        queue.end([this](const PassChain& c) { return send_chain(c); }, [this](const ChainPass& c) { send(chain_stage(c)); });
     }
-    void stage(const StageArgs& a_in) {
-        if (chaining) {
-            if (chain.n == MAX_CHAIN) {
-                chain_end();
-                chain_begin();
-            }
-            ChainPass& c = chain.pass[chain.n++];
-            c = ChainPass{a_in.x, a_in.u, a_in.a, a_in.y_out, a_in.acc_out, a_in.src_slot, 0, 0,
-                          a_in.cx, a_in.ch, a_in.cu, a_in.ck, a_in.ca, a_in.cau, a_in.cak, a_in.cay, a_in.cax};
+    bool send_chain(const PassChain& c) {
+        if (launch_chain(E->R, E->ntiles, E->d_probs, E->d_tile_prob, c, E->d_chain_bar, E->d_err, s) != 0) {
+            cudaGetLastError();
+            E->chain_ok = false;
+            return false;
+        }
+        ++*launches;
+        return true;
+    }
+    void stage(const StageArgs& a) {
+        if (!queue.collecting()) {
+            send(a);
             return;
         }
+        queue.add(ChainPass{a.x, a.u, a.a, a.y_out, a.acc_out, a.src_slot, 0, 0, a.cx, a.ch, a.cu, a.ck, a.ca, a.cau,
+                            a.cak, a.cay, a.cax},
+                  [this](const PassChain& c) { return send_chain(c); }, [this](const ChainPass& c) { send(chain_stage(c)); });
+    }
+    void send(const StageArgs& a_in) {
         StageArgs a = a_in;
         a.store_bf16 = E->store_bf16;
         cudaEvent_t e0 = nullptr, e1 = nullptr;

@@ -144,10 +144,10 @@ struct ChainPass {
     int x, u, a, y_out, acc_out, src_slot, terms, pad;
     double cx, ch, cu, ck, ca, cau, cak, cay, cax;
 };
-constexpr int MAX_CHAIN = 128;
 struct PassChain {
+    static constexpr int capacity = 128;
     int n, pad;
-    ChainPass pass[MAX_CHAIN];
+    ChainPass pass[capacity];
 };
 __host__ __device__ inline StageArgs chain_stage(const ChainPass& c) {
     StageArgs a{};
