@@ -86,12 +86,33 @@ struct DotSum<float4> {
         return (double)h + (double)l;
     }
 };
-// Block-wide total (fixed order), valid on thread 0; red: one double per warp.  Called by all threads.
+// (the exponent's bits: a comparison of FP64 values would occupy the FP64 pipe)
+__device__ __forceinline__ bool out_of_range(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+
+// sum <a[q], b[q]> over the vectors q < n that the warp's lanes visit (q = lane's thread number, + NTHREADS,
+// ...), accumulated in FP64 by one thread.
 template <typename V>
-__device__ __forceinline__ double block_total(const DotSum<V>& d, double* red) {
+__device__ __forceinline__ double warp_dot_in_fp64(const V* a, const V* b, int n, int warp) {
+    double s = 0.0;
+    if constexpr (sizeof(a->x) == 4)
+        for (int q0 = 32 * warp; q0 < n; q0 += NTHREADS)
+            for (int q = q0; q < q0 + 32 && q < n; ++q) s += (double)dot16(a[q], b[q]);
+    return s;
+}
+
+// Block-wide total (fixed order), valid on thread 0; red: one double per warp.  Called by all threads.
+// again(warp): the warp's sum from memory in FP64 (warp_dot_in_fp64), for FP32 pairs that left their
+// range: a pair holds a warp's sum up to 3.4e38, a 256th of what the sums of four products that make
+// it up may reach.
+template <typename V, class F>
+__device__ __forceinline__ double block_total(const DotSum<V>& d, double* red, F&& again) {
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
-    const double w = d.warp_total();
-    if ((tid & 31) == 0) red[tid >> 5] = w;
+    double w = d.warp_total();
+    if ((tid & 31) == 0) {
+        if constexpr (sizeof(V) / sizeof(decltype(V::x)) == 4)
+            if (out_of_range(w)) w = again(tid >> 5);
+        red[tid >> 5] = w;
+    }
     __syncthreads();
     double s = 0.0;
     if (tid == 0)

@@ -472,7 +472,13 @@ point_flat_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
         }
     }
     if (pa.mode == 1 && pa.k == pa.j && pa.j == pa.m) return;   // h_{m+1,m} unused
-    const double bsum = block_total(acc, red);
+    if (pa.mode == 1) __syncwarp();    // (the sum may be formed again from what the other lanes stored)
+    const double bsum = block_total(acc, red, [&](int warp) {
+        const int a = pa.mode == 0 ? 0 : pa.j;
+        const int b = pa.mode == 5 ? pa.k - 1 : pa.mode == 1 && pa.k < pa.j ? pa.k : a;
+        return warp_dot_in_fp64(reinterpret_cast<const V*>(vptr<T>(P, a)) + q0,
+                                reinterpret_cast<const V*>(vptr<T>(P, b)) + q0, (int)(q1 - q0), warp);
+    });
     StageArgs a{};
     a.fin_mode = pa.mode == 0 ? (pa.notail == 2 ? FIN_NORM0_TAIL : pa.notail ? FIN_NORM0_NOTAIL : FIN_NORM0)
                : pa.mode == 7 ? FIN_STORE_NORM

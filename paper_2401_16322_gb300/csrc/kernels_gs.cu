@@ -84,6 +84,19 @@ __device__ __forceinline__ void dot_chunk(const float4 (&a)[GS_VPT], const float
     for (int i = 0; i < GS_VPT; ++i) two_sum_add(hi, lo, dot16(a[i], b[i]));
 }
 
+// The sums of a chunk once more, in FP64, where a pair left its range (flat_vec.cuh): a thread per sum.
+__device__ __noinline__ void dots_in_fp64(const ProblemDev* P, long long q0, int nv, int j, int k0, double* partials,
+                                          size_t stride) {
+    auto vec = [&](int k) { return reinterpret_cast<const float4*>(vptr<float>(P, k - 1)) + q0; };   // slot k
+    for (int v = threadIdx.x; v < 2 * (j - k0) + 1; v += NTHREADS) {
+        const float4* a = vec((v & 1) ? j : j + 1);
+        const float4* b = vec(k0 + (v >> 1));
+        double s = 0.0;
+        for (int q = 0; q < nv; ++q) s += (double)dot16(a[q], b[q]);
+        partials[(size_t)v * stride] = s;
+    }
+}
+
 // One warp: column j of H and row j of L from the totals d[k - k0] = <q_{j+1}, q_k> (k = k0 .. j)
 // and l[k - k0] = <q_j, q_k> (k = k0 .. j - 1); tail_{j+1} = J (s_j tail_j) less the h_k v_k tails of
 // k = k0 .. j - 1 (the update's finalisation takes k = j).  sh: MAX_M doubles of shared memory.
@@ -143,7 +156,7 @@ gs_dots_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ pba
     __shared__ float2 sred[2 * GS_BATCH][NTHREADS];
     __shared__ double s_tot[2 * MAX_M];
     __shared__ double s_h[MAX_M];
-    __shared__ int s_last;
+    __shared__ int s_last, s_out;      // s_out: a sum left the range of the pairs
     const Chunk c(probs, pbase, nprob, (int)(gridDim.x - 1 - blockIdx.x));
     const ProblemDev* P = probs + c.pid;
     if (P->kry[KRY_ACTIVE] == 0.0) return;       // Arnoldi stopped
@@ -152,6 +165,7 @@ gs_dots_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ pba
     float4 w[GS_VPT], p[GS_VPT];
     load_chunk(w, reinterpret_cast<const float4*>(vptr<float>(P, j)), c, tid);          // slot j+1
     load_chunk(p, reinterpret_cast<const float4*>(vptr<float>(P, j - 1)), c, tid);      // slot j
+    if (tid == 0) s_out = 0;
     // sums 2 (k - k0) and 2 (k - k0) + 1: <w, q_k> and <q_j, q_k>
     for (int b0 = 0; b0 < n; b0 += GS_BATCH) {
         for (int b = b0; b < n && b < b0 + GS_BATCH; ++b) {
@@ -178,8 +192,16 @@ gs_dots_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ pba
             }
             double v = (double)hi + (double)lo;
             for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-            if (lane == 0) ga.partials[(size_t)(2 * b0 + warp) * gridDim.x + c.slot] = v;
+            if (lane == 0) {
+                ga.partials[(size_t)(2 * b0 + warp) * gridDim.x + c.slot] = v;
+                if (out_of_range(v)) s_out = 1;
+            }
         }
+        __syncthreads();
+    }
+    if (s_out) {                       // (rare, and the same in every thread)
+        dots_in_fp64(P, c.q0, c.n, j, k0, ga.partials + c.slot, gridDim.x);
+        __threadfence();
         __syncthreads();
     }
     // the problem's last block sums every total in a fixed order and solves for the column
@@ -245,7 +267,11 @@ gs_update_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ p
         if (tid + i * NTHREADS < c.n) W[c.q0 + tid + i * NTHREADS] = w[i];
         acc.add(w[i], w[i]);
     }
-    const double bsum = block_total(acc, red);
+    __syncwarp();
+    const double bsum = block_total(acc, red, [&](int warp) {
+        const float4* wc = reinterpret_cast<const float4*>(vptr<float>(P, j)) + c.q0;
+        return warp_dot_in_fp64(wc, wc, c.n, warp);
+    });
     StageArgs a{};
     a.fin_mode = FIN_MGS;
     a.fin_j = j;

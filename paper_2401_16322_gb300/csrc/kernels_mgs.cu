@@ -121,7 +121,10 @@ mgs_column_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
             ws[q - q0] = w;
             acc.add(w, D[q]);
         }
-        const double bsum = block_total(acc, red);
+        __syncwarp();
+        const double bsum = block_total(acc, red, [&](int warp) {
+            return warp_dot_in_fp64(static_cast<const V*>(ws), D + q0, (int)(q1 - q0), warp);
+        });
         if (tid == 0) ma.partials[g] = bsum;
         double* kry = P->kry;
         if (tid < P->p) {
@@ -199,7 +202,12 @@ mgs_column_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__ 
                 ws[q - q0] = w;
                 acc.add(w, Qn ? qn : w);
             }
-            const double bsum = block_total(acc, red);
+            __syncwarp();
+            const double bsum = block_total(acc, red, [&](int warp) {
+                const V* w = wsh + (size_t)sl * QPC;
+                const V* b = k < j ? reinterpret_cast<const V*>(vptr<T>(P, k)) + q0 : w;
+                return warp_dot_in_fp64(w, b, (int)(q1 - q0), warp);
+            });
             if (tid == 0) part[g] = bsum;
             double* kry = P->kry;
             if (tid < P->p) {
