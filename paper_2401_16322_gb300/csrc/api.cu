@@ -12,6 +12,7 @@
 #include <memory>
 #include <string>
 #include <tuple>
+#include <unordered_map>
 #include <vector>
 
 #include "../../include/ewave.h"
@@ -173,6 +174,7 @@ struct ewv_model {
     bool lf_history_valid = false;
     // device metadata
     int* d_rec = nullptr;
+    int* d_link = nullptr;      // from a receiver to the next on its node (inject_kernel)
     int* d_nrec = nullptr;      // receivers per shot
     double* d_sigma = nullptr;
     float* d_btab = nullptr;    // damping profile at half-cell distances (FP32 models)
@@ -1902,6 +1904,7 @@ int ewv_create_model(const ewv_model_desc* desc, ewv_model_t* out) {
     const int nr = d.max_receivers > 0 ? d.max_receivers : 1;
     cudaError_t e = cudaSuccess;
     if (e == cudaSuccess) e = cudaMalloc(&m->d_rec, sizeof(int) * (size_t)nr * d.nshots);
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_link, sizeof(int) * (size_t)nr * d.nshots);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_nrec, sizeof(int) * (size_t)d.nshots);
     if (e == cudaSuccess) e = cudaMemset(m->d_nrec, 0, sizeof(int) * (size_t)d.nshots);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_sigma, sizeof(double) * (size_t)MAX_SIGMA * d.nshots);
@@ -1940,6 +1943,7 @@ int ewv_destroy_model(ewv_model_t m) {
     if (!m) return EWV_ERR_INVALID_ARG;
     delete m->engine;
     cudaFree(m->d_rec);
+    cudaFree(m->d_link);
     cudaFree(m->d_nrec);
     cudaFree(m->d_sigma);
     cudaFree(m->d_btab);
@@ -2111,9 +2115,22 @@ static int set_src_rec(ewv_model_t m, int shot, const double* spos, double f_pea
     s.t0 = t0;
     s.amp = amp;
     s.rec_off = off;
-    if (nrec > 0)
-        CUDA_OR_FAIL(m->err, cudaMemcpy(m->d_rec + (size_t)shot * m->d.max_receivers, off.data(),
-                                        sizeof(int) * nrec, cudaMemcpyHostToDevice));
+    // receivers of one node, in order (a next receiver is never the first of all: 0 ends a list)
+    std::vector<int> link(nrec, 0);
+    std::unordered_map<int, int> last;
+    for (int r = 0; r < nrec; ++r) {
+        const auto at = last.emplace(off[r], r);
+        if (at.second) continue;
+        const int q = at.first->second;                    // the one before on this node
+        link[q] = link[q] < 0 ? ~r : r;
+        link[r] = ~0;
+        at.first->second = r;
+    }
+    if (nrec > 0) {
+        const size_t first = (size_t)shot * m->d.max_receivers;
+        CUDA_OR_FAIL(m->err, cudaMemcpy(m->d_rec + first, off.data(), sizeof(int) * nrec, cudaMemcpyHostToDevice));
+        CUDA_OR_FAIL(m->err, cudaMemcpy(m->d_link + first, link.data(), sizeof(int) * nrec, cudaMemcpyHostToDevice));
+    }
     CUDA_OR_FAIL(m->err, cudaMemcpy(m->d_nrec + shot, &nrec, sizeof(int), cudaMemcpyHostToDevice));
     if (src_idx_out)
         for (int a = 0; a < nd; ++a) src_idx_out[a] = (int32_t)si[a];
@@ -3334,7 +3351,7 @@ int ewv_adjoint_inject(ewv_model_t m, void* adj_state, const void* values) {
     // lambda_u[rec] += values[shot][rec]; receivers of one shot are added in order
     if (nr == 0) return EWV_OK;
     if (!aligned(adj_state)) return fail(m->err, EWV_ERR_BAD_SIZE_OR_ALIGNMENT, "adj_state must be 256-B aligned");
-    launch_inject(m->d.precision, adj_state, (long long)m->vec_elems, values, m->d_rec, m->d_nrec, ns,
+    launch_inject(m->d.precision, adj_state, (long long)m->vec_elems, values, m->d_rec, m->d_link, m->d_nrec, ns,
                   nr, m->stream);
     ++m->launches;
     return check_launch(m->err);

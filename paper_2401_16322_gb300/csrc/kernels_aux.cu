@@ -220,23 +220,24 @@ between_kernel(const ProblemDev* probs, int nprob, int record, int vec, int kind
 // lambda_u[rec] += values[shot][rec] (the transpose of recording, R^T r); one block per shot, one
 // thread per receiver.  Of coincident receivers the first adds all their values in order, so the
 // sums are deterministic (62 us with one thread per shot adding 200 receivers one after another).
+// link[r] leads from a receiver to the next on its node (0: none), complemented where r is not the
+// first there: the list is made with the receivers, because a search among them here would grow
+// with their square (2 shots of 32768: 85 ms with the search).
 template <typename T>
 __global__ void inject_kernel(T* adj, long long vec_elems, const T* values, const int* rec_off,
-                              const int* nrec, int max_rec) {
+                              const int* rec_link, const int* nrec, int max_rec) {
     const int sh = blockIdx.x;
     T* lam = adj + (long long)sh * vec_elems;
     const int* off = rec_off + (long long)sh * max_rec;
+    const int* link = rec_link + (long long)sh * max_rec;
     const T* val = values + (long long)sh * max_rec;
     const int n = nrec[sh];
     for (int r = threadIdx.x; r < n; r += blockDim.x) {
-        const int o = off[r];
-        bool first = true;
-        for (int e = 0; e < r && first; ++e) first = off[e] != o;
-        if (!first) continue;
-        T v = lam[o] + val[r];
-        for (int e = r + 1; e < n; ++e)
-            if (off[e] == o) v += val[e];
-        lam[o] = v;
+        int e = link[r];
+        if (e < 0) continue;
+        T v = lam[off[r]] + val[r];
+        for (; e > 0; e = ~link[e]) v += val[e];
+        lam[off[r]] = v;
     }
 }
 
@@ -812,13 +813,14 @@ void launch_record_next(int precision, const ProblemDev* probs, int nprob, int v
                         double c0, double c1, cudaStream_t s) {
     launch_between(precision, probs, nprob, 1, vec, kind, m, gamma, c0, c1, s);
 }
-void launch_inject(int precision, void* adj, long long vec_elems, const void* values,
-                   const int* rec_off, const int* nrec, int nshots, int max_rec, cudaStream_t s) {
+void launch_inject(int precision, void* adj, long long vec_elems, const void* values, const int* rec_off,
+                   const int* rec_link, const int* nrec, int nshots, int max_rec, cudaStream_t s) {
     if (precision == 0)
-        inject_kernel<float><<<nshots, 256, 0, s>>>((float*)adj, vec_elems, (const float*)values, rec_off, nrec, max_rec);
+        inject_kernel<float><<<nshots, 256, 0, s>>>((float*)adj, vec_elems, (const float*)values, rec_off, rec_link,
+                                                    nrec, max_rec);
     else
-        inject_kernel<double><<<nshots, 256, 0, s>>>((double*)adj, vec_elems, (const double*)values, rec_off, nrec,
-                                                     max_rec);
+        inject_kernel<double><<<nshots, 256, 0, s>>>((double*)adj, vec_elems, (const double*)values, rec_off, rec_link,
+                                                     nrec, max_rec);
 }
 
 void launch_sum_shots(int precision, const void* in, void* out, long long n, int nshots,
