@@ -508,13 +508,15 @@ int ewv_batch_sync(ewv_batch_t batch);
  * Restore 1000000000 afterwards.  INVALID_ARG above 1e9. */
 int ewv_debug_set_wait_limit(unsigned long long ns);
 
-/* Testing aid: whether Krylov steps (and the exponential Krylov adjoint) run each Arnoldi
- * column's modified Gram-Schmidt steps on the column kernel -- one cooperative launch per
- * column with q_{j+1} in shared memory and a bounded grid barrier per step, taken when every
- * flat chunk of the engine fits one co-resident grid -- (1, the default) or on one flat
- * pass per step (0).  Both give the same values bit for bit.  FP32 problem sets too large for
- * the column kernel take two passes per column (dots and a triangular solve, then the update)
- * whatever this is set to.  Process-wide; waits for the device to be idle first. */
+/* Testing aid: the form of the Krylov steps' Gram-Schmidt (and of the exponential Krylov
+ * adjoint's).  1, the default: on the column kernel -- one cooperative launch per column with
+ * q_{j+1} in shared memory and a bounded grid barrier per step -- where every flat chunk of the
+ * engine fits one co-resident grid (up to about 30 MB a vector of all shots); larger FP32 sets
+ * take two passes per column (dots and a triangular solve, then the update); larger FP64 sets a
+ * flat pass per step.  0: a flat pass per step for all.  The column kernel and the flat passes
+ * agree to FP64 rounding in their coefficients, which leaves FP32 vectors with the same bits;
+ * the two passes sum in another order, so an FP32 step depends in its rounding on whether its
+ * set of shots is above that size.  Process-wide; waits for the device to be idle first. */
 int ewv_debug_set_column_kernel(int enable);
 
 #ifdef __cplusplus

@@ -327,8 +327,9 @@ struct ewv_batch {
 
 namespace {
 
-// Modified Gram-Schmidt steps run on the column kernel when the engine's chunks fit one
-// co-resident grid (ewv_debug_set_column_kernel(0) keeps the flat passes, for comparisons)
+// Gram-Schmidt steps run on the column kernel when the engine's chunks fit one co-resident grid,
+// larger FP32 sets on the two passes a column (ewv_debug_set_column_kernel(0) keeps the flat
+// passes in both, for comparisons)
 bool g_mgs_enabled = true;
 
 int fail(std::string& err, int code, const char* fmt, ...) {
@@ -1182,7 +1183,7 @@ int run_rk(Ctx& C, double t, double dt, int scheme, int nsteps) {
 }
 
 // Whether the engine's Arnoldi columns take the two Gram-Schmidt passes (see gram_schmidt).
-bool gs_two_pass(const Engine* E) { return E->precision == EWV_F32 && E->mgs_cpb == 0; }
+bool gs_two_pass(const Engine* E) { return g_mgs_enabled && E->precision == EWV_F32 && E->mgs_cpb == 0; }
 
 // Buffers of the two Gram-Schmidt passes (not inside a capture).
 int gs_ready(Engine* E, std::string& err) {

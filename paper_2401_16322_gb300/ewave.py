@@ -530,8 +530,8 @@ def debug_set_wait_limit(ns):
 
 
 def debug_set_column_kernel(enable):
-    """Testing aid: run the Krylov Gram-Schmidt steps on the column kernel (True, default,
-    where the engine's chunks fit one co-resident grid) or on the flat passes (False)."""
+    """Testing aid: run the Krylov Gram-Schmidt steps on the column kernel, or in two passes a
+    column for larger FP32 sets (True, default), or on the flat passes everywhere (False)."""
     rc = load_library().ewv_debug_set_column_kernel(1 if enable else 0)
     if rc != EWV_OK:
         raise EwaveError(f"debug_set_column_kernel: {ERRORS.get(rc, rc)}")
