@@ -1202,7 +1202,11 @@ int gs_ready(Engine* E, std::string& err) {
 //   FP32 sets that fit: modified Gram-Schmidt step by step in one cooperative launch.  The two
 //     passes are faster there too (5.2 -> 3.6 ms of a step on 401 x 201, 16 shots), but another
 //     order of the sums moves the gradient of the large Krylov steps used for inversion (dt |H|
-//     near m) by 1.3e-5 to 2.1e-5: it amplifies FP32 rounding about a hundredfold.
+//     near m) by 1.3e-5 to 2.1e-5: it amplifies FP32 rounding about a hundredfold.  Neither order
+//     is the nearer one.  On sets above the line (28 and 48 shots of 401 x 201, 16 of 601 x 301,
+//     Krylov 20 at 8 times the leap-frog step, three inputs each) the gradient is off the FP64
+//     library's by 0.7e-5 to 1.7e-5 with the two passes and by 0.7e-5 to 2.5e-5 with a pass per
+//     step (geometric mean of the ratios 1.03); at 4 times the step both by 2.4e-7 to 7e-7.
 //   FP64: the cooperative launch, or a pass per step: its dots are bound by the FP64 pipe, which
 //     the two passes would load with twice the dots.
 void gram_schmidt(Engine* E, const ProblemDev* probs, int j, int k0, int m, double tol, cudaStream_t s,
