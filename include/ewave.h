@@ -500,8 +500,8 @@ int ewv_sync(ewv_model_t model);
 int ewv_batch_sync(ewv_batch_t batch);
 
 /* Testing aid: the limit, in ns (at most 1e9, the default), after which a pipeline wait of
- * the 2D FP32 TMA pass, or a grid-barrier wait of the Gram-Schmidt column kernel, on the
- * current device gives up.  The TMA kernel then waits (up to 1 s) for its copies in flight;
+ * the 2D FP32 TMA pass, or a grid-barrier wait of the Gram-Schmidt column kernel or of the
+ * chained FP64 passes of small grids, on the current device gives up.  The TMA kernel then waits (up to 1 s) for its copies in flight;
  * either sets the timeout bit of the error word and returns, so that a test can check the
  * EWV_ERR_TIMEOUT path on a healthy GPU with a limit a normal pass outruns (e.g. 0).  Waits
  * for the device to be idle first; applies to later launches, graph replays included.

@@ -251,15 +251,15 @@ int launch_leapfrog_tma(int R, const ProblemDev* probs, const int* tbase, int np
 // tiles, the 30-row map set).
 int launch_grad_tma(int R, const ProblemDev* probs, const int* tbase, int nprob, int ntiles,
                     const StageArgs& a, int* err, cudaStream_t s);
-// The transposed pass H^T through the persistent TMA pipeline (FP32, no gradient); tbase and
-// ntiles are those of the map set of tma_transpose_height rows.
+// The transposed pass H^T through the persistent TMA pipeline (FP32; adds to the gradient where a
+// tape is set); tbase and ntiles are those of the map set of tma_transpose_height rows.
 int tma_transpose_height(bool reads_u, bool reads_a);
 int launch_transpose_tma(int R, const ProblemDev* probs, const int* tbase, int nprob, int ntiles,
                          const StageArgs& a, int* err, cudaStream_t s);
 int launch_stage_tma(int variant, int R, const ProblemDev* probs, const int* tbase, int nprob,
                      int ntiles, const StageArgs& a, int* err, cudaStream_t s);
 int tma_variant_tile_height(int v);
-int tma_tape_variant(int v);   // the variant that writes a gradient tape when v is selected (column pairs)
+int tma_tape_variant(int v);   // the variant that writes a gradient tape when v is selected
 // Tile height of variant v for a pass that does (reads_a) or does not read an A operand
 // (composite variants pick their tile by it).
 int tma_variant_tile_height_for(int v, bool reads_u, bool reads_a);
@@ -327,7 +327,7 @@ struct MgsArgs {
     int j, k0, kmax, m, cpb;
     double tol;
     double* partials;     // 2 x nchunks
-    unsigned int* bar;    // [2]: grid-barrier arrivals and generation
+    unsigned int* bar;    // [2]: grid-barrier arrivals and departures
     int* err;             // error word (bit 0: a barrier wait gave up)
 };
 // Chunks per block for which the grid is co-resident (smallest), or 0 if none is.

@@ -33,7 +33,7 @@ __global__ void reset_cursor_kernel(const ProblemDev* probs, int nprob) {
 
 // ---------------------------------------------------------------- source scalars
 // Ricker r(tau) = (1 - 2 a tau^2) exp(-a tau^2), a = (pi f)^2 (Sec. 4.1).  Its derivatives
-// (prologue_kernel) follow r^(k) = -g^(k+2) / (2a), g = exp(-a tau^2), with the Hermite
+// (source_scalars) follow r^(k) = -g^(k+2) / (2a), g = exp(-a tau^2), with the Hermite
 // recurrence g^(k) = -2 a tau g^(k-1) - 2 a (k-1) g^(k-2).
 __device__ __forceinline__ double ricker(double t, double f, double t0) {
     const double a = (M_PI * f) * (M_PI * f);
@@ -222,7 +222,8 @@ between_kernel(const ProblemDev* probs, int nprob, int record, int vec, int kind
 // sums are deterministic (62 us with one thread per shot adding 200 receivers one after another).
 // link[r] leads from a receiver to the next on its node (0: none), complemented where r is not the
 // first there: the list is made with the receivers, because a search among them here would grow
-// with their square (2 shots of 32768: 85 ms with the search).
+// with their square (2 shots of 32768: 85 ms with the search, 0.15 ms with the links; 2 of 4096: 1.4
+// and 0.02 ms).
 template <typename T>
 __global__ void inject_kernel(T* adj, long long vec_elems, const T* values, const int* rec_off,
                               const int* rec_link, const int* nrec, int max_rec) {

@@ -643,9 +643,14 @@ static void with_pass(int precision, int R, const StageArgs& a, F&& launch) {
     else with_type<PASS_FORWARD>(precision, R, launch);
 }
 
-// Programmatic dependent launch for grids that fill the chip several times over (1520 blocks of 601
-// x 301: 37.8 -> 35 us a Faber degree in FP64); a grid of a block per SM or less runs slower that
-// way (112 blocks of 101 x 101: 7.7 -> 8.2 us a pass), its blocks set up early end up sharing SMs.
+// Programmatic dependent launch from about four blocks per SM on, which is where chained steps end
+// too.  us a pass in FP64, dependent and plain: Faber 19.5 and 19.9 at 640 blocks (300 x 250), 22.7 and
+// 22.7 at 912, 27.7 and 28.2 at 1120, 33.4 and 33.9 at 1520 (601 x 301), 54.4 and 54.9 at 2704; Horner
+// HORK 17.1 and 17.6, 19.4 and 19.8, 23.6 and 24.1, 27.9 and 28.6, 44.5 and 45.0; H x 14.9 and 16.7,
+// 16.9 and 18.8, 21.1 and 23.2, 25.0 and 27.1, 40.6 and 43.2.  It loses at single sizes only (Faber and
+// low-storage HORK at 680 blocks, by 2 and 4 %; the leap-frog step at 912, by 6 %).  A grid of a block
+// per SM or less ran slower that way (112 blocks of 101 x 101: 7.7 -> 8.2 us a pass), its blocks set
+// up early end up sharing SMs.
 template <class... P, class... A>
 static void launch_plain(void (*kernel)(P...), int blocks, cudaStream_t s, A... args) {
     const dim3 block(DBX, DBY);

@@ -1351,6 +1351,11 @@ int tma_variant_tile_height_for(int v, bool reads_u, bool reads_a) {
 }
 
 int tma_variant_tile_height(int v) { return kVariants[v].by; }
+// The pass that writes a gradient tape reads no A operand, so it runs on 14's tall tiles where one of
+// the small shapes below 7 is selected (same bits on every shape).  FWI gradient, Horner HORK 20, 16
+// shots of 401 x 201, on 14's shape and on the selected one: 12.8 and 13.7 ms (variant 0), 14.1 and
+// 16.2 (2), 14.0 and 16.0 (3), 12.5 and 13.2 (5); on 2 shots of 301 x 151, whose tiles do not fill the
+// chip either way, 4.46 and 4.29 ms (0), 4.53 and 4.41 (2).
 int tma_tape_variant(int v) { return v >= 7 ? v : 14; }
 void tma_variant_describe(int v, int* by, int* nw, int* nst) {
     *by = kVariants[v].by;
@@ -1458,10 +1463,10 @@ static int launch_t(const ProblemDev* probs, const int* tbase, int nprob, int nt
                       ntiles, map_set_of(BYv), a, err);
 }
 
-// The transposed pass H^T (FP32, no gradient) on the column-pair consumers, two rows a thread.  The
-// tile is as tall as three stages fit shared memory, since the consumer warps hide the latency:
-// 64 x 18 with 9 warps for a pass with a U and an A operand, 64 x 24 with 12 for one of them, 64 x
-// 30 with 15 for the plain product; tbase and ntiles are those of that height's map set.
+// The transposed pass H^T (FP32; with a tape set, the gradient too) on the column-pair consumers, two
+// rows a thread.  The tile is as tall as three stages fit shared memory, since the consumer warps hide
+// the latency: 64 x 18 with 9 warps for a pass with a U and an A operand, 64 x 24 with 12 for one of
+// them, 64 x 30 with 15 for the plain product; tbase and ntiles are those of that height's map set.
 int tma_transpose_height(bool reads_u, bool reads_a) { return reads_u && reads_a ? 18 : reads_u || reads_a ? 24 : 30; }
 int launch_transpose_tma(int R, const ProblemDev* probs, const int* tbase, int nprob, int ntiles,
                          const StageArgs& a_in, int* err, cudaStream_t s) {

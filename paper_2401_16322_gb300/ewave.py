@@ -523,7 +523,7 @@ def checkpoint_stride(nsteps, budget):
 
 def debug_set_wait_limit(ns):
     """Testing aid: wait limit (ns, default 1e9) of the 2D FP32 TMA pass's pipeline waits and
-    of the Gram-Schmidt column kernel's grid barriers."""
+    of the grid barriers (the Gram-Schmidt column kernel's and the chained FP64 passes')."""
     rc = load_library().ewv_debug_set_wait_limit(int(ns))
     if rc != EWV_OK:
         raise EwaveError(f"debug_set_wait_limit: {ERRORS.get(rc, rc)}")
