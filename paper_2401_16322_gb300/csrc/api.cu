@@ -173,8 +173,7 @@ struct ewv_model {
     int kry_adjoint = EWV_KRYLOV_ADJOINT_EXACT;   // which Krylov adjoint ewv_adjoint_step runs
     bool lf_history_valid = false;
     // device metadata
-    int* d_rec = nullptr;
-    int* d_link = nullptr;      // from a receiver to the next on its node (inject_kernel)
+    int* d_rec = nullptr;       // 2 max_receivers entries a shot: the receivers' offsets, then their links
     int* d_nrec = nullptr;      // receivers per shot
     double* d_sigma = nullptr;
     float* d_btab = nullptr;    // damping profile at half-cell distances (FP32 models)
@@ -454,7 +453,7 @@ ProblemDev make_problem(ewv_model* m, int shot, int tile_base) {
     P.work = m->work;
     P.c2 = m->params;
     P.sigma = m->d_sigma + (size_t)shot * MAX_SIGMA;
-    P.rec_off = m->d_rec + (size_t)shot * (d.max_receivers > 0 ? d.max_receivers : 1);
+    P.rec_off = m->d_rec + (size_t)shot * 2 * (d.max_receivers > 0 ? d.max_receivers : 1);
     P.seismo = m->seismo ? (char*)m->seismo + (size_t)shot * m->capacity * d.max_receivers * m->elem
                          : nullptr;
     P.kry = m->d_kry + (size_t)shot * KRY_STRIDE;
@@ -1910,8 +1909,7 @@ int ewv_create_model(const ewv_model_desc* desc, ewv_model_t* out) {
     m->shots.resize(d.nshots);
     const int nr = d.max_receivers > 0 ? d.max_receivers : 1;
     cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_rec, sizeof(int) * (size_t)nr * d.nshots);
-    if (e == cudaSuccess) e = cudaMalloc(&m->d_link, sizeof(int) * (size_t)nr * d.nshots);
+    if (e == cudaSuccess) e = cudaMalloc(&m->d_rec, sizeof(int) * 2 * (size_t)nr * d.nshots);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_nrec, sizeof(int) * (size_t)d.nshots);
     if (e == cudaSuccess) e = cudaMemset(m->d_nrec, 0, sizeof(int) * (size_t)d.nshots);
     if (e == cudaSuccess) e = cudaMalloc(&m->d_sigma, sizeof(double) * (size_t)MAX_SIGMA * d.nshots);
@@ -1950,7 +1948,6 @@ int ewv_destroy_model(ewv_model_t m) {
     if (!m) return EWV_ERR_INVALID_ARG;
     delete m->engine;
     cudaFree(m->d_rec);
-    cudaFree(m->d_link);
     cudaFree(m->d_nrec);
     cudaFree(m->d_sigma);
     cudaFree(m->d_btab);
@@ -2123,7 +2120,9 @@ static int set_src_rec(ewv_model_t m, int shot, const double* spos, double f_pea
     s.amp = amp;
     s.rec_off = off;
     // receivers of one node, in order (a next receiver is never the first of all: 0 ends a list)
-    std::vector<int> link(nrec, 0);
+    std::vector<int> rows(off);                            // the offsets, then the links
+    rows.resize(2 * (size_t)nrec, 0);
+    int* link = rows.data() + nrec;
     std::unordered_map<int, int> last;
     for (int r = 0; r < nrec; ++r) {
         const auto at = last.emplace(off[r], r);
@@ -2133,11 +2132,9 @@ static int set_src_rec(ewv_model_t m, int shot, const double* spos, double f_pea
         link[r] = ~0;
         at.first->second = r;
     }
-    if (nrec > 0) {
-        const size_t first = (size_t)shot * m->d.max_receivers;
-        CUDA_OR_FAIL(m->err, cudaMemcpy(m->d_rec + first, off.data(), sizeof(int) * nrec, cudaMemcpyHostToDevice));
-        CUDA_OR_FAIL(m->err, cudaMemcpy(m->d_link + first, link.data(), sizeof(int) * nrec, cudaMemcpyHostToDevice));
-    }
+    if (nrec > 0)
+        CUDA_OR_FAIL(m->err, cudaMemcpy(m->d_rec + (size_t)shot * 2 * m->d.max_receivers, rows.data(),
+                                        sizeof(int) * rows.size(), cudaMemcpyHostToDevice));
     CUDA_OR_FAIL(m->err, cudaMemcpy(m->d_nrec + shot, &nrec, sizeof(int), cudaMemcpyHostToDevice));
     if (src_idx_out)
         for (int a = 0; a < nd; ++a) src_idx_out[a] = (int32_t)si[a];
@@ -3358,7 +3355,7 @@ int ewv_adjoint_inject(ewv_model_t m, void* adj_state, const void* values) {
     // lambda_u[rec] += values[shot][rec]; receivers of one shot are added in order
     if (nr == 0) return EWV_OK;
     if (!aligned(adj_state)) return fail(m->err, EWV_ERR_BAD_SIZE_OR_ALIGNMENT, "adj_state must be 256-B aligned");
-    launch_inject(m->d.precision, adj_state, (long long)m->vec_elems, values, m->d_rec, m->d_link, m->d_nrec, ns,
+    launch_inject(m->d.precision, adj_state, (long long)m->vec_elems, values, m->d_rec, m->d_nrec, ns,
                   nr, m->stream);
     ++m->launches;
     return check_launch(m->err);

@@ -292,8 +292,9 @@ void launch_nonfinite_scan(int precision, int nchunks, const ProblemDev* probs, 
                            int nprob, int* err, cudaStream_t s);
 // Pipeline-wait limit of the 2D TMA pass in ns (default 1 s) on the current device.
 int set_tma_wait_limit_ns(unsigned long long ns);
-void launch_inject(int precision, void* adj, long long vec_elems, const void* values, const int* rec_off,
-                   const int* rec_link, const int* nrec, int nshots, int max_rec, cudaStream_t s);
+// rec: per shot (2 max_rec entries) the nrec receivers' offsets, then their links (inject_kernel).
+void launch_inject(int precision, void* adj, long long vec_elems, const void* values, const int* rec, const int* nrec,
+                   int nshots, int max_rec, cudaStream_t s);
 void launch_sum_shots(int precision, const void* in, void* out, long long n, int nshots,
                       cudaStream_t s);
 int launch_expm(const ProblemDev* probs, int nprob, int mmax, cudaStream_t s, double hscale = 1.0);

@@ -225,14 +225,14 @@ between_kernel(const ProblemDev* probs, int nprob, int record, int vec, int kind
 // with their square (2 shots of 32768: 85 ms with the search, 0.15 ms with the links; 2 of 4096: 1.4
 // and 0.02 ms).
 template <typename T>
-__global__ void inject_kernel(T* adj, long long vec_elems, const T* values, const int* rec_off,
-                              const int* rec_link, const int* nrec, int max_rec) {
+__global__ void inject_kernel(T* adj, long long vec_elems, const T* values, const int* rec, const int* nrec,
+                              int max_rec) {
     const int sh = blockIdx.x;
     T* lam = adj + (long long)sh * vec_elems;
-    const int* off = rec_off + (long long)sh * max_rec;
-    const int* link = rec_link + (long long)sh * max_rec;
     const T* val = values + (long long)sh * max_rec;
     const int n = nrec[sh];
+    const int* off = rec + (long long)sh * 2 * max_rec;
+    const int* link = off + n;
     for (int r = threadIdx.x; r < n; r += blockDim.x) {
         int e = link[r];
         if (e < 0) continue;
@@ -814,14 +814,12 @@ void launch_record_next(int precision, const ProblemDev* probs, int nprob, int v
                         double c0, double c1, cudaStream_t s) {
     launch_between(precision, probs, nprob, 1, vec, kind, m, gamma, c0, c1, s);
 }
-void launch_inject(int precision, void* adj, long long vec_elems, const void* values, const int* rec_off,
-                   const int* rec_link, const int* nrec, int nshots, int max_rec, cudaStream_t s) {
+void launch_inject(int precision, void* adj, long long vec_elems, const void* values, const int* rec, const int* nrec,
+                   int nshots, int max_rec, cudaStream_t s) {
     if (precision == 0)
-        inject_kernel<float><<<nshots, 256, 0, s>>>((float*)adj, vec_elems, (const float*)values, rec_off, rec_link,
-                                                    nrec, max_rec);
+        inject_kernel<float><<<nshots, 256, 0, s>>>((float*)adj, vec_elems, (const float*)values, rec, nrec, max_rec);
     else
-        inject_kernel<double><<<nshots, 256, 0, s>>>((double*)adj, vec_elems, (const double*)values, rec_off, rec_link,
-                                                     nrec, max_rec);
+        inject_kernel<double><<<nshots, 256, 0, s>>>((double*)adj, vec_elems, (const double*)values, rec, nrec, max_rec);
 }
 
 void launch_sum_shots(int precision, const void* in, void* out, long long n, int nshots,
