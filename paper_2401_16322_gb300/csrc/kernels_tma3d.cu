@@ -177,18 +177,26 @@ __device__ __forceinline__ float bt3(const float* t, int n, int k) {
     return (unsigned)k < (unsigned)n ? __ldg(t + k) : 0.f;
 }
 
+// A tap of the input vector from global memory.  Not __ldg: this kernel is resident while the pass
+// before it still writes X, and the read-only path gives no ordering against that.  Not a plain load
+// either, which the compiler keeps behind the stores of the plane before (1 % of a leap-frog step);
+// it may pass those, as no pass writes the vector it reads, but no wait.
+__device__ __forceinline__ float ld_x(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+
 // Half-point derivative of psi along one axis (unscaled), plain loads: p points at psi of the
 // output node, `stride` is the axis stride, idx the node index and n the extent (zero
 // extension); up = true for the vertical axis (sum_q s_q (psi_{k-q} - psi_{k+1+q})).
-// (Not __ldg, here and in the free-surface columns: this kernel is resident while the pass before
-// it still writes X, and the read-only path gives no ordering against that.)
 template <int R>
 __device__ __forceinline__ float dpsi3(const float* p, long long stride, int idx, int n, bool up) {
     float d[R];
 #pragma unroll
     for (int q = 0; q < R; ++q) {
-        const float fwd = (idx + 1 + q < n) ? p[(long long)(1 + q) * stride] : 0.f;
-        const float bwd = (idx - q >= 0) ? p[-(long long)q * stride] : 0.f;
+        const float fwd = (idx + 1 + q < n) ? ld_x(p + (long long)(1 + q) * stride) : 0.f;
+        const float bwd = (idx - q >= 0) ? ld_x(p - (long long)q * stride) : 0.f;
         d[q] = up ? bwd - fwd : fwd - bwd;
     }
     return st_tree<R>(d);
@@ -434,11 +442,11 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                             uzz = 0.f;
 #pragma unroll
                             for (int q = 0; q < 9; ++q)
-                                uzz += g3t_fs[T3_UZZ + c * 9 + q] * (q < nz ? ucol[q * ps] : 0.f);
+                                uzz += g3t_fs[T3_UZZ + c * 9 + q] * (q < nz ? ld_x(ucol + q * ps) : 0.f);
                             dwz = 0.f;
 #pragma unroll
                             for (int q = 0; q < 8; ++q)
-                                dwz += g3t_fs[T3_DWZ + c * 8 + q] * (q < nz - 1 ? wcol[q * ps] : 0.f);
+                                dwz += g3t_fs[T3_DWZ + c * 8 + q] * (q < nz - 1 ? ld_x(wcol + q * ps) : 0.f);
                         } else {
                             float pz[R], dwzv[R];
 #pragma unroll
@@ -481,7 +489,7 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                                 duz = 0.f;
 #pragma unroll
                                 for (int q = 0; q < 8; ++q)
-                                    duz += g3t_fs[T3_UZ + c * 8 + q] * (q < nz ? ucol[q * ps] : 0.f);
+                                    duz += g3t_fs[T3_UZ + c * 8 + q] * (q < nz ? ld_x(ucol + q * ps) : 0.f);
                             } else {
                                 float dz[R];
 #pragma unroll
@@ -499,7 +507,7 @@ stage_tma3d_kernel(const ProblemDev* __restrict__ probs, const int* __restrict__
                                     const float* col = ti.X + 5 * fstr + oc;
 #pragma unroll
                                     for (int q = 0; q < 8; ++q)
-                                        d += g3t_fs[T3_UZ + c * 8 + q] * (q < nz ? col[q * ps] : 0.f);
+                                        d += g3t_fs[T3_UZ + c * 8 + q] * (q < nz ? ld_x(col + q * ps) : 0.f);
                                 } else {
                                     d = dpsi3<R>(pc, ps, c, nz, true);
                                 }
