@@ -27,6 +27,7 @@
 
 #include <vector>
 
+#include "chunk3d.hpp"
 #include "ewave_internal.cuh"
 #include "pdl.cuh"
 
@@ -666,36 +667,16 @@ int tma3d_tasks_of(const ProblemDev& P) {
     return ((P.nx + BX - 1) / BX) * ((P.ny + BY3 - 1) / BY3) * ((P.nz + P.kc3 - 1) / P.kc3);
 }
 
-// Planes per task, the same for every problem of an engine.  A task of kc planes costs about as
-// much as kc + R full stages (its 2 R warm-up stages carry two planes instead of twenty), and the
-// pass as many rounds of tasks as the busiest SM gets: take the chunk that makes rounds x stages
-// smallest.  251 x 229 x 197: 5 chunks of 40 planes (4 rounds of 44) instead of chunks of 32 (6
-// rounds of 36); with the undamped points' shorter form and the dependent launch, Faber degree 40
-// takes 12.7 ms instead of 13.0, and 100 x 95 x 260, whose 32-plane chunks left a second round
-// nearly empty, 4.1 instead of 6.1.  Chunks shorter than 16 planes are not worth their warm-up.
-void tma3d_choose_chunk(std::vector<ProblemDev>& probs, int R) {
-    int dev = 0, nsm = 0, nz = 1;
+// Planes per task, the same for every problem of an engine (chunk3d.hpp).
+void tma3d_choose_chunk(std::vector<ProblemDev>& probs) {
+    int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
         nsm = 1;
-    for (const ProblemDev& P : probs) nz = P.nz > nz ? P.nz : nz;
-    const int warm = R;
-    long long best = -1;
-    int best_kc = nz;
-    for (int n = 1; n == 1 || nz / n >= 16; ++n) {
-        const int kc = (nz + n - 1) / n;
-        long long tasks = 0;
-        for (ProblemDev& P : probs) {
-            P.kc3 = kc;
-            tasks += tma3d_tasks_of(P);
-        }
-        const long long cost = (tasks + nsm - 1) / nsm * (kc + warm);
-        if (best < 0 || cost < best) {
-            best = cost;
-            best_kc = kc;
-        }
-    }
-    for (ProblemDev& P : probs) P.kc3 = best_kc;
+    std::vector<Grid3> grids;
+    for (const ProblemDev& P : probs) grids.push_back(Grid3{P.nx, P.ny, P.nz, P.pml, P.fs != 0});
+    const int kc = planes_per_task(grids, nsm, BX, BY3);
+    for (ProblemDev& P : probs) P.kc3 = kc;
 }
 
 // NMAP3 maps per problem: state and workspace, each with the u halo box, the w_x box, the w_y
