@@ -553,7 +553,7 @@ int build_engine(Engine* E, std::string& err) {
         CUDA_OR_FAIL(err, cudaMemcpy(E->d_tbase, pre.data(), sizeof(int) * pre.size(), cudaMemcpyHostToDevice));
     }
     if (E->precision == EWV_F32 && E->dims == 3) {
-        tma3d_choose_chunk(E->probs);
+        tma3d_choose_chunk(E->probs, E->R);
         if (build_tensor_maps3d(E->probs, E->R, work_vecs, &E->d_maps) != 0)
             return fail(err, EWV_ERR_CUDA, "TMA tensor-map encoding failed (3D)");
         std::vector<int> pre((size_t)E->nprob + 1, 0);

@@ -229,7 +229,7 @@ void launch_leapfrog3d(int precision, int R, int nblocks, const ProblemDev* prob
 // kernels_tma3d.cu: persistent TMA-fed FP32 forward pass of three-dimensional problems.
 int upload_tma3d_tables(const double* fs_uzz, const double* fs_uz, const double* fs_dwz);
 int tma3d_tasks_of(const ProblemDev& P);
-void tma3d_choose_chunk(std::vector<ProblemDev>& probs);   // sets kc3
+void tma3d_choose_chunk(std::vector<ProblemDev>& probs, int R);   // sets kc3
 int build_tensor_maps3d(std::vector<ProblemDev>& probs, int R, const std::vector<int>& work_vecs,
                         void** d_maps_inout);
 int launch_stage_tma3d(int R, int warps, const ProblemDev* probs, const int* tbase, int nprob,

@@ -668,14 +668,14 @@ int tma3d_tasks_of(const ProblemDev& P) {
 }
 
 // Planes per task, the same for every problem of an engine (chunk3d.hpp).
-void tma3d_choose_chunk(std::vector<ProblemDev>& probs) {
+void tma3d_choose_chunk(std::vector<ProblemDev>& probs, int R) {
     int dev = 0, nsm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || nsm <= 0)
         nsm = 1;
     std::vector<Grid3> grids;
     for (const ProblemDev& P : probs) grids.push_back(Grid3{P.nx, P.ny, P.nz, P.pml, P.fs != 0});
-    const int kc = planes_per_task(grids, nsm, BX, BY3);
+    const int kc = planes_per_task(grids, nsm, BX, BY3, R);
     for (ProblemDev& P : probs) P.kc3 = kc;
 }
 
